@@ -34,9 +34,12 @@ extern "C" {
 #endif
 
 /* Options for pjds_cg_solve. max_outer = 0 / inner_iters = 0 take defaults
- * (6 and 50: 300 inner steps). use_graph = 1 captures the inner iterations in
- * a CUDA graph once and replays it every outer step (the stream must not be
- * capturing already). */
+ * (6 and 50: 300 inner steps). use_graph = 1 captures the inner iterations of
+ * a large system in a CUDA graph once and replays it every outer step (the
+ * stream must not be capturing already). A small system (one whose inner matrix
+ * fits in the SMs' shared memory, about 125,000 rows of 24 fp32 entries, or
+ * one of at most 512 rows per SM) is solved by one cooperative launch, with
+ * use_graph and without. */
 typedef struct pjds_cg_opts {
   int32_t max_outer;
   int32_t inner_iters;
@@ -70,8 +73,10 @@ int pjds_cg_workspace_bytes(int32_t n_rows, int32_t n_pad, int32_t vec_dtype, si
  * A_hi: PJDS_F64, permute_cols = 1. A_lo: NULL, or the same matrix in any
  * dtype, permute_cols = 1. b, x: device fp64 vectors of n_rows (x holds the
  * initial guess on entry). res may be NULL. Synchronises the stream once per
- * outer step (to read the residual norm).
- * Errors: PJDS_EINVAL (shapes, dtypes, bases, workspace too small), PJDS_ECUDA.
+ * outer step (to read the residual norm), for a small system once at the end.
+ * Errors: PJDS_EINVAL (shapes, dtypes, bases, workspace too small), PJDS_ECUDA
+ * (also when a small system's CTAs, whose waits for one another are bounded,
+ * waited in vain).
  */
 int pjds_cg_solve(const pjds_dev *A_hi, const pjds_dev *A_lo, const double *b, double *x, const pjds_cg_opts *opts,
                   pjds_cg_result *res, void *work, size_t work_bytes, void *stream);
@@ -92,11 +97,12 @@ int pjds_cg_solve(const pjds_dev *A_hi, const pjds_dev *A_lo, const double *b, d
  *     array's device address once and keeps it for the life of the process;
  *     make that first call before any stream capture, and do not use the
  *     library across cudaDeviceReset (the kept address would then be stale);
- *   - opts->use_graph is ignored: the inner steps are launched one by one on
- *     `stream`, so the call creates no stream, graph or other driver object;
+ *   - opts->use_graph is ignored: the inner steps run in one launch or are
+ *     launched one by one on `stream`, so the call creates no stream, graph or
+ *     other driver object;
  *   - no cudaMalloc, cudaFree or allocating library call is made (the call
- *     issues kernels, one cudaMemsetAsync on the array and a small
- *     device-to-host copy of the residual norm per outer step);
+ *     issues kernels, cudaMemsetAsync on the array and small device-to-host
+ *     copies of the residual norms);
  *   - all calls share the one array per device and it keeps the previous
  *     call's contents: each call clears the scalar block it reads and writes
  *     every vector before reading it, but calls that overlap on the GPU

@@ -19,6 +19,7 @@
 #include <mutex>
 #include <vector>
 
+#include "cg.h"
 #include "common.h"
 #include "pjds_krylov.h"
 #include "spmv_kernels.cuh"
@@ -609,7 +610,7 @@ static void launch_dot(const Dot<TX, MODE> &d, const pjds_dev *A, const typename
 
 static size_t cg_bytes(int32_t n, int vec_bytes) {
   return align256((size_t)n_blocks_of(n) * 8) + align256(S_COUNT * 8) + 4 * align256((size_t)n * vec_bytes) +
-         align256((size_t)n * 8);
+         align256((size_t)n * 8) + align256(sizeof(CgOut)) + align256(cg_slots_bytes());
 }
 
 template <typename TL>
@@ -622,6 +623,17 @@ static int cg_run(const pjds_dev *Ah, const pjds_dev *Al, const double *b, doubl
   TL *r = cv.take<TL>((size_t)n), *p = cv.take<TL>((size_t)n), *q = cv.take<TL>((size_t)n);
   TL *d = cv.take<TL>((size_t)n);
   double *r64 = cv.take<double>((size_t)n);
+  CgOut *small_out = cv.take<CgOut>(1);
+  char *slots = cv.take<char>(cg_slots_bytes());
+  pjds_cg_result small_res;
+  bool small = false;
+  const int rc_small = cg_small(
+      Ah, Al, CgSystem{b, x, r64, r, p, q, slots, small_out, &small_res, o.max_outer, o.inner_iters, o.tol}, &small, s);
+  if (rc_small) return rc_small;
+  if (small) {
+    if (res) *res = small_res;
+    return PJDS_OK;
+  }
   auto fin = [&](int32_t op, int32_t j) { return Fin{partial, scal, nullptr, op, j}; };
   int rc;
   Dot<TL, 0> dot_lo;

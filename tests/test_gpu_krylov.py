@@ -183,3 +183,53 @@ def test_lanczos_basis_rows_of_odd_length(mods, oracle_lib, dtype):
     if dtype == "f64":
         ra, rb, _ = ok.lanczos(A, v0, k)
         assert np.allclose(a1[:10], ra[:10], rtol=1e-10, atol=0)
+
+
+def _spd(name, n):
+    """Symmetric, strictly diagonally dominant: `tri` three diagonals and empty
+    couplings every 13 rows (rows of 1 to 3 entries), `arrow` a dense first row
+    and column beside the diagonal (one row of n entries)."""
+    i = np.arange(n)
+    if name == "tri":
+        off = np.where(np.arange(n - 1) % 13 == 5, 0.0, -1.0 / (1 + np.arange(n - 1) % 7))
+        keep = np.nonzero(off)[0]
+        r, c = np.concatenate([keep, keep + 1]), np.concatenate([keep + 1, keep])
+        v = np.concatenate([off[keep], off[keep]])
+        d = np.full(n, 3.0)
+    else:
+        r, c = np.concatenate([np.zeros(n - 1, int), i[1:]]), np.concatenate([i[1:], np.zeros(n - 1, int)])
+        v = np.full(2 * (n - 1), 1.0 / n)
+        d = np.full(n, 2.0)
+    r, c, v = np.concatenate([r, i]), np.concatenate([c, i]), np.concatenate([v, d])
+    o = np.lexsort((c, r))
+    ptr = np.concatenate([[0], np.cumsum(np.bincount(r, minlength=n))]).astype(np.int64)
+    return synth.Crs(n, n, ptr, c[o].astype(np.int32), v[o])
+
+
+# one launch for the solve: sizes at the edges of a warp's rows (32, 16, 8 for 1,
+# 2, 4 threads per row) and of the rule that takes it (512 rows per SM without
+# the matrix in shared memory: the arrow's long row); beyond it a launch a step
+@pytest.mark.parametrize("lo,max_outer", [(None, 3), ("f32", 6), ("bf16", 12)])
+@pytest.mark.parametrize("name,n", [("tri", 1), ("tri", 7), ("tri", 8), ("tri", 33), ("tri", 4097), ("tri", 40001),
+                                    ("tri", 77857), ("arrow", 2), ("arrow", 3001), ("arrow", 77001),
+                                    ("arrow", 78001)])
+def test_cg_small_and_large_systems(mods, oracle_lib, name, n, lo, max_outer):
+    torch, pjds, krylov = mods
+    A = _spd(name, n)
+    b = synth.vector(n, seed=n)
+    D64, perm = _dev(pjds, A, "f64")
+    Dlo = _dev(pjds, A, lo)[0] if lo else None
+    bp = torch.from_numpy(b[perm]).cuda()
+    x1, x2 = torch.zeros_like(bp), torch.zeros_like(bp)
+    res = krylov.cg_solve(D64, Dlo, bp, x1, max_outer=max_outer, inner_iters=20, tol=1e-13)
+    krylov.cg_solve(D64, Dlo, bp, x2, max_outer=max_outer, inner_iters=20, tol=1e-13)
+    assert torch.equal(x1, x2)
+    x = np.empty(n)
+    x[perm] = x1.cpu().numpy()
+    # kappa below 5: 20 steps reduce the error by ((sqrt 5 - 1) / (sqrt 5 + 1))^20 < 1e-8 or to the inner
+    # type's rounding, and the outer steps repeat it until the residual is at 1e-13 (rounding of b - A x
+    # in fp64: a few 1e-16 times (|A||x| + |b|) / |b| < 10)
+    rel = _true_rel_residual(oracle_lib, A, x, b)
+    assert rel <= 1e-12, (rel, res)
+    assert res["rel_residual"] <= 1e-12 and res["inner_total"] == 20 * res["outer"]
+    assert len(res["history"]) == res["outer"] + 1 and res["history"][-1] == res["rel_residual"]
