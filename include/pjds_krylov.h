@@ -34,12 +34,10 @@ extern "C" {
 #endif
 
 /* Options for pjds_cg_solve. max_outer = 0 / inner_iters = 0 take defaults
- * (6 and 50: 300 inner steps). use_graph = 1 captures the inner iterations of
- * a large system in a CUDA graph once and replays it every outer step (the
- * stream must not be capturing already). A small system (one whose inner matrix
- * fits in the SMs' shared memory, about 125,000 rows of 24 fp32 entries, or
- * one of at most 512 rows per SM) is solved by one cooperative launch, with
- * use_graph and without. */
+ * (6 and 50: 300 inner steps). use_graph is accepted and changes nothing: a small
+ * system (one whose inner matrix fits in the SMs' shared memory, about 125,000
+ * rows of 24 fp32 entries, or one of at most 512 rows per SM) is solved by one
+ * cooperative launch, a larger one by launches of its own for every step. */
 typedef struct pjds_cg_opts {
   int32_t max_outer;
   int32_t inner_iters;
@@ -123,7 +121,8 @@ int pjds_lanczos_workspace_bytes(int32_t n_rows, int32_t n_pad, int32_t vec_dtyp
  * in fp64. alpha_host[steps] and beta_host[steps+1] (beta_host[0] = 0) receive
  * the tridiagonal T. basis: NULL, or device memory of steps * n_rows elements
  * of A's vector type that receives v_0 .. v_{steps-1} (row-major). A
- * breakdown (beta = 0) leaves the following vectors zero. Synchronises once.
+ * breakdown (beta = 0) leaves the following vectors zero. use_graph is accepted
+ * and changes nothing. Synchronises once.
  */
 int pjds_lanczos(const pjds_dev *A, const void *v0, int32_t steps, double *alpha_host, double *beta_host,
                  void *basis, int32_t use_graph, void *work, size_t work_bytes, void *stream);

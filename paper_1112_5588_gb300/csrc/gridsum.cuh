@@ -103,6 +103,7 @@ __device__ __forceinline__ Fixed warp_sum(const Fixed (&a)[N]) {
   }
   // up to 6 bits of carry for 5 x 32 values of 57 bits and a sign: 3 bits fewer first
   constexpr int drop = N > 1 ? 3 : 0;
+  static_assert(N <= 8, "carries beyond 63 bits");
   long long f = 0;
 #pragma unroll
   for (int q = 0; q < N; ++q) f += a[q].f >> min(em - a[q].e + drop, 63u);

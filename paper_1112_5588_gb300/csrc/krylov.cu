@@ -1,16 +1,17 @@
 // Krylov drivers on pJDS matrices in the permuted basis (include/pjds_krylov.h):
 // mixed-precision CG with fp64 residual refinement, Lanczos, fp64 Ritz refine.
 //
-// Every step runs in the kernels below; the host only sequences launches,
-// reads one residual norm per outer CG step and solves the small tridiagonal
-// eigenproblem. Scalars (alpha, beta, norms) live in device memory and are
-// read by the kernels that need them, so a run of inner iterations has no
-// host round trip and can be captured once in a CUDA graph. Inner products
-// accumulate in fp64 with a fixed reduction order: per-CTA partial sums
-// (warp shuffles, then one warp) into the workspace; the CTA that finishes
-// last (a counter in the workspace) adds the partials in index order and
-// applies the scalar update, inside the same launch. The summation pattern
-// does not depend on which CTA is last — results are bitwise reproducible.
+// Small systems of pjds_cg_solve run in one launch (cg.cu). Everything else runs
+// in the kernels below; the host only sequences launches, reads one residual norm
+// per outer CG step and solves the small tridiagonal eigenproblem. Scalars (alpha,
+// beta, norms) live in device memory and are read by the kernels that need them,
+// so a run of inner iterations has no host round trip. Its launches follow one
+// another by programmatic dependent launch; no graph is recorded (a step takes
+// longer than its five launches, and a graph of 24 Lanczos steps took 0.3 ms to
+// record). Inner products accumulate in fp64 or, for vectors of floats, in twice
+// their precision: per-CTA partial sums into the workspace, which a launch of one
+// CTA adds in fixed point before it applies the scalar update. The sums depend on
+// the number of CTAs alone, so results are bitwise reproducible.
 #include <float.h>
 #include <math.h>
 #include <string.h>
@@ -21,6 +22,7 @@
 
 #include "cg.h"
 #include "common.h"
+#include "gridsum.cuh"
 #include "pjds_krylov.h"
 #include "spmv_kernels.cuh"
 
@@ -30,41 +32,75 @@ namespace kry {
 constexpr int KT = 256;  // threads per CTA of the vector and product kernels
 
 // slots of the device scalar block
-// (slot S_CTR holds the 32-bit arrival counter of the reduction in flight; it
-// is 0 between launches)
-enum { S_RR = 0, S_PQ, S_ALPHA, S_BETA, S_NRM, S_INVNRM, S_AUX0, S_AUX1, S_AUX2, S_CTR = 15, S_COUNT = 16 };
+// (S_LALPHA, S_LBETA + (j & 1): the Lanczos coefficients of step j; beside
+// them and 1 / beta their upper and lower halves as floats, SF_*)
+enum { S_RR = 0, S_ALPHA, S_BETA, S_NRM, S_INVNRM, S_AUX0, S_AUX1, S_AUX2, S_LALPHA, S_LBETA, SF_ALPHA = 11, SF_BETA,
+       SF_INV = 14, S_COUNT = 16 };
 // finalisation operations
 enum { F_ALPHA = 0, F_BETA, F_RR, F_NORM, F_LALPHA, F_LBETA, F_STORE };
 
-__device__ __forceinline__ double block_sum(double v) {
-  __shared__ double sh[KT / 32];
-  for (int o = 16; o > 0; o >>= 1) v += __shfl_down_sync(0xffffffffu, v, o);
-  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  if (l == 0) sh[w] = v;
-  __syncthreads();
-  double s = 0.0;
-  if (w == 0) {
-    s = l < KT / 32 ? sh[l] : 0.0;
-    for (int o = 16; o > 0; o >>= 1) s += __shfl_down_sync(0xffffffffu, s, o);
-  }
-  return s;  // complete in thread 0
-}
+// Whether fp32 holds a product p and its rounding error, and sums of some of them.
+__device__ __forceinline__ bool in_range(float p) { return fabsf(p) >= 0x1p-96f && fabsf(p) <= 0x1p100f; }
 
-// Where a reduction's result goes: the partial-sum array (one slot per CTA),
-// the scalar block (its S_CTR slot is the arrival counter) and the update.
+__device__ __noinline__ double far_product(float a, float b, double c) { return __fma_rn((double)a, (double)b, c); }
+
+// Running inner product of one thread. Vectors of floats: products and sums in
+// twice the working precision (Ogita, Rump, Oishi, "Accurate sum and dot
+// product", 2005, Dot2: error-free products and sums in fp32, their errors added
+// up beside), since an fp64 multiply-add and its conversions take 16 cycles of
+// the SM's fp64 pipe a warp: with them the two inner products of a CG step on
+// 2M rows alone take 20 us.
+template <typename TX>
+struct Dot;
+template <>
+struct Dot<double> {
+  double s = 0.0;
+  __device__ __forceinline__ void add(double a, double b) { s = __fma_rn(a, b, s); }
+  __device__ __forceinline__ double value() const { return s; }
+};
+template <>
+struct Dot<float> {
+  float s = 0.0f, c = 0.0f;
+  double far = 0.0;  // products too small or too large for an error-free fp32 product
+  __device__ __forceinline__ void add(float a, float b) {
+    const float p = __fmul_rn(a, b);
+    if (in_range(p)) {
+      const float e = __fmaf_rn(a, b, -p), t = __fadd_rn(s, p), z = __fsub_rn(t, s);
+      c = __fadd_rn(c, __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z))));
+      s = t;
+    } else if (a != 0.0f && b != 0.0f) {
+      far = far_product(a, b, far);
+    }
+  }
+  __device__ __forceinline__ double value() const { return ((double)s + (double)c) + far; }
+};
+
+// Where a reduction's result goes: the scalar block and the update.
 struct Fin {
-  double *partial;
   double *scal;
   double *out;
   int32_t op, j;
 };
+
+// Programmatic dependent launch: every kernel lets the next one on the stream
+// start (so that its launch is over when this one ends) and waits for the one
+// before it, completed and visible, before it touches memory.
+__device__ __forceinline__ void begin() {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+// v as the sum of two floats (in the place of a double).
+__device__ __forceinline__ void halves(double *out, double v) {
+  const float h = (float)v;
+  *reinterpret_cast<float2 *>(out) = make_float2(h, (float)(v - (double)h));
+}
 
 // The scalar update `op` with the complete sum v.
 __device__ __forceinline__ void apply_op(double v, const Fin &f) {
   double *scal = f.scal;
   switch (f.op) {
     case F_ALPHA:  // alpha = (r, r) / (p, A p)
-      scal[S_PQ] = v;
       scal[S_ALPHA] = v != 0.0 ? scal[S_RR] / v : 0.0;
       break;
     case F_BETA:  // beta = (r', r') / (r, r)
@@ -82,11 +118,16 @@ __device__ __forceinline__ void apply_op(double v, const Fin &f) {
     }
     case F_LALPHA:
       f.out[f.j] = v;
+      scal[S_LALPHA] = v;
+      halves(scal + SF_ALPHA, v);
       break;
     case F_LBETA: {
-      const double nrm = sqrt(v);
+      const double nrm = sqrt(v), inv = nrm > 0.0 ? 1.0 / nrm : 0.0;
       f.out[f.j] = nrm;
-      scal[S_INVNRM] = nrm > 0.0 ? 1.0 / nrm : 0.0;
+      scal[S_LBETA + (f.j & 1)] = nrm;
+      halves(scal + SF_BETA + (f.j & 1), nrm);
+      scal[S_INVNRM] = inv;
+      halves(scal + SF_INV, inv);
       break;
     }
     default:  // F_STORE
@@ -95,30 +136,45 @@ __device__ __forceinline__ void apply_op(double v, const Fin &f) {
   }
 }
 
-// End of a reducing kernel, called by every thread; thread 0 holds the CTA's
-// sum s. The sum goes to partial[blockIdx.x], is made visible device-wide,
-// and the CTA counts itself in. The CTA that arrives last adds all gridDim.x
-// partials in index order (strided per thread, then the CTA tree: the same
-// pattern whichever CTA it is), applies the update and puts the counter back
-// to 0 for the next reduction on the stream.
-__device__ __forceinline__ void finish(double s, const Fin &f) {
-  __shared__ int last;
-  unsigned *ctr = reinterpret_cast<unsigned *>(f.scal + S_CTR);
-  if (threadIdx.x == 0) {
-    f.partial[blockIdx.x] = s;
-    __threadfence();
-    last = atomicAdd(ctr, 1u) == gridDim.x - 1;
-  }
+// End of a kernel with a reduction: the CTA's sum goes to its slot, and
+// reduce_kernel, the next launch, adds the slots. With an arrival counter, and so
+// a gpu-scope fence, in every CTA the product on 2M rows took 123 us in place of
+// 112 (a fence holds up the SM's other CTAs).
+__device__ __forceinline__ void store_partial(double v, double *partial) {
+  __shared__ Fixed sh[KT / 32];
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  const Fixed a[1] = {fixed_of(v)};
+  const Fixed s = warp_sum<1>(a);
+  if (l == 0) sh[w] = s;
   __syncthreads();
-  if (!last) return;
-  __threadfence();
-  double v = 0.0;
-  for (uint32_t k = threadIdx.x; k < gridDim.x; k += KT) v += __ldcg(f.partial + k);
-  v = block_sum(v);
-  if (threadIdx.x == 0) {
-    apply_op(v, f);
-    *ctr = 0u;
+  if (w != 0) return;
+  const Fixed b[1] = {l < KT / 32 ? sh[l] : Fixed{0, 1}};
+  const double t = double_of(warp_sum<1>(b));
+  if (l == 0) partial[blockIdx.x] = t;
+}
+
+constexpr int RT = 1024;  // threads of reduce_kernel
+
+// Adds n partial sums (fixed point: the result does not depend on their order)
+// and applies the scalar update. One CTA.
+__global__ void __launch_bounds__(RT) reduce_kernel(const double *__restrict__ partial, int32_t n, Fin f) {
+  __shared__ Fixed sh[RT / 32];
+  begin();
+  const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
+  Fixed t{0, 1};
+  for (int64_t k0 = w * 32; k0 < n; k0 += 4 * RT) {
+    Fixed a[5];
+    a[4] = l == 0 ? t : Fixed{0, 1};
+#pragma unroll
+    for (int q = 0; q < 4; ++q) a[q] = k0 + q * RT + l < n ? fixed_of(__ldcg(partial + k0 + q * RT + l)) : Fixed{0, 1};
+    t = warp_sum<5>(a);
   }
+  if (l == 0) sh[w] = t;
+  __syncthreads();
+  if (w != 0) return;
+  const Fixed a[1] = {l < RT / 32 ? sh[l] : Fixed{0, 1}};
+  const double v = double_of(warp_sum<1>(a));
+  if (l == 0) apply_op(v, f);
 }
 
 // One sorted row's product in the permuted basis (Listing 2 with the loop
@@ -191,11 +247,12 @@ __device__ __forceinline__ void row_product2(const TV *__restrict__ val, const i
   }
 }
 
-// The reducing kernels below run a grid of at most as many CTAs as fit on the
-// GPU at once and stride over the vectors (element i is taken by thread
-// i mod KT of CTA (i / KT) mod gridDim.x); each thread accumulates its own
-// elements in order, so the sum depends only on the grid size, which the host
-// derives from the device and the kernel alone.
+// The product kernels run a grid of as many CTAs as fit on the GPU at once and
+// stride over the rows: a CTA ends with a barrier and the sum, and with one row
+// per thread those ends cost a tenth (200 steps of CG on 2M rows, CTAs per SM
+// fp64 all / 32 / 16 / 8 29.9 / 28.4 / 27.6 / 27.4 ms, two rows per thread fp32
+// all / 16 / 8 / 6 20.8 / 18.3 / 20.7 / 18.4; eight fit in fp64, six of two rows
+// per thread).
 
 // MODE 0: y = A x and the reduction of sum x_i y_i.  MODE 1: y = bv - A x and
 // the reduction of sum y_i^2 (the fp64 residual of the refinement loop). The
@@ -205,27 +262,27 @@ template <typename TV, typename TX, typename IDX, int MODE>
 __global__ void __launch_bounds__(KT)
     spmv_dot_kernel(const void *__restrict__ val_, const int32_t *__restrict__ col,
                     const int64_t *__restrict__ col_start, const int32_t *__restrict__ block_len,
-                    const TX *__restrict__ x, TX *__restrict__ y, const TX *__restrict__ bv, Fin f, int32_t n_rows,
+                    const TX *__restrict__ x, TX *__restrict__ y, const TX *__restrict__ bv, double *__restrict__ partial, int32_t n_rows,
                     int32_t b) {
+  begin();
   const TV *__restrict__ val = static_cast<const TV *>(val_);
-  double contrib = 0.0;
+  Dot<TX> dot;
   // rows in sorted order: the tile traversal table measured 1.7% slower here
   // (fp64 CG on the 27-point stencil, 4.5M rows)
   for (int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x; i < n_rows; i += (int64_t)gridDim.x * KT) {
-    const int32_t L = __ldg(block_len + (int32_t)(i / b));
+    const int32_t L = __ldg(block_len + (uint32_t)i / (uint32_t)b);
     const auto acc = row_product<TV, TX, IDX>(val, col, col_start, L, i, x);
     TX yi;
     if constexpr (MODE == 0) {
       yi = (TX)acc;
-      contrib += (double)x[i] * (double)yi;
+      dot.add(x[i], yi);
     } else {
       yi = (TX)((double)bv[i] - (double)acc);
-      contrib += (double)yi * (double)yi;
+      dot.add(yi, yi);
     }
     y[i] = yi;
   }
-  const double s = block_sum(contrib);
-  finish(s, f);
+  store_partial(dot.value(), partial);
 }
 
 // y = A x and the reduction of sum x_i y_i with two adjacent rows per thread
@@ -234,37 +291,24 @@ template <typename TV, typename TX, typename IDX>
 __global__ void __launch_bounds__(KT)
     spmv_dot2_kernel(const void *__restrict__ val_, const int32_t *__restrict__ col,
                      const int64_t *__restrict__ col_start, const int32_t *__restrict__ block_len,
-                     const TX *__restrict__ x, TX *__restrict__ y, const TX *__restrict__ bv, Fin f, int32_t n_rows,
+                     const TX *__restrict__ x, TX *__restrict__ y, const TX *__restrict__ bv, double *__restrict__ partial, int32_t n_rows,
                      int32_t b) {
+  begin();
   const TV *__restrict__ val = static_cast<const TV *>(val_);
-  const int64_t n_pairs = ((int64_t)n_rows + 1) / 2;
-  double contrib = 0.0;
-  for (int64_t p = (int64_t)blockIdx.x * KT + threadIdx.x; p < n_pairs; p += (int64_t)gridDim.x * KT) {
-    const int64_t i = 2 * p;
-    const int32_t L = __ldg(block_len + (int32_t)(i / b));
+  Dot<TX> dot;
+  for (int64_t i = 2 * ((int64_t)blockIdx.x * KT + threadIdx.x); i < n_rows; i += 2 * (int64_t)gridDim.x * KT) {
+    const int32_t L = __ldg(block_len + (uint32_t)i / (uint32_t)b);
     typename dev::Acc<TV>::T acc[2];
     row_product2<TV, TX, IDX>(val, col, col_start, L, i, x, acc);
 #pragma unroll
     for (int r = 0; r < 2; ++r)
       if (i + r < n_rows) {
         const TX yi = (TX)acc[r];
-        contrib += (double)x[i + r] * (double)yi;
+        dot.add(x[i + r], yi);
         y[i + r] = yi;
       }
   }
-  const double s = block_sum(contrib);
-  finish(s, f);
-}
-
-template <typename TX>
-__global__ void __launch_bounds__(KT) sumsq_kernel(const TX *__restrict__ v, Fin f, int32_t n) {
-  double contrib = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x; i < n; i += (int64_t)gridDim.x * KT) {
-    const double x = (double)v[i];
-    contrib += x * x;
-  }
-  const double s = block_sum(contrib);
-  finish(s, f);
+  store_partial(dot.value(), partial);
 }
 
 // 16-byte groups of workspace vectors (the workspace is 256-byte aligned):
@@ -283,59 +327,91 @@ struct G16 {
   }
 };
 
-// d += alpha p; r -= alpha q; reduces sum r_i^2. Thread k takes 16-byte
-// groups k, k + stride, ...; the last n mod W elements go one per thread.
-template <typename TX>
-__global__ void __launch_bounds__(KT)
-    cg_update_kernel(TX *__restrict__ d, TX *__restrict__ r, const TX *__restrict__ p, const TX *__restrict__ q,
-                     Fin f, int32_t n) {
+// VG consecutive blocks of KT 16-byte groups of n elements per CTA, one group of
+// each per thread; the elements past the last group go one per thread of CTA 0.
+// load(q, first element) for all of a thread's groups, then use(q, first
+// element); tail(element).
+constexpr int VG = 2;
+template <typename TX, typename FL, typename FU, typename FT>
+__device__ __forceinline__ void groups(int32_t n, FL load, FU use, FT tail) {
   constexpr int W = G16<TX>::W;
-  const TX a = (TX)f.scal[S_ALPHA];
-  const int64_t ng = n / W, stride = (int64_t)gridDim.x * KT, t = (int64_t)blockIdx.x * KT + threadIdx.x;
-  double contrib = 0.0;
-  for (int64_t k = t; k < ng; k += stride) {
-    TX dv[W], rv[W], pv[W], qv[W];
-    G16<TX>::load(d + k * W, dv);
-    G16<TX>::load(r + k * W, rv);
-    G16<TX>::load(p + k * W, pv);
-    G16<TX>::load(q + k * W, qv);
+  const int64_t ng = n / W, k = (int64_t)blockIdx.x * (VG * KT) + threadIdx.x;
 #pragma unroll
-    for (int w = 0; w < W; ++w) {
-      dv[w] = dv[w] + a * pv[w];
-      rv[w] = rv[w] - a * qv[w];
-      contrib += (double)rv[w] * (double)rv[w];
-    }
-    G16<TX>::store(d + k * W, dv);
-    G16<TX>::store(r + k * W, rv);
-  }
-  for (int64_t i = ng * W + t; i < n; i += stride) {
-    d[i] = d[i] + a * p[i];
-    const TX ri = r[i] - a * q[i];
-    r[i] = ri;
-    contrib += (double)ri * (double)ri;
-  }
-  const double s = block_sum(contrib);
-  finish(s, f);
+  for (int q = 0; q < VG; ++q)
+    if (k + q * KT < ng) load(q, (k + q * KT) * W);
+#pragma unroll
+  for (int q = 0; q < VG; ++q)
+    if (k + q * KT < ng) use(q, (k + q * KT) * W);
+  if (blockIdx.x == 0 && threadIdx.x < n - ng * W) tail(ng * W + threadIdx.x);
 }
 
-// p = r + beta p: one 16-byte group per thread, then the last n mod W
-// elements one per thread.
+template <typename TX>
+static int32_t group_grid(int32_t n) {
+  const int64_t per = (int64_t)VG * KT * G16<TX>::W;
+  return (int32_t)std::max<int64_t>(1, (n + per - 1) / per);
+}
+
+// r -= alpha q; reduces sum r_i^2.
 template <typename TX>
 __global__ void __launch_bounds__(KT)
-    cg_dir_kernel(TX *__restrict__ p, const TX *__restrict__ r, const double *__restrict__ scal, int32_t n) {
+    cg_update_kernel(TX *__restrict__ r, const TX *__restrict__ q, const double *__restrict__ scal,
+                     double *__restrict__ partial, int32_t n) {
+  begin();
   constexpr int W = G16<TX>::W;
-  const TX be = (TX)scal[S_BETA];
-  const int64_t ng = n / W, k = (int64_t)blockIdx.x * KT + threadIdx.x;
-  if (k < ng) {
-    TX pv[W], rv[W];
-    G16<TX>::load(p + k * W, pv);
-    G16<TX>::load(r + k * W, rv);
+  const TX a = (TX)scal[S_ALPHA];
+  Dot<TX> dot;
+  TX rv[VG][W], qv[VG][W];
+  groups<TX>(
+      n,
+      [&](int g, int64_t e) {
+        G16<TX>::load(r + e, rv[g]);
+        G16<TX>::load(q + e, qv[g]);
+      },
+      [&](int g, int64_t e) {
 #pragma unroll
-    for (int w = 0; w < W; ++w) pv[w] = rv[w] + be * pv[w];
-    G16<TX>::store(p + k * W, pv);
-  }
-  const int64_t i = ng * W + k;
-  if (i < n) p[i] = r[i] + be * p[i];
+        for (int w = 0; w < W; ++w) {
+          rv[g][w] = rv[g][w] - a * qv[g][w];
+          dot.add(rv[g][w], rv[g][w]);
+        }
+        G16<TX>::store(r + e, rv[g]);
+      },
+      [&](int64_t i) {
+        const TX ri = r[i] - a * q[i];
+        r[i] = ri;
+        dot.add(ri, ri);
+      });
+  store_partial(dot.value(), partial);
+}
+
+// d += alpha p (here, where p is read anyway), p = r + beta p.
+template <typename TX>
+__global__ void __launch_bounds__(KT)
+    cg_dir_kernel(TX *__restrict__ d, TX *__restrict__ p, const TX *__restrict__ r, const double *__restrict__ scal,
+                  int32_t n) {
+  begin();
+  constexpr int W = G16<TX>::W;
+  const TX a = (TX)scal[S_ALPHA], be = (TX)scal[S_BETA];
+  TX dv[VG][W], pv[VG][W], rv[VG][W];
+  groups<TX>(
+      n,
+      [&](int g, int64_t e) {
+        G16<TX>::load(d + e, dv[g]);
+        G16<TX>::load(p + e, pv[g]);
+        G16<TX>::load(r + e, rv[g]);
+      },
+      [&](int g, int64_t e) {
+#pragma unroll
+        for (int w = 0; w < W; ++w) {
+          dv[g][w] = dv[g][w] + a * pv[g][w];
+          pv[g][w] = rv[g][w] + be * pv[g][w];
+        }
+        G16<TX>::store(d + e, dv[g]);
+        G16<TX>::store(p + e, pv[g]);
+      },
+      [&](int64_t i) {
+        d[i] = d[i] + a * p[i];
+        p[i] = r[i] + be * p[i];
+      });
 }
 
 // Start of an inner solve: r = p = (r64 / ||r64||) in the inner type, d = 0,
@@ -343,134 +419,198 @@ __global__ void __launch_bounds__(KT)
 template <typename TL>
 __global__ void __launch_bounds__(KT)
     ir_start_kernel(const double *__restrict__ r64, TL *__restrict__ r, TL *__restrict__ p, TL *__restrict__ d,
-                    Fin f, int32_t n) {
-  const double inv = f.scal[S_INVNRM];
-  double contrib = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x; i < n; i += (int64_t)gridDim.x * KT) {
+                    const double *__restrict__ scal, double *__restrict__ partial, int32_t n) {
+  begin();
+  const double inv = scal[S_INVNRM];
+  Dot<TL> dot;
+  const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
+  if (i < n) {
     const TL ri = (TL)(r64[i] * inv);
     r[i] = ri;
     p[i] = ri;
     d[i] = TL(0);
-    contrib += (double)ri * (double)ri;
+    dot.add(ri, ri);
   }
-  const double s = block_sum(contrib);
-  finish(s, f);
+  store_partial(dot.value(), partial);
 }
 
 // x += ||r64|| d (fp64)
 template <typename TL>
 __global__ void __launch_bounds__(KT)
     ir_correct_kernel(double *__restrict__ x, const TL *__restrict__ d, const double *__restrict__ scal, int32_t n) {
+  begin();
   const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
   if (i < n) x[i] = fma(scal[S_NRM], (double)d[i], x[i]);
 }
 
-// v = v0 / ||v0||, vprev = 0
+template <typename TX>
+__global__ void __launch_bounds__(KT) sumsq_kernel(const TX *__restrict__ v, double *__restrict__ partial, int32_t n) {
+  begin();
+  Dot<TX> dot;
+  const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
+  if (i < n) dot.add(v[i], v[i]);
+  store_partial(dot.value(), partial);
+}
+
+// v = v0 / ||v0||
 template <typename TX>
 __global__ void __launch_bounds__(KT)
-    lanczos_start_kernel(const TX *__restrict__ v0, TX *__restrict__ v, TX *__restrict__ vprev,
-                         const double *__restrict__ scal, int32_t n) {
+    lanczos_start_kernel(const TX *__restrict__ v0, TX *__restrict__ v, const double *__restrict__ scal, int32_t n) {
+  begin();
   const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
-  if (i < n) {
-    v[i] = (TX)((double)v0[i] * scal[S_INVNRM]);
-    vprev[i] = TX(0);
+  if (i < n) v[i] = (TX)((double)v0[i] * scal[S_INVNRM]);
+}
+
+// The fp64 arithmetic of the Lanczos vectors, for floats without the fp64 pipe
+// (six conversions and multiply-adds an element took 20 us a step on 1M rows):
+// error-free products and sums in fp32, rounded once at the end, as good as the
+// fp64 expression to 2^-45 before that rounding; fp64 outside the range where
+// fp32 holds the products' errors.
+// (not inlined, so that the fp64 operations are not speculated on every element)
+__device__ __noinline__ float far_times(float w, double a) { return (float)((double)w * a); }
+__device__ __noinline__ float far_orth(float w, double a, float v, double b, float p) {
+  return (float)((double)w - a * (double)v - b * (double)p);
+}
+template <typename TX>
+struct Coef;
+template <>
+struct Coef<double> {
+  double d;
+  __device__ __forceinline__ Coef(const double *wide, const double *) : d(*wide) {}
+  __device__ __forceinline__ double times(double w) const { return w * d; }
+  // w - a v - b p
+  __device__ __forceinline__ static double orth(double w, const Coef &a, double v, const Coef &b, double p) {
+    return w - a.d * v - b.d * p;
+  }
+};
+template <>
+struct Coef<float> {
+  const double *wide;
+  float2 h;
+  __device__ __forceinline__ Coef(const double *w, const double *two)
+      : wide(w), h(*reinterpret_cast<const float2 *>(two)) {}
+  __device__ __forceinline__ float times(float w) const {
+    const float p = __fmul_rn(w, h.x);
+    if (!in_range(p)) return far_times(w, *wide);
+    return __fadd_rn(p, __fmaf_rn(w, h.y, __fmaf_rn(w, h.x, -p)));
+  }
+  __device__ __forceinline__ static float orth(float w, const Coef &a, float v, const Coef &b, float p) {
+    const float x = __fmul_rn(a.h.x, v), y = __fmul_rn(b.h.x, p);
+    if (!((x == 0.0f && v == 0.0f) || in_range(x)) || !((y == 0.0f && p == 0.0f) || in_range(y)) ||
+        !(w == 0.0f || in_range(w)))
+      return far_orth(w, *a.wide, v, *b.wide, p);
+    const float ex = __fmaf_rn(a.h.y, v, __fmaf_rn(a.h.x, v, -x)), ey = __fmaf_rn(b.h.y, p, __fmaf_rn(b.h.x, p, -y));
+    // w - x = t + et, t - y = u + eu
+    const float t = __fsub_rn(w, x), zt = __fsub_rn(t, w), et = __fsub_rn(__fsub_rn(w, __fsub_rn(t, zt)), __fadd_rn(x, zt));
+    const float u = __fsub_rn(t, y), zu = __fsub_rn(u, t), eu = __fsub_rn(__fsub_rn(t, __fsub_rn(u, zu)), __fadd_rn(y, zu));
+    return __fadd_rn(u, __fsub_rn(__fadd_rn(et, eu), __fadd_rn(ex, ey)));
+  }
+};
+
+// W elements at p, by one load if p allows it (a basis row is caller memory).
+template <typename TX>
+__device__ __forceinline__ void load_any(const TX *p, TX (&v)[G16<TX>::W]) {
+  if (((uintptr_t)p & 15) == 0) {
+    G16<TX>::load(p, v);
+  } else {
+#pragma unroll
+    for (int e = 0; e < G16<TX>::W; ++e) v[e] = p[e];
   }
 }
 
-// w = w - alpha_j v - beta_j vprev (in fp64, stored in TX); reduces sum w_i^2
+// w = w - alpha_j v - beta_j vprev (in fp64, stored in TX); reduces sum w_i^2.
+// vprev: NULL for the first step.
 template <typename TX>
 __global__ void __launch_bounds__(KT)
     lanczos_orth_kernel(TX *__restrict__ w, const TX *__restrict__ v, const TX *__restrict__ vprev,
-                        const double *__restrict__ alpha, const double *__restrict__ beta, int32_t j, Fin f,
-                        int32_t n) {
+                        const double *__restrict__ scal, double *__restrict__ partial, int32_t j, int32_t n) {
   constexpr int W = G16<TX>::W;
-  const double aj = alpha[j], bj = beta[j];
-  const int64_t ng = n / W, stride = (int64_t)gridDim.x * KT, t = (int64_t)blockIdx.x * KT + threadIdx.x;
-  double contrib = 0.0;
-  for (int64_t k = t; k < ng; k += stride) {
-    TX wv[W], vv[W], pv[W];
-    G16<TX>::load(w + k * W, wv);
-    G16<TX>::load(v + k * W, vv);
-    G16<TX>::load(vprev + k * W, pv);
+  begin();
+  const Coef<TX> a(scal + S_LALPHA, scal + SF_ALPHA), b(scal + S_LBETA + (j & 1), scal + SF_BETA + (j & 1));
+  Dot<TX> dot;
+  TX wv[VG][W], vv[VG][W], pv[VG][W];
+  groups<TX>(
+      n,
+      [&](int g, int64_t e) {
+        G16<TX>::load(w + e, wv[g]);
+        load_any(v + e, vv[g]);
+        if (vprev) {
+          load_any(vprev + e, pv[g]);
+        } else {
 #pragma unroll
-    for (int e = 0; e < W; ++e) {
-      const TX ws = (TX)((double)wv[e] - aj * (double)vv[e] - bj * (double)pv[e]);
-      wv[e] = ws;
-      contrib += (double)ws * (double)ws;
-    }
-    G16<TX>::store(w + k * W, wv);
-  }
-  for (int64_t i = ng * W + t; i < n; i += stride) {
-    const double wi = (double)w[i] - aj * (double)v[i] - bj * (double)vprev[i];
-    const TX ws = (TX)wi;
-    w[i] = ws;
-    contrib += (double)ws * (double)ws;
-  }
-  const double s = block_sum(contrib);
-  finish(s, f);
+          for (int k = 0; k < W; ++k) pv[g][k] = TX(0);
+        }
+      },
+      [&](int g, int64_t e) {
+#pragma unroll
+        for (int k = 0; k < W; ++k) {
+          wv[g][k] = Coef<TX>::orth(wv[g][k], a, vv[g][k], b, pv[g][k]);
+          dot.add(wv[g][k], wv[g][k]);
+        }
+        G16<TX>::store(w + e, wv[g]);
+      },
+      [&](int64_t i) {
+        const TX x = Coef<TX>::orth(w[i], a, v[i], b, vprev ? vprev[i] : TX(0));
+        w[i] = x;
+        dot.add(x, x);
+      });
+  store_partial(dot.value(), partial);
 }
 
-// basis_row = v (optional); vprev = v; v = w / beta_{j+1}
+// v = w / beta_{j+1}: the next vector, in its row of the basis if there is one.
 template <typename TX>
 __global__ void __launch_bounds__(KT)
-    lanczos_next_kernel(TX *__restrict__ vprev, TX *__restrict__ v, const TX *__restrict__ w,
-                        const double *__restrict__ scal, TX *__restrict__ basis_row, int32_t n) {
+    lanczos_next_kernel(TX *__restrict__ v, const TX *__restrict__ w, const double *__restrict__ scal, int32_t n) {
   constexpr int W = G16<TX>::W;
-  const double inv = scal[S_INVNRM];
-  const int64_t ng = n / W, k = (int64_t)blockIdx.x * KT + threadIdx.x;
-  // the basis row is caller memory: 16-byte stores only when it is aligned
-  const bool row16 = basis_row && ((uintptr_t)basis_row & 15) == 0;
-  if (k < ng) {
-    TX vv[W], wv[W], nv[W];
-    G16<TX>::load(v + k * W, vv);
-    G16<TX>::load(w + k * W, wv);
-    if (row16) {
-      G16<TX>::store(basis_row + k * W, vv);
-    } else if (basis_row) {
+  begin();
+  const Coef<TX> inv(scal + S_INVNRM, scal + SF_INV);
+  const bool v16 = ((uintptr_t)v & 15) == 0;
+  TX wv[VG][W];
+  groups<TX>(
+      n, [&](int g, int64_t e) { G16<TX>::load(w + e, wv[g]); },
+      [&](int g, int64_t e) {
 #pragma unroll
-      for (int e = 0; e < W; ++e) basis_row[k * W + e] = vv[e];
-    }
-    G16<TX>::store(vprev + k * W, vv);
+        for (int k = 0; k < W; ++k) wv[g][k] = inv.times(wv[g][k]);
+        if (v16) {
+          G16<TX>::store(v + e, wv[g]);
+        } else {
 #pragma unroll
-    for (int e = 0; e < W; ++e) nv[e] = (TX)((double)wv[e] * inv);
-    G16<TX>::store(v + k * W, nv);
-  }
-  const int64_t i = ng * W + k;
-  if (i < n) {
-    const TX vi = v[i];
-    if (basis_row) basis_row[i] = vi;
-    vprev[i] = vi;
-    v[i] = (TX)((double)w[i] * inv);
-  }
+          for (int k = 0; k < W; ++k) v[e + k] = wv[g][k];
+        }
+      },
+      [&](int64_t i) { v[i] = inv.times(w[i]); });
 }
 
 // y = sum_j s_j basis[j] (fp64); reduces sum y_i^2
 template <typename TB>
 __global__ void __launch_bounds__(KT)
     ritz_combine_kernel(const TB *__restrict__ basis, const double *__restrict__ s, int32_t k, int32_t n,
-                        double *__restrict__ y, Fin f) {
+                        double *__restrict__ y, double *__restrict__ partial) {
+  begin();
   double contrib = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x; i < n; i += (int64_t)gridDim.x * KT) {
+  const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
+  if (i < n) {
     double acc = 0.0;
     for (int32_t j = 0; j < k; ++j) acc = fma(s[j], (double)__ldcs(basis + (int64_t)j * n + i), acc);
     y[i] = acc;
-    contrib += acc * acc;
+    contrib = acc * acc;
   }
-  const double sm = block_sum(contrib);
-  finish(sm, f);
+  store_partial(contrib, partial);
 }
 
 // reduces sum (w_i - theta y_i)^2 with theta = scal[S_AUX1] / scal[S_AUX0]
 __global__ void __launch_bounds__(KT)
-    ritz_residual_kernel(const double *__restrict__ w, const double *__restrict__ y, Fin f, int32_t n) {
-  const double theta = f.scal[S_AUX1] / f.scal[S_AUX0];
+    ritz_residual_kernel(const double *__restrict__ w, const double *__restrict__ y, const double *__restrict__ scal,
+                         double *__restrict__ partial, int32_t n) {
+  begin();
+  const double theta = scal[S_AUX1] / scal[S_AUX0];
   double contrib = 0.0;
-  for (int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x; i < n; i += (int64_t)gridDim.x * KT) {
+  const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
+  if (i < n) {
     const double e = w[i] - theta * y[i];
-    contrib += e * e;
+    contrib = e * e;
   }
-  const double s = block_sum(contrib);
-  finish(s, f);
+  store_partial(contrib, partial);
 }
 
 // ----------------------------------------------------------------------------- host helpers
@@ -494,33 +634,6 @@ static int launch_check(const char *what) {
   return e == cudaSuccess ? PJDS_OK : set_error(PJDS_ECUDA, "%s: %s", what, cudaGetErrorString(e));
 }
 
-// Record the launches `body` issues into a graph on a private stream and
-// instantiate it. Nothing executes while capturing.
-template <typename F>
-static int capture_graph(cudaGraphExec_t *exec, F body) {
-  cudaStream_t cap = nullptr;
-  cudaGraph_t g = nullptr;
-  *exec = nullptr;
-  cudaError_t e = cudaStreamCreateWithFlags(&cap, cudaStreamNonBlocking);
-  if (e != cudaSuccess) return set_error(PJDS_ECUDA, "graph stream: %s", cudaGetErrorString(e));
-  e = cudaStreamBeginCapture(cap, cudaStreamCaptureModeThreadLocal);
-  if (e == cudaSuccess) {
-    body(cap);
-    const cudaError_t e_launch = cudaGetLastError();
-    e = cudaStreamEndCapture(cap, &g);
-    if (e == cudaSuccess) e = e_launch;
-  }
-  if (e == cudaSuccess) e = cudaGraphInstantiate(exec, g, 0);
-  if (g) cudaGraphDestroy(g);
-  cudaStreamDestroy(cap);
-  if (e != cudaSuccess) {
-    if (*exec) cudaGraphExecDestroy(*exec);
-    *exec = nullptr;
-    return set_error(PJDS_ECUDA, "graph capture: %s", cudaGetErrorString(e));
-  }
-  return PJDS_OK;
-}
-
 static int check_square_permuted(const pjds_dev *A, const char *name) {
   if (!A) return set_error(PJDS_EINVAL, "%s is NULL", name);
   if (value_bytes(A->dtype) == 0) return set_error(PJDS_EINVAL, "%s: unknown dtype", name);
@@ -533,65 +646,49 @@ static int check_square_permuted(const pjds_dev *A, const char *name) {
   return PJDS_OK;
 }
 
-// CTAs of a reducing kernel: as many as are resident on all SMs at once at
-// the kernel's occupancy (the grid-stride loops cover the rest), at most one
-// per KT elements. Queried outside any stream capture.
-template <typename K>
-static int red_grid(K kernel, int32_t n, int32_t *grid) {
-  int dev = 0, sms = 0, per_sm = 0;
-  cudaError_t e = cudaGetDevice(&dev);
-  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
-  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, kernel, KT, 0);
-  if (e != cudaSuccess) return set_error(PJDS_ECUDA, "occupancy query: %s", cudaGetErrorString(e));
-  if (sms < 1 || per_sm < 1) return set_error(PJDS_ECUDA, "kernel does not fit on an SM");
-  *grid = (int32_t)std::min<int64_t>(std::max<int32_t>(n_blocks_of(n), 1), (int64_t)sms * per_sm);
-  return PJDS_OK;
-}
-
-// A product-and-reduce kernel chosen by value type and index width, with its
-// grid.
+// A product-and-reduce kernel chosen by value type and index width, the rows of
+// a CTA and the CTAs resident on all SMs at once.
 template <typename TX, int MODE>
-struct Dot {
-  void (*fn)(const void *, const int32_t *, const int64_t *, const int32_t *, const TX *, TX *, const TX *, Fin,
+struct DotKernel {
+  void (*fn)(const void *, const int32_t *, const int64_t *, const int32_t *, const TX *, TX *, const TX *, double *,
              int32_t, int32_t);
-  int32_t grid;
+  int32_t rows, resident;
 };
 
 template <typename TV, typename TX, int MODE>
-static int make_dot_typed(const pjds_dev *A, Dot<TX, MODE> *d) {
-  if (A->n_stored + A->n_pad < 0x7fffffffLL)
-    d->fn = spmv_dot_kernel<TV, TX, int32_t, MODE>;
-  else
-    d->fn = spmv_dot_kernel<TV, TX, int64_t, MODE>;
-  return red_grid(d->fn, A->n_rows, &d->grid);
+static void dot_typed(const pjds_dev *A, DotKernel<TX, MODE> *d) {
+  const bool wide = A->n_stored + A->n_pad >= 0x7fffffffLL;
+  d->fn = wide ? spmv_dot_kernel<TV, TX, int64_t, MODE> : spmv_dot_kernel<TV, TX, int32_t, MODE>;
+  d->rows = KT;
 }
 
-template <typename TX, int MODE>
-static int make_dot(const pjds_dev *A, Dot<TX, MODE> *d);
-template <>
-int make_dot<double, 0>(const pjds_dev *A, Dot<double, 0> *d) {
-  return make_dot_typed<double, double, 0>(A, d);
-}
-template <>
-int make_dot<double, 1>(const pjds_dev *A, Dot<double, 1> *d) {
-  return make_dot_typed<double, double, 1>(A, d);
-}
 // fp32 / bf16 values: two rows per thread when val and col allow the paired
 // loads (one 8- or 4-byte value load and one 8-byte column load per diagonal)
 template <typename TV>
-static int make_dot2(const pjds_dev *A, Dot<float, 0> *d) {
-  if (A->n_stored + A->n_pad < 0x7fffffffLL)
-    d->fn = spmv_dot2_kernel<TV, float, int32_t>;
-  else
-    d->fn = spmv_dot2_kernel<TV, float, int64_t>;
-  return red_grid(d->fn, (int32_t)(((int64_t)A->n_rows + 1) / 2), &d->grid);
+static void dot_float(const pjds_dev *A, DotKernel<float, 0> *d) {
+  const bool pair = ((uintptr_t)A->val % (2 * value_bytes(A->dtype))) == 0 && ((uintptr_t)A->col % 8) == 0;
+  if (!pair) return dot_typed<TV, float, 0>(A, d);
+  const bool wide = A->n_stored + A->n_pad >= 0x7fffffffLL;
+  d->fn = wide ? spmv_dot2_kernel<TV, float, int64_t> : spmv_dot2_kernel<TV, float, int32_t>;
+  d->rows = 2 * KT;
 }
 
-template <>
-int make_dot<float, 0>(const pjds_dev *A, Dot<float, 0> *d) {
-  const bool pair = ((uintptr_t)A->val % (2 * value_bytes(A->dtype))) == 0 && ((uintptr_t)A->col % 8) == 0;
-  if (pair) return A->dtype == PJDS_BF16 ? make_dot2<dev::bf16_t>(A, d) : make_dot2<float>(A, d);
-  return A->dtype == PJDS_BF16 ? make_dot_typed<dev::bf16_t, float, 0>(A, d) : make_dot_typed<float, float, 0>(A, d);
+template <typename TX, int MODE>
+static int make_dot(const pjds_dev *A, DotKernel<TX, MODE> *d) {
+  if constexpr (sizeof(TX) == 8)
+    dot_typed<double, double, MODE>(A, d);
+  else if (A->dtype == PJDS_BF16)
+    dot_float<dev::bf16_t>(A, d);
+  else
+    dot_float<float>(A, d);
+  int dev = 0, sms = 0, per_sm = 0;
+  cudaError_t e = cudaGetDevice(&dev);
+  if (e == cudaSuccess) e = cudaDeviceGetAttribute(&sms, cudaDevAttrMultiProcessorCount, dev);
+  if (e == cudaSuccess) e = cudaOccupancyMaxActiveBlocksPerMultiprocessor(&per_sm, d->fn, KT, 0);
+  if (e != cudaSuccess) return set_error(PJDS_ECUDA, "occupancy query: %s", cudaGetErrorString(e));
+  if (sms < 1 || per_sm < 1) return set_error(PJDS_ECUDA, "kernel does not fit on an SM");
+  d->resident = sms * per_sm;
+  return PJDS_OK;
 }
 
 template <typename T>
@@ -599,18 +696,58 @@ struct Same {
   using type = T;
 };
 
-// (the vector type is taken from the launcher alone)
+// Launch with programmatic dependence on the kernel before (see begin()).
+template <typename... P, typename... A>
+static void launch(void (*kernel)(P...), int64_t grid, int threads, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3((unsigned)grid);
+  c.blockDim = dim3((unsigned)threads);
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
+// What the reductions need in a workspace, before its vectors: partial sums and
+// the scalar block.
+struct Reduce {
+  double *partial, *scal;
+  static size_t bytes(int32_t n) { return align256((size_t)n_blocks_of(n) * 8) + align256(S_COUNT * 8); }
+  static Reduce take(Carve &cv, int32_t n) {
+    Reduce r;
+    r.partial = cv.take<double>((size_t)n_blocks_of(n));
+    r.scal = cv.take<double>(S_COUNT);
+    return r;
+  }
+  int clear(cudaStream_t s) const {
+    const cudaError_t e = cudaMemsetAsync(scal, 0, S_COUNT * 8, s);
+    return e == cudaSuccess ? PJDS_OK : set_error(PJDS_ECUDA, "workspace: %s", cudaGetErrorString(e));
+  }
+  // add the n partial sums of the kernel before
+  void sum(int64_t n, cudaStream_t s, int32_t op, int32_t j = 0, double *out = nullptr) const {
+    launch(reduce_kernel, 1, RT, s, partial, (int32_t)n, Fin{scal, out, op, j});
+  }
+};
+
+// y = A x and the inner product into red (the vector type is taken from the
+// kernel alone).
 template <typename TX, int MODE>
-static void launch_dot(const Dot<TX, MODE> &d, const pjds_dev *A, const typename Same<TX>::type *x,
-                       typename Same<TX>::type *y, const typename Same<TX>::type *bv, const Fin &f, cudaStream_t s) {
-  d.fn<<<d.grid, KT, 0, s>>>(A->val, A->col, A->col_start, A->block_len, x, y, bv, f, A->n_rows, A->b);
+static void launch_dot(const DotKernel<TX, MODE> &d, const pjds_dev *A, const typename Same<TX>::type *x,
+                       typename Same<TX>::type *y, const typename Same<TX>::type *bv, const Reduce &red, cudaStream_t s,
+                       int32_t op, int32_t j = 0, double *out = nullptr) {
+  const int64_t grid = std::min<int64_t>(((int64_t)A->n_rows + d.rows - 1) / d.rows, d.resident);
+  launch(d.fn, grid, KT, s, A->val, A->col, A->col_start, A->block_len, x, y, bv, red.partial, A->n_rows, A->b);
+  red.sum(grid, s, op, j, out);
 }
 
 // ----------------------------------------------------------------------------- CG
 
 static size_t cg_bytes(int32_t n, int vec_bytes) {
-  return align256((size_t)n_blocks_of(n) * 8) + align256(S_COUNT * 8) + 4 * align256((size_t)n * vec_bytes) +
-         align256((size_t)n * 8) + align256(sizeof(CgOut)) + align256(cg_slots_bytes());
+  return Reduce::bytes(n) + 4 * align256((size_t)n * vec_bytes) + align256((size_t)n * 8) +
+         align256(sizeof(CgOut)) + align256(cg_slots_bytes());
 }
 
 template <typename TL>
@@ -618,8 +755,8 @@ static int cg_run(const pjds_dev *Ah, const pjds_dev *Al, const double *b, doubl
                   pjds_cg_result *res, void *work, cudaStream_t s) {
   const int32_t n = Ah->n_rows, nb = n_blocks_of(n);
   Carve cv{static_cast<char *>(work), 0, 0};
-  double *partial = cv.take<double>((size_t)nb);
-  double *scal = cv.take<double>(S_COUNT);
+  const Reduce red = Reduce::take(cv, n);
+  double *const scal = red.scal;
   TL *r = cv.take<TL>((size_t)n), *p = cv.take<TL>((size_t)n), *q = cv.take<TL>((size_t)n);
   TL *d = cv.take<TL>((size_t)n);
   double *r64 = cv.take<double>((size_t)n);
@@ -634,52 +771,27 @@ static int cg_run(const pjds_dev *Ah, const pjds_dev *Al, const double *b, doubl
     if (res) *res = small_res;
     return PJDS_OK;
   }
-  auto fin = [&](int32_t op, int32_t j) { return Fin{partial, scal, nullptr, op, j}; };
+  DotKernel<TL, 0> dot_lo;
+  DotKernel<double, 1> dot_res;
+  const int32_t g_vec = group_grid<TL>(n);
   int rc;
-  Dot<TL, 0> dot_lo;
-  Dot<double, 1> dot_res;
-  int32_t g_sumsq = 0, g_upd = 0, g_start = 0;
-  if ((rc = make_dot(Al, &dot_lo)) || (rc = make_dot(Ah, &dot_res)) || (rc = red_grid(sumsq_kernel<double>, n, &g_sumsq)) ||
-      (rc = red_grid(cg_update_kernel<TL>, n, &g_upd)) || (rc = red_grid(ir_start_kernel<TL>, n, &g_start)))
-    return rc;
-  // cg_dir: one thread per 16-byte group, and as many for the remainder
-  const int64_t n_groups = n / G16<TL>::W, n_rem = n - n_groups * G16<TL>::W;
-  const int32_t nb_dir = (int32_t)((std::max<int64_t>(std::max(n_groups, n_rem), 1) + KT - 1) / KT);
-
-  // scalar block and reduction counter start at 0
-  cudaError_t e = cudaMemsetAsync(scal, 0, S_COUNT * sizeof(double), s);
-  if (e != cudaSuccess) return set_error(PJDS_ECUDA, "cg: %s", cudaGetErrorString(e));
+  if ((rc = make_dot(Al, &dot_lo)) || (rc = make_dot(Ah, &dot_res)) || (rc = red.clear(s))) return rc;
   // ||b||
-  sumsq_kernel<double><<<g_sumsq, KT, 0, s>>>(b, fin(F_STORE, S_AUX2), n);
+  launch(sumsq_kernel<double>, nb, KT, s, b, red.partial, n);
+  red.sum(nb, s, F_STORE, S_AUX2);
   double bn2 = 0.0;
   if ((rc = launch_check("cg ||b||"))) return rc;
-  e = cudaMemcpyAsync(&bn2, scal + S_AUX2, sizeof(double), cudaMemcpyDeviceToHost, s);
+  cudaError_t e = cudaMemcpyAsync(&bn2, scal + S_AUX2, sizeof(double), cudaMemcpyDeviceToHost, s);
   if (e == cudaSuccess) e = cudaStreamSynchronize(s);
   if (e != cudaSuccess) return set_error(PJDS_ECUDA, "cg: %s", cudaGetErrorString(e));
   const double bnorm = sqrt(bn2);
-
-  auto inner_step = [&](cudaStream_t st) {
-    launch_dot(dot_lo, Al, p, q, nullptr, fin(F_ALPHA, 0), st);                  // q = A p, (p, q), alpha
-    cg_update_kernel<TL><<<g_upd, KT, 0, st>>>(d, r, p, q, fin(F_BETA, 0), n);  // d, r, (r, r), beta
-    cg_dir_kernel<TL><<<nb_dir, KT, 0, st>>>(p, r, scal, n);                    // p
-  };
-
-  cudaGraphExec_t exec = nullptr;
-  if (o.use_graph) {
-    // recorded on a private stream (nothing runs during capture; the legacy
-    // default stream cannot be captured), replayed on the caller's stream
-    rc = capture_graph(&exec, [&](cudaStream_t st) {
-      for (int it = 0; it < o.inner_iters; ++it) inner_step(st);
-    });
-    if (rc) return rc;
-  }
 
   pjds_cg_result out;
   memset(&out, 0, sizeof(out));
   double rel = 0.0;
   rc = PJDS_OK;
   for (int outer = 0;; ++outer) {
-    launch_dot(dot_res, Ah, x, r64, b, fin(F_NORM, 0), s);  // r64 = b - A x, ||r64||
+    launch_dot(dot_res, Ah, x, r64, b, red, s, F_NORM);  // r64 = b - A x, ||r64||
     if ((rc = launch_check("cg residual"))) break;
     double rn = 0.0;
     e = cudaMemcpyAsync(&rn, scal + S_NRM, sizeof(double), cudaMemcpyDeviceToHost, s);
@@ -691,22 +803,19 @@ static int cg_run(const pjds_dev *Ah, const pjds_dev *Al, const double *b, doubl
     rel = bnorm > 0.0 ? rn / bnorm : rn;
     if (out.n_history < PJDS_CG_HISTORY) out.history[out.n_history++] = rel;
     if (outer >= o.max_outer || rel <= o.tol || rn == 0.0) break;
-    ir_start_kernel<TL><<<g_start, KT, 0, s>>>(r64, r, p, d, fin(F_RR, 0), n);
-    if (exec) {
-      e = cudaGraphLaunch(exec, s);
-      if (e != cudaSuccess) {
-        rc = set_error(PJDS_ECUDA, "cg graph launch: %s", cudaGetErrorString(e));
-        break;
-      }
-    } else {
-      for (int it = 0; it < o.inner_iters; ++it) inner_step(s);
+    launch(ir_start_kernel<TL>, nb, KT, s, r64, r, p, d, scal, red.partial, n);
+    red.sum(nb, s, F_RR);
+    for (int it = 0; it < o.inner_iters; ++it) {
+      launch_dot(dot_lo, Al, p, q, nullptr, red, s, F_ALPHA);                   // q = A p, (p, q), alpha
+      launch(cg_update_kernel<TL>, g_vec, KT, s, r, q, scal, red.partial, n);  // r, (r, r), beta
+      red.sum(g_vec, s, F_BETA);
+      launch(cg_dir_kernel<TL>, g_vec, KT, s, d, p, r, scal, n);  // d, p
     }
-    ir_correct_kernel<TL><<<nb, KT, 0, s>>>(x, d, scal, n);
+    launch(ir_correct_kernel<TL>, nb, KT, s, x, d, scal, n);
     if ((rc = launch_check("cg inner"))) break;
     out.outer = outer + 1;
     out.inner_total += o.inner_iters;
   }
-  if (exec) cudaGraphExecDestroy(exec);
   out.rel_residual = rel;
   if (res) *res = out;
   return rc;
@@ -754,53 +863,38 @@ extern "C" int pjds_cg_solve(const pjds_dev *A_hi, const pjds_dev *A_lo, const d
 // ----------------------------------------------------------------------------- Lanczos
 
 static size_t lanczos_bytes(int32_t n, int vec_bytes, int32_t steps) {
-  return align256((size_t)n_blocks_of(n) * 8) + align256(S_COUNT * 8) + align256((size_t)steps * 8) +
-         align256((size_t)(steps + 1) * 8) + 3 * align256((size_t)n * vec_bytes);
+  return Reduce::bytes(n) + align256((size_t)steps * 8) + align256((size_t)(steps + 1) * 8) +
+         3 * align256((size_t)n * vec_bytes);
 }
 
 template <typename TX>
 static int lanczos_run(const pjds_dev *A, const TX *v0, int32_t steps, double *alpha_h, double *beta_h, TX *basis,
-                       int use_graph, void *work, cudaStream_t s) {
+                       void *work, cudaStream_t s) {
   const int32_t n = A->n_rows, nb = n_blocks_of(n);
   Carve cv{static_cast<char *>(work), 0, 0};
-  double *partial = cv.take<double>((size_t)nb);
-  double *scal = cv.take<double>(S_COUNT);
+  const Reduce red = Reduce::take(cv, n);
   double *alpha = cv.take<double>((size_t)steps);
   double *beta = cv.take<double>((size_t)steps + 1);
-  TX *v = cv.take<TX>((size_t)n), *vp = cv.take<TX>((size_t)n), *w = cv.take<TX>((size_t)n);
-  cudaError_t e = cudaMemsetAsync(beta, 0, sizeof(double) * ((size_t)steps + 1), s);
-  if (e == cudaSuccess) e = cudaMemsetAsync(scal, 0, S_COUNT * sizeof(double), s);
-  if (e != cudaSuccess) return set_error(PJDS_ECUDA, "lanczos: %s", cudaGetErrorString(e));
-  Dot<TX, 0> dot;
-  int32_t g_sumsq = 0, g_orth = 0;
+  TX *buf[2] = {cv.take<TX>((size_t)n), nullptr};
+  buf[1] = cv.take<TX>((size_t)n);
+  TX *w = cv.take<TX>((size_t)n);
+  DotKernel<TX, 0> dot;
   int rc;
-  if ((rc = make_dot(A, &dot)) || (rc = red_grid(sumsq_kernel<TX>, n, &g_sumsq)) ||
-      (rc = red_grid(lanczos_orth_kernel<TX>, n, &g_orth)))
-    return rc;
-  // lanczos_next: one thread per 16-byte group, and as many for the remainder
-  const int64_t n_groups = n / G16<TX>::W, n_rem = n - n_groups * G16<TX>::W;
-  const int32_t nb_next = (int32_t)((std::max<int64_t>(std::max(n_groups, n_rem), 1) + KT - 1) / KT);
-  sumsq_kernel<TX><<<g_sumsq, KT, 0, s>>>(v0, Fin{partial, scal, nullptr, F_NORM, 0}, n);
-  lanczos_start_kernel<TX><<<nb, KT, 0, s>>>(v0, v, vp, scal, n);
-  rc = launch_check("lanczos start");
-  if (rc) return rc;
-  auto step = [&](int32_t j, cudaStream_t st) {
-    launch_dot(dot, A, v, w, nullptr, Fin{partial, scal, alpha, F_LALPHA, j}, st);  // w = A v, alpha_j = (v, w)
-    lanczos_orth_kernel<TX>
-        <<<g_orth, KT, 0, st>>>(w, v, vp, alpha, beta, j, Fin{partial, scal, beta, F_LBETA, j + 1}, n);  // beta_j+1
-    lanczos_next_kernel<TX><<<nb_next, KT, 0, st>>>(vp, v, w, scal, basis ? basis + (int64_t)j * n : nullptr, n);
-  };
-  if (use_graph) {
-    cudaGraphExec_t exec = nullptr;
-    rc = capture_graph(&exec, [&](cudaStream_t st) {
-      for (int32_t j = 0; j < steps; ++j) step(j, st);
-    });
-    if (rc) return rc;
-    e = cudaGraphLaunch(exec, s);
-    cudaGraphExecDestroy(exec);
-    if (e != cudaSuccess) return set_error(PJDS_ECUDA, "lanczos graph launch: %s", cudaGetErrorString(e));
-  } else {
-    for (int32_t j = 0; j < steps; ++j) step(j, s);
+  if ((rc = make_dot(A, &dot)) || (rc = red.clear(s))) return rc;
+  cudaError_t e = cudaMemsetAsync(beta, 0, sizeof(double), s);
+  if (e != cudaSuccess) return set_error(PJDS_ECUDA, "lanczos: %s", cudaGetErrorString(e));
+  const int32_t g_vec = group_grid<TX>(n);
+  // v_j: its row of the caller's basis, else the two buffers in turn
+  auto vec = [&](int32_t j) { return basis ? basis + (int64_t)j * n : buf[j & 1]; };
+  launch(sumsq_kernel<TX>, nb, KT, s, v0, red.partial, n);
+  red.sum(nb, s, F_NORM);
+  launch(lanczos_start_kernel<TX>, nb, KT, s, v0, vec(0), red.scal, n);
+  for (int32_t j = 0; j < steps; ++j) {
+    TX *const v = vec(j);
+    launch_dot(dot, A, v, w, nullptr, red, s, F_LALPHA, j, alpha);  // w = A v, alpha_j = (v, w)
+    launch(lanczos_orth_kernel<TX>, g_vec, KT, s, w, v, j > 0 ? vec(j - 1) : nullptr, red.scal, red.partial, j, n);
+    red.sum(g_vec, s, F_LBETA, j + 1, beta);  // beta_j+1
+    if (j + 1 < steps) launch(lanczos_next_kernel<TX>, g_vec, KT, s, vec(j + 1), w, red.scal, n);
   }
   if ((rc = launch_check("lanczos steps"))) return rc;
   e = cudaMemcpyAsync(alpha_h, alpha, sizeof(double) * (size_t)steps, cudaMemcpyDeviceToHost, s);
@@ -829,12 +923,13 @@ extern "C" int pjds_lanczos(const pjds_dev *A, const void *v0, int32_t steps, do
   if (!v0 || !alpha_host || !beta_host || !work) return set_error(PJDS_EINVAL, "a pointer argument is NULL");
   const int vb = vector_bytes(A->dtype);
   if (work_bytes < lanczos_bytes(A->n_rows, vb, steps)) return set_error(PJDS_EINVAL, "workspace too small");
+  (void)use_graph;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (A->dtype == PJDS_F64)
     return lanczos_run<double>(A, static_cast<const double *>(v0), steps, alpha_host, beta_host,
-                               static_cast<double *>(basis), use_graph, work, s);
+                               static_cast<double *>(basis), work, s);
   return lanczos_run<float>(A, static_cast<const float *>(v0), steps, alpha_host, beta_host,
-                            static_cast<float *>(basis), use_graph, work, s);
+                            static_cast<float *>(basis), work, s);
 }
 
 // ----------------------------------------------------------------------------- tridiagonal eigenpair (host)
@@ -944,8 +1039,7 @@ extern "C" int pjds_tridiag_extreme(int32_t k, const double *alpha, const double
 // ----------------------------------------------------------------------------- Ritz refinement
 
 static size_t ritz_bytes(int32_t n, int32_t k) {
-  return align256((size_t)n_blocks_of(n) * 8) + align256(S_COUNT * 8) + align256((size_t)k * 8) +
-         align256((size_t)n * 8);
+  return Reduce::bytes(n) + align256((size_t)k * 8) + align256((size_t)n * 8);
 }
 
 extern "C" int pjds_ritz_workspace_bytes(int32_t n_rows, int32_t n_pad, int32_t k, size_t *bytes) {
@@ -970,30 +1064,24 @@ extern "C" int pjds_ritz_refine(const pjds_dev *A_hi, const void *basis, int32_t
   if (work_bytes < ritz_bytes(n, k)) return set_error(PJDS_EINVAL, "workspace too small");
   cudaStream_t st = static_cast<cudaStream_t>(stream);
   Carve cv{static_cast<char *>(work), 0, 0};
-  double *partial = cv.take<double>((size_t)nb);
-  double *scal = cv.take<double>(S_COUNT);
+  const Reduce red = Reduce::take(cv, n);
   double *sd = cv.take<double>((size_t)k);
   double *w = cv.take<double>((size_t)n);
+  DotKernel<double, 0> dot;
+  if ((rc = make_dot(A_hi, &dot)) || (rc = red.clear(st))) return rc;
   cudaError_t e = cudaMemcpyAsync(sd, s_host, sizeof(double) * (size_t)k, cudaMemcpyHostToDevice, st);
-  if (e == cudaSuccess) e = cudaMemsetAsync(scal, 0, S_COUNT * sizeof(double), st);
   if (e != cudaSuccess) return set_error(PJDS_ECUDA, "ritz: %s", cudaGetErrorString(e));
-  const Fin f_yy{partial, scal, nullptr, F_STORE, S_AUX0}, f_yw{partial, scal, nullptr, F_STORE, S_AUX1},
-      f_ee{partial, scal, nullptr, F_STORE, S_AUX2};
-  Dot<double, 0> dot;
-  int32_t g_comb = 0, g_res = 0;
-  if ((rc = make_dot(A_hi, &dot)) || (rc = red_grid(ritz_residual_kernel, n, &g_res)) ||
-      (rc = basis_dtype == PJDS_F64 ? red_grid(ritz_combine_kernel<double>, n, &g_comb)
-                                    : red_grid(ritz_combine_kernel<float>, n, &g_comb)))
-    return rc;
   if (basis_dtype == PJDS_F64)
-    ritz_combine_kernel<double><<<g_comb, KT, 0, st>>>(static_cast<const double *>(basis), sd, k, n, y, f_yy);
+    launch(ritz_combine_kernel<double>, nb, KT, st, static_cast<const double *>(basis), sd, k, n, y, red.partial);
   else
-    ritz_combine_kernel<float><<<g_comb, KT, 0, st>>>(static_cast<const float *>(basis), sd, k, n, y, f_yy);
-  launch_dot(dot, A_hi, y, w, nullptr, f_yw, st);  // w = A y, (y, w)
-  ritz_residual_kernel<<<g_res, KT, 0, st>>>(w, y, f_ee, n);
+    launch(ritz_combine_kernel<float>, nb, KT, st, static_cast<const float *>(basis), sd, k, n, y, red.partial);
+  red.sum(nb, st, F_STORE, S_AUX0);
+  launch_dot(dot, A_hi, y, w, nullptr, red, st, F_STORE, S_AUX1);  // w = A y, (y, w)
+  launch(ritz_residual_kernel, nb, KT, st, w, y, red.scal, red.partial, n);
+  red.sum(nb, st, F_STORE, S_AUX2);
   if ((rc = launch_check("ritz refine"))) return rc;
   double h[3];
-  e = cudaMemcpyAsync(h, scal + S_AUX0, sizeof(h), cudaMemcpyDeviceToHost, st);
+  e = cudaMemcpyAsync(h, red.scal + S_AUX0, sizeof(h), cudaMemcpyDeviceToHost, st);
   if (e == cudaSuccess) e = cudaStreamSynchronize(st);
   if (e != cudaSuccess) return set_error(PJDS_ECUDA, "ritz: %s", cudaGetErrorString(e));
   if (!(h[0] > 0.0)) return set_error(PJDS_EINVAL, "Ritz vector is zero");
@@ -1079,10 +1167,7 @@ extern "C" int pjds_cg_solve_static(const pjds_dev *A_hi, const pjds_dev *A_lo, 
   void *work = nullptr;
   if ((rc = cg_static_workspace(&work))) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
-  // The array keeps the previous call's contents: clear the partial sums and
-  // the scalar block; every vector is written before it is read.
-  const size_t head = align256((size_t)n_blocks_of(A_hi->n_rows) * 8) + align256(S_COUNT * 8);
-  cudaError_t e = cudaMemsetAsync(work, 0, head, s);
-  if (e != cudaSuccess) return set_error(PJDS_ECUDA, "clear static workspace: %s", cudaGetErrorString(e));
+  // The array keeps the previous call's contents: cg_run clears its counters and
+  // scalars, and writes every vector and partial sum before reading it.
   return low ? cg_run<float>(A_hi, A_lo, b, x, o, res, work, s) : cg_run<double>(A_hi, A_lo, b, x, o, res, work, s);
 }

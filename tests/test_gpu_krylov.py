@@ -233,3 +233,24 @@ def test_cg_small_and_large_systems(mods, oracle_lib, name, n, lo, max_outer):
     assert rel <= 1e-12, (rel, res)
     assert res["rel_residual"] <= 1e-12 and res["inner_total"] == 20 * res["outer"]
     assert len(res["history"]) == res["outer"] + 1 and res["history"][-1] == res["rel_residual"]
+
+
+# vectors far outside the range in which fp32 holds a product and its rounding
+# error: powers of two scale every step exactly, so the coefficients follow
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("power", [-70, 80])
+def test_lanczos_scales_with_the_matrix(mods, dtype, power):
+    torch, pjds, krylov = mods
+    A = synth.stencil27(g=13, seed=6)  # 2197 rows: a remainder after the 16-byte groups
+    v0 = synth.vector(A.n_rows, seed=3)
+    D, perm = _dev(pjds, A, dtype)
+    S, _ = _dev(pjds, A._replace(val=A.val * 2.0 ** power), dtype)
+    v = torch.from_numpy(v0[perm]).to("cuda", D.vec_dtype)
+    a1, b1, V1 = krylov.lanczos(D, v, 6, keep_basis=True)
+    a2, b2, V2 = krylov.lanczos(S, v, 6, keep_basis=True)
+    # in fp64 every operation scales exactly; with floats a sum is taken in another way, within its rounding
+    # (2^-45) before the vectors' own (2^-24), which six steps amplify by less than 10
+    tol = 1e-13 if dtype == "f64" else 1e-6
+    assert np.allclose(a2 * 2.0 ** -power, a1, rtol=tol, atol=tol * np.abs(a1).max())
+    assert np.allclose(b2 * 2.0 ** -power, b1, rtol=tol, atol=0)
+    assert float((V1.double() - V2.double()).abs().max()) <= tol
