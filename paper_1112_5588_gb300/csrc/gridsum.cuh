@@ -106,18 +106,27 @@ __device__ __forceinline__ Fixed warp_sum(const Fixed (&a)[N]) {
   static_assert(N <= 8, "carries beyond 63 bits");
   long long f = 0;
 #pragma unroll
-  for (int q = 0; q < N; ++q) f += a[q].f >> min(em - a[q].e + drop, 63u);
+  for (int q = 0; q < N; ++q) {
+    const uint32_t d = min(em - a[q].e + drop, 62u);
+    // to nearest where many are cut: 160 of them would add up to 80 units
+    f += N > 1 ? (a[q].f + ((1ll << d) >> 1)) >> d : a[q].f >> d;
+  }
   // in three parts, whose sums over 32 lanes fit 32 bits
   const uint32_t s0 = __reduce_add_sync(0xffffffffu, (uint32_t)f & 0x3ffffffu);
   const uint32_t s1 = __reduce_add_sync(0xffffffffu, (uint32_t)(f >> 26) & 0x3ffffffu);
   const int32_t s2 = __reduce_add_sync(0xffffffffu, (int32_t)(f >> 52));
   f = (long long)s0 + ((long long)s1 << 26) + ((long long)s2 << 52);
-  // back below 2^57, with as many bits as there are
+  // back to 57 bits: below 2^57, and up to it, so that the next sum's shifts drop zeros
   const unsigned long long m = f < 0 ? 0ull - (unsigned long long)f : (unsigned long long)f;
-  const int sh = m ? 7 - __clzll((long long)m) : 0;  // > 0: too large by sh bits
-  if (sh > 0) f >>= sh;
+  int sh = m ? 7 - __clzll((long long)m) : 0;  // > 0: too large by sh bits
+  if (sh > 0) {
+    f >>= sh;
+  } else {
+    sh = -min(-sh, (int)em + drop - 1);
+    f = (long long)((unsigned long long)f << -sh);
+  }
   s.f = f;
-  s.e = em + drop + (sh > 0 ? sh : 0);
+  s.e = (uint32_t)((int)em + drop + sh);
   if (s.e >= 0x7ffu) {  // the sum overflows
     s.e = 0x7ffu;
     s.f = f < 0 ? (long long)0xfff0000000000000ull : 0x7ff0000000000000ll;

@@ -83,10 +83,14 @@ struct Fin {
 };
 
 // Programmatic dependent launch: every kernel lets the next one on the stream
-// start (so that its launch is over when this one ends) and waits for the one
-// before it, completed and visible, before it touches memory.
+// start (so that its launch is over when this one ends), and that one waits for
+// this one, completed and visible, before it touches memory. A load through the
+// read-only path may be moved ahead of that wait, so no pointer in those kernels
+// is __restrict__. The products, which gather through it, are launched after the
+// kernel before them has ended.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void begin() {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  let_next_start();
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -155,25 +159,21 @@ __device__ __forceinline__ void store_partial(double v, double *partial) {
 
 constexpr int RT = 1024;  // threads of reduce_kernel
 
-// Adds n partial sums (fixed point: the result does not depend on their order)
-// and applies the scalar update. One CTA.
-__global__ void __launch_bounds__(RT) reduce_kernel(const double *__restrict__ partial, int32_t n, Fin f) {
+// Adds n partial sums (one or two a thread after a product) and applies the
+// scalar update. One CTA.
+__global__ void __launch_bounds__(RT) reduce_kernel(const double *partial, int32_t n, Fin f) {
   __shared__ Fixed sh[RT / 32];
   begin();
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  Fixed t{0, 1};
-  for (int64_t k0 = w * 32; k0 < n; k0 += 4 * RT) {
-    Fixed a[5];
-    a[4] = l == 0 ? t : Fixed{0, 1};
-#pragma unroll
-    for (int q = 0; q < 4; ++q) a[q] = k0 + q * RT + l < n ? fixed_of(__ldcg(partial + k0 + q * RT + l)) : Fixed{0, 1};
-    t = warp_sum<5>(a);
-  }
+  double v = 0.0;
+  for (int32_t k = threadIdx.x; k < n; k += RT) v += __ldcg(partial + k);
+  const Fixed one[1] = {fixed_of(v)};
+  const Fixed t = warp_sum<1>(one);
   if (l == 0) sh[w] = t;
   __syncthreads();
   if (w != 0) return;
   const Fixed a[1] = {l < RT / 32 ? sh[l] : Fixed{0, 1}};
-  const double v = double_of(warp_sum<1>(a));
+  v = double_of(warp_sum<1>(a));
   if (l == 0) apply_op(v, f);
 }
 
@@ -262,9 +262,9 @@ template <typename TV, typename TX, typename IDX, int MODE>
 __global__ void __launch_bounds__(KT)
     spmv_dot_kernel(const void *__restrict__ val_, const int32_t *__restrict__ col,
                     const int64_t *__restrict__ col_start, const int32_t *__restrict__ block_len,
-                    const TX *__restrict__ x, TX *__restrict__ y, const TX *__restrict__ bv, double *__restrict__ partial, int32_t n_rows,
-                    int32_t b) {
-  begin();
+                    const TX *__restrict__ x, TX *__restrict__ y, const TX *__restrict__ bv,
+                    double *__restrict__ partial, int32_t n_rows, int32_t b) {
+  let_next_start();
   const TV *__restrict__ val = static_cast<const TV *>(val_);
   Dot<TX> dot;
   // rows in sorted order: the tile traversal table measured 1.7% slower here
@@ -291,9 +291,9 @@ template <typename TV, typename TX, typename IDX>
 __global__ void __launch_bounds__(KT)
     spmv_dot2_kernel(const void *__restrict__ val_, const int32_t *__restrict__ col,
                      const int64_t *__restrict__ col_start, const int32_t *__restrict__ block_len,
-                     const TX *__restrict__ x, TX *__restrict__ y, const TX *__restrict__ bv, double *__restrict__ partial, int32_t n_rows,
-                     int32_t b) {
-  begin();
+                     const TX *__restrict__ x, TX *__restrict__ y, const TX *__restrict__ bv,
+                     double *__restrict__ partial, int32_t n_rows, int32_t b) {
+  let_next_start();
   const TV *__restrict__ val = static_cast<const TV *>(val_);
   Dot<TX> dot;
   for (int64_t i = 2 * ((int64_t)blockIdx.x * KT + threadIdx.x); i < n_rows; i += 2 * (int64_t)gridDim.x * KT) {
@@ -354,8 +354,8 @@ static int32_t group_grid(int32_t n) {
 // r -= alpha q; reduces sum r_i^2.
 template <typename TX>
 __global__ void __launch_bounds__(KT)
-    cg_update_kernel(TX *__restrict__ r, const TX *__restrict__ q, const double *__restrict__ scal,
-                     double *__restrict__ partial, int32_t n) {
+    cg_update_kernel(TX *r, const TX *q, const double *scal,
+                     double *partial, int32_t n) {
   begin();
   constexpr int W = G16<TX>::W;
   const TX a = (TX)scal[S_ALPHA];
@@ -386,7 +386,7 @@ __global__ void __launch_bounds__(KT)
 // d += alpha p (here, where p is read anyway), p = r + beta p.
 template <typename TX>
 __global__ void __launch_bounds__(KT)
-    cg_dir_kernel(TX *__restrict__ d, TX *__restrict__ p, const TX *__restrict__ r, const double *__restrict__ scal,
+    cg_dir_kernel(TX *d, TX *p, const TX *r, const double *scal,
                   int32_t n) {
   begin();
   constexpr int W = G16<TX>::W;
@@ -418,8 +418,8 @@ __global__ void __launch_bounds__(KT)
 // reduces sum r_i^2.
 template <typename TL>
 __global__ void __launch_bounds__(KT)
-    ir_start_kernel(const double *__restrict__ r64, TL *__restrict__ r, TL *__restrict__ p, TL *__restrict__ d,
-                    const double *__restrict__ scal, double *__restrict__ partial, int32_t n) {
+    ir_start_kernel(const double *r64, TL *r, TL *p, TL *d,
+                    const double *scal, double *partial, int32_t n) {
   begin();
   const double inv = scal[S_INVNRM];
   Dot<TL> dot;
@@ -437,14 +437,14 @@ __global__ void __launch_bounds__(KT)
 // x += ||r64|| d (fp64)
 template <typename TL>
 __global__ void __launch_bounds__(KT)
-    ir_correct_kernel(double *__restrict__ x, const TL *__restrict__ d, const double *__restrict__ scal, int32_t n) {
+    ir_correct_kernel(double *x, const TL *d, const double *scal, int32_t n) {
   begin();
   const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
   if (i < n) x[i] = fma(scal[S_NRM], (double)d[i], x[i]);
 }
 
 template <typename TX>
-__global__ void __launch_bounds__(KT) sumsq_kernel(const TX *__restrict__ v, double *__restrict__ partial, int32_t n) {
+__global__ void __launch_bounds__(KT) sumsq_kernel(const TX *v, double *partial, int32_t n) {
   begin();
   Dot<TX> dot;
   const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
@@ -455,7 +455,7 @@ __global__ void __launch_bounds__(KT) sumsq_kernel(const TX *__restrict__ v, dou
 // v = v0 / ||v0||
 template <typename TX>
 __global__ void __launch_bounds__(KT)
-    lanczos_start_kernel(const TX *__restrict__ v0, TX *__restrict__ v, const double *__restrict__ scal, int32_t n) {
+    lanczos_start_kernel(const TX *v0, TX *v, const double *scal, int32_t n) {
   begin();
   const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
   if (i < n) v[i] = (TX)((double)v0[i] * scal[S_INVNRM]);
@@ -522,8 +522,8 @@ __device__ __forceinline__ void load_any(const TX *p, TX (&v)[G16<TX>::W]) {
 // vprev: NULL for the first step.
 template <typename TX>
 __global__ void __launch_bounds__(KT)
-    lanczos_orth_kernel(TX *__restrict__ w, const TX *__restrict__ v, const TX *__restrict__ vprev,
-                        const double *__restrict__ scal, double *__restrict__ partial, int32_t j, int32_t n) {
+    lanczos_orth_kernel(TX *w, const TX *v, const TX *vprev,
+                        const double *scal, double *partial, int32_t j, int32_t n) {
   constexpr int W = G16<TX>::W;
   begin();
   const Coef<TX> a(scal + S_LALPHA, scal + SF_ALPHA), b(scal + S_LBETA + (j & 1), scal + SF_BETA + (j & 1));
@@ -560,7 +560,7 @@ __global__ void __launch_bounds__(KT)
 // v = w / beta_{j+1}: the next vector, in its row of the basis if there is one.
 template <typename TX>
 __global__ void __launch_bounds__(KT)
-    lanczos_next_kernel(TX *__restrict__ v, const TX *__restrict__ w, const double *__restrict__ scal, int32_t n) {
+    lanczos_next_kernel(TX *v, const TX *w, const double *scal, int32_t n) {
   constexpr int W = G16<TX>::W;
   begin();
   const Coef<TX> inv(scal + S_INVNRM, scal + SF_INV);
@@ -584,8 +584,8 @@ __global__ void __launch_bounds__(KT)
 // y = sum_j s_j basis[j] (fp64); reduces sum y_i^2
 template <typename TB>
 __global__ void __launch_bounds__(KT)
-    ritz_combine_kernel(const TB *__restrict__ basis, const double *__restrict__ s, int32_t k, int32_t n,
-                        double *__restrict__ y, double *__restrict__ partial) {
+    ritz_combine_kernel(const TB *basis, const double *s, int32_t k, int32_t n,
+                        double *y, double *partial) {
   begin();
   double contrib = 0.0;
   const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
@@ -600,8 +600,8 @@ __global__ void __launch_bounds__(KT)
 
 // reduces sum (w_i - theta y_i)^2 with theta = scal[S_AUX1] / scal[S_AUX0]
 __global__ void __launch_bounds__(KT)
-    ritz_residual_kernel(const double *__restrict__ w, const double *__restrict__ y, const double *__restrict__ scal,
-                         double *__restrict__ partial, int32_t n) {
+    ritz_residual_kernel(const double *w, const double *y, const double *scal,
+                         double *partial, int32_t n) {
   begin();
   const double theta = scal[S_AUX1] / scal[S_AUX0];
   double contrib = 0.0;
@@ -696,8 +696,9 @@ struct Same {
   using type = T;
 };
 
-// Launch with programmatic dependence on the kernel before (see begin()).
-template <typename... P, typename... A>
+// Launch with programmatic dependence on the kernel before (see begin()), or
+// after its end.
+template <bool EARLY = true, typename... P, typename... A>
 static void launch(void (*kernel)(P...), int64_t grid, int threads, cudaStream_t s, A... args) {
   cudaLaunchAttribute at{};
   at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
@@ -707,7 +708,7 @@ static void launch(void (*kernel)(P...), int64_t grid, int threads, cudaStream_t
   c.blockDim = dim3((unsigned)threads);
   c.stream = s;
   c.attrs = &at;
-  c.numAttrs = 1;
+  c.numAttrs = EARLY ? 1 : 0;
   cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
 }
 
@@ -739,7 +740,7 @@ static void launch_dot(const DotKernel<TX, MODE> &d, const pjds_dev *A, const ty
                        typename Same<TX>::type *y, const typename Same<TX>::type *bv, const Reduce &red, cudaStream_t s,
                        int32_t op, int32_t j = 0, double *out = nullptr) {
   const int64_t grid = std::min<int64_t>(((int64_t)A->n_rows + d.rows - 1) / d.rows, d.resident);
-  launch(d.fn, grid, KT, s, A->val, A->col, A->col_start, A->block_len, x, y, bv, red.partial, A->n_rows, A->b);
+  launch<false>(d.fn, grid, KT, s, A->val, A->col, A->col_start, A->block_len, x, y, bv, red.partial, A->n_rows, A->b);
   red.sum(grid, s, op, j, out);
 }
 

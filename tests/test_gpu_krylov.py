@@ -254,3 +254,18 @@ def test_lanczos_scales_with_the_matrix(mods, dtype, power):
     assert np.allclose(a2 * 2.0 ** -power, a1, rtol=tol, atol=tol * np.abs(a1).max())
     assert np.allclose(b2 * 2.0 ** -power, b1, rtol=tol, atol=0)
     assert float((V1.double() - V2.double()).abs().max()) <= tol
+
+
+def test_reduction_of_many_partial_sums_keeps_fp64(mods, oracle_lib):
+    # 17,000 partial sums (1.1M rows, a group of rows per CTA) through the Ritz refinement, whose Rayleigh
+    # quotient the oracle recomputes from the returned vector: y is one basis row, so theta = (v, A v) / (v, v)
+    torch, pjds, krylov = mods
+    A = synth.stencil27(g=103, seed=4)
+    D, perm = _dev(pjds, A, "f64")
+    v = synth.vector(A.n_rows, seed=12)
+    y, theta, _ = krylov.ritz_refine(D, torch.from_numpy(v[perm]).cuda().reshape(1, -1), np.ones(1))
+    assert torch.equal(y, torch.from_numpy(v[perm]).cuda())
+    want = float(np.sum(v.astype(np.longdouble) * oracle_lib.crs_spmv(A, v)) / np.sum(v.astype(np.longdouble) ** 2))
+    # two sums of 1.1M products, each in fp64 within a few ulps of the exact one (they are added in trees),
+    # and the products' own rounding: 2^-53 on average over the rows, far below 1e-14
+    assert theta == pytest.approx(want, rel=1e-14)
