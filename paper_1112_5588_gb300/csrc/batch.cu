@@ -4,6 +4,7 @@
 
 #include <algorithm>
 #include <numeric>
+#include <type_traits>
 #include <vector>
 
 #include "common.h"
@@ -43,6 +44,35 @@ struct V16<double> {
   }
 };
 
+// Whether the rows of a matrix share their columns in fours (sorted rows 4p ..
+// 4p + 3, blocks of four rows or a multiple): 32 sets of four spread over the
+// rows, compared by their first columns (entry 0 of row i is element i), of which
+// 28 have to agree. Read by every CTA of both kernels that a block product on
+// such a matrix launches (spmm_quad_kernel and the one it falls back to), so that
+// one of them does the work: pair_share, which the host has, does not tell blocks
+// of two or six rows from blocks of four.
+__device__ __forceinline__ bool in_fours(const int32_t *__restrict__ col, int32_t n_rows, int32_t n_stored0) {
+  const uint32_t l = threadIdx.x & 31;
+  const int64_t i = (int64_t)(n_rows / 4 - 1) * l / 31 * 4;
+  bool same = false;
+  if (i + 4 <= n_stored0) {
+    const int4 a = __ldg(reinterpret_cast<const int4 *>(col + i));
+    same = a.x == a.y && a.x == a.z && a.x == a.w;
+  }
+  return __popc(__ballot_sync(0xffffffffu, same)) >= 28;
+}
+
+// For the kernel that a block product falls back to (fours = the rows of the
+// first jagged diagonal, 0 when spmm_quad_kernel was not launched): true when
+// spmm_quad_kernel, which this launch overlaps, does the work. The launch's end
+// is that kernel's too.
+__device__ __forceinline__ bool left_to_quads(const int32_t *__restrict__ col, int32_t n_rows, int32_t fours) {
+  if (fours == 0) return false;
+  const bool yes = in_fours(col, n_rows, fours);
+  if (!yes || blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  return yes;
+}
+
 // Thread t: sorted row i = t / lr and, of its k columns, the CH 16-byte chunks
 // [q W, q W + W), W = CH * (elements per chunk), q = t % lr (lr = k / W lanes
 // per row). Wider lanes spread the loads of col_start, col and val and the
@@ -57,9 +87,10 @@ template <typename TV, typename TX, typename IDX, bool SCATTER, int CH, bool PAT
 __global__ void __launch_bounds__(BT)
     spmm_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
                 const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *__restrict__ X,
-                TX *__restrict__ Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr) {
+                TX *__restrict__ Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
   using TA = typename dev::Acc<TV>::T;
   constexpr int VW = V16<TX>::W, W = VW * CH, U = 4;
+  if (left_to_quads(col, n_rows, fours)) return;
   const int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
   const int64_t i = t / lr;
   const int32_t q = (int32_t)(t % lr);
@@ -145,6 +176,15 @@ __device__ __forceinline__ void ld_ones2(const dev::bf16_t *p, dev::bf16_t (&v)[
   v[1].bits = (uint16_t)(a >> 16);
 }
 
+// The ones as R adjacent values.
+template <int R, typename TV>
+__device__ __forceinline__ void ld_ones(const TV *p, TV (&v)[R]) {
+  TV a[2];
+  ld_ones2(p, a);
+#pragma unroll
+  for (int r = 0; r < R; ++r) v[r] = a[r & 1];
+}
+
 // Paired rows: thread t takes sorted rows 2p and 2p + 1 (p = t / lr) and the
 // same CH chunks of their k columns as spmm_kernel. Where the two rows have
 // the same column at a jagged diagonal (block-structured matrices), one
@@ -156,9 +196,10 @@ template <typename TV, typename TX, typename IDX, bool SCATTER, int CH, int U, b
 __global__ void __launch_bounds__(BT)
     spmm_pair_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
                      const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *__restrict__ X,
-                     TX *__restrict__ Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr) {
+                     TX *__restrict__ Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
   using TA = typename dev::Acc<TV>::T;
   constexpr int VW = V16<TX>::W, W = VW * CH;
+  if (left_to_quads(col, n_rows, fours)) return;
   const int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
   const int64_t i = 2 * (t / lr);
   const int32_t q = (int32_t)(t % lr);
@@ -233,6 +274,155 @@ __global__ void __launch_bounds__(BT)
 #pragma unroll
     for (int h = 0; h < CH; ++h)
       V16<TX>::store(Y + row * k + (int64_t)q * W + h * VW, *reinterpret_cast<const TX(*)[VW]>(&out[h * VW]));
+  }
+}
+
+// R adjacent sorted rows i .. i + R - 1 of one block (L entries) and one thread's W = CH chunks of their k
+// columns. Where the R rows have the same column at a jagged diagonal, one gather of the X row serves all of
+// them, else each row gathers its own. A round's columns are loaded during the round before, so that a round
+// is one latency and not two, and of R equal ones one is kept. Each row sums in the order and with the fused
+// multiply-adds of spmm_kernel.
+template <typename TV, typename TX, typename IDX, int R, int CH, int U, bool PAT>
+__device__ __forceinline__ void shared_rows(const TV *__restrict__ val, const int32_t *__restrict__ col,
+                                            const int64_t *__restrict__ col_start, const TX *__restrict__ X,
+                                            int32_t k, int32_t i, int32_t L,
+                                            typename dev::Acc<TV>::T (&acc)[R][V16<TX>::W * CH]) {
+  using TA = typename dev::Acc<TV>::T;
+  constexpr int VW = V16<TX>::W, W = VW * CH;
+  constexpr int32_t NONE = -1, MIXED = -2;
+  auto offset = [&](int32_t j) { return (IDX)__ldg(col_start + j) + (IDX)i; };
+  auto gather = [&](int32_t c, TX (&x)[W]) {
+#pragma unroll
+    for (int h = 0; h < CH; ++h)
+      V16<TX>::load(X + (int64_t)c * k + h * VW, *reinterpret_cast<TX(*)[VW]>(&x[h * VW]));
+  };
+  auto columns = [&](int32_t j, int32_t (&c)[U]) {  // the rows' common columns
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      c[u] = NONE;
+      if (j + u < L && PJDS_IN(j + u, PJDS_EXT(n_diag), dev::CHK_DIAG)) {
+        const IDX o = offset(j + u);
+        if (PJDS_IN(o, PJDS_EXT(stored), dev::CHK_OFFSET) &&
+            PJDS_IN((int64_t)o + (R - 1), PJDS_EXT(stored), dev::CHK_OFFSET)) {
+          int32_t m[R];
+          dev::ld_stream<R>(col + o, m);
+          bool same = true;
+#pragma unroll
+          for (int r = 1; r < R; ++r) same = same && m[r] == m[0];
+          c[u] = same ? m[0] : MIXED;
+        }
+      }
+    }
+  };
+  int32_t next[U];
+  columns(0, next);
+  for (int32_t j = 0; j < L; j += U) {
+    int32_t c[U];
+    TV v[U][R];
+    TX x[U][W];
+#pragma unroll
+    for (int u = 0; u < U; ++u) c[u] = next[u];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (c[u] >= 0 && PJDS_IN(c[u], PJDS_EXT(n_cols), dev::CHK_COLUMN)) {
+        gather(c[u], x[u]);
+      } else {
+#pragma unroll
+        for (int w = 0; w < W; ++w) x[u][w] = TX(0);
+      }
+      if (c[u] != NONE) {
+        const IDX o = offset(j + u);
+        if constexpr (PAT)
+          ld_ones<R>(val + pair_pattern_slot(val + o), v[u]);  // val holds the ones
+        else
+          dev::ld_stream<R>(val + o, v[u]);
+      }
+    }
+    columns(j + U, next);
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      if (c[u] >= 0) {
+#pragma unroll
+        for (int r = 0; r < R; ++r)
+#pragma unroll
+          for (int w = 0; w < W; ++w) acc[r][w] = dev::fma_acc(dev::to_acc(v[u][r]), (TA)x[u][w], acc[r][w]);
+      } else if (c[u] == MIXED) {
+        int32_t m[R];
+        dev::ld_stream<R>(col + offset(j + u), m);
+#pragma unroll
+        for (int r = 0; r < R; ++r) {
+          if (m[r] >= 0 && PJDS_IN(m[r], PJDS_EXT(n_cols), dev::CHK_COLUMN)) {
+            gather(m[r], x[u]);
+#pragma unroll
+            for (int w = 0; w < W; ++w) acc[r][w] = dev::fma_acc(dev::to_acc(v[u][r]), (TA)x[u][w], acc[r][w]);
+          }
+        }
+      }
+    }
+  }
+}
+
+// Four rows per thread, for matrices whose rows share their columns in fours
+// (in_fours; the launch exits otherwise): thread t takes sorted rows 4p .. 4p + 3
+// (p = t / lr) and two chunks of their k columns, together where their first
+// columns agree, else two and two.
+// Bound by the X rows that L2 gives to the SMs (a block row's X rows are read
+// once by the SM that has it: 1.29 GB at k = 32 on 280,000 rows of 144, against
+// 5.2 GB gathered with one row per thread) and their latency. Times on that
+// matrix, before (one row or one pair per thread) and now: fp32 k = 8 / 16 / 32 /
+// 64 / 128 104 / 173 / 330 / 660 / 1260 us, now 95 / 115 / 200 / 326 / 617; bf16
+// values 101 / 150 / 240 / 480 / 912, now 93 / 111 / 195 / 328 / 662.
+// U jagged diagonals a round and MB CTAs per SM: 4 and 2 while the launch has
+// fewer than 2^18 threads (k = 16: 115 us against 146 with 2 and 3), else 2 and 3
+// (k = 64: 326 against 386).
+template <typename TV, typename TX, typename IDX, bool SCATTER, int U, int MB, bool PAT>
+__global__ void __launch_bounds__(BT, MB)
+    spmm_quad_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
+                     const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *__restrict__ X,
+                     TX *__restrict__ Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
+  using TA = typename dev::Acc<TV>::T;
+  constexpr int CH = 2, VW = V16<TX>::W, W = VW * CH;
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  if (!in_fours(col, n_rows, fours)) return;
+  const uint32_t t = blockIdx.x * (uint32_t)BT + threadIdx.x, p = t / (uint32_t)lr, q = t - p * (uint32_t)lr;
+  if (p >= ((uint32_t)n_rows + 3) / 4) return;
+  const int32_t i = 4 * (int32_t)p;
+  const int32_t L = PJDS_IN(i / b, PJDS_EXT(n_blocks), dev::CHK_BLOCK) ? __ldg(block_len + (uint32_t)i / (uint32_t)b) : 0;
+  const TX *__restrict__ Xq = X + q * W;
+  auto store = [&](int32_t row, const TA (&a)[W]) {
+    if (row >= n_rows) return;
+    TX out[W];
+#pragma unroll
+    for (int w = 0; w < W; ++w) out[w] = (TX)a[w];
+    const int64_t y = SCATTER ? (int64_t)__ldcs(perm + row) : row;
+    if (!PJDS_IN(y, PJDS_EXT(n_rows), dev::CHK_ROW)) return;
+#pragma unroll
+    for (int h = 0; h < CH; ++h)
+      V16<TX>::store(Y + y * k + (int64_t)q * W + h * VW, *reinterpret_cast<const TX(*)[VW]>(&out[h * VW]));
+  };
+  int32_t m[4] = {0, 0, 0, 0};
+  if (L > 0 && PJDS_IN((int64_t)i + 3, PJDS_EXT(stored), dev::CHK_OFFSET)) dev::ld_stream<4>(col + i, m);
+  if (m[0] == m[1] && m[0] == m[2] && m[0] == m[3]) {
+    TA acc[4][W];
+#pragma unroll
+    for (int r = 0; r < 4; ++r)
+#pragma unroll
+      for (int w = 0; w < W; ++w) acc[r][w] = TA(0);
+    shared_rows<TV, TX, IDX, 4, CH, U, PAT>(val, col, col_start, Xq, k, i, L, acc);
+#pragma unroll
+    for (int r = 0; r < 4; ++r) store(i + r, acc[r]);
+  } else {
+#pragma unroll 1
+    for (int32_t h = i; h < i + 4; h += 2) {
+      TA acc[2][W];
+#pragma unroll
+      for (int r = 0; r < 2; ++r)
+#pragma unroll
+        for (int w = 0; w < W; ++w) acc[r][w] = TA(0);
+      shared_rows<TV, TX, IDX, 2, CH, U, PAT>(val, col, col_start, Xq, k, h, L, acc);
+#pragma unroll
+      for (int r = 0; r < 2; ++r) store(h + r, acc[r]);
+    }
   }
 }
 
@@ -332,6 +522,32 @@ static int spmm_chunks(const pjds_dev *A, int32_t k, int vw) {
   return lanes >= 2 && (int64_t)A->n_rows * lanes >= (1 << 19) ? 2 : 1;
 }
 
+// Whether to offer the product to spmm_quad_kernel: nearly every paired row
+// shares its columns (blocks of 2, 4, 6, ... rows; the kernel then looks for
+// fours), rows of 16 entries or more on average, k a multiple of 8 and at least
+// 2^20 elements of Y (60,000 rows of 80: k = 8 33 us against 38, not taken, k = 32
+// 62 against 36; 280,000 rows of 40: k = 8 42 against 36), and val and col aligned
+// for 16-byte loads. If the rows turn out not to share in fours, the other kernel
+// runs, 2 us later.
+static bool offer_quads(const pjds_dev *A, int32_t k) {
+  return A->dtype != PJDS_F64 && A->pair_share >= 900 && A->nnz >= 16 * (int64_t)A->n_rows && k % 8 == 0 &&
+         (int64_t)A->n_rows * k >= (1 << 20) && (int64_t)A->n_rows * k < (1ll << 36) && A->n_rows >= 128 &&
+         (((uintptr_t)A->val | (uintptr_t)A->col) & 15) == 0;
+}
+
+template <typename TV, typename TX, typename IDX, bool SC, bool PAT>
+static void launch_quads(const pjds_dev *A, const TV *val, int32_t k, const TX *x, TX *y, int32_t fours, cudaStream_t s) {
+  const int32_t lr = k / 8;
+  const int64_t threads = ((int64_t)A->n_rows + 3) / 4 * lr;
+  const unsigned grid = (unsigned)((threads + BT - 1) / BT);
+  if (threads < (1 << 18))
+    spmm_quad_kernel<TV, TX, IDX, SC, 4, 2, PAT><<<grid, BT, 0, s>>>(val, A->col, A->col_start, A->block_len, A->perm, x,
+                                                                  y, A->n_rows, A->b, k, lr, fours);
+  else
+    spmm_quad_kernel<TV, TX, IDX, SC, 2, 3, PAT><<<grid, BT, 0, s>>>(val, A->col, A->col_start, A->block_len, A->perm, x,
+                                                                  y, A->n_rows, A->b, k, lr, fours);
+}
+
 template <typename TV, typename TX, bool PAT = false>
 static int launch_spmm(const pjds_dev *A, int32_t k, const void *X, void *Y, cudaStream_t s) {
   constexpr int VW = V16<TX>::W;
@@ -362,10 +578,33 @@ static int launch_spmm(const pjds_dev *A, int32_t k, const void *X, void *Y, cud
 #ifdef PJDS_CHECKED
   dev::set_extents(dev::Extents{A->n_stored, A->n_cols, A->n_rows, A->n_blocks, A->n_max + 1}, s);
 #endif
-#define SPMM(IDX, SC, CH)                                                                                        \
-  spmm_kernel<TV, TX, IDX, SC, CH, PAT><<<(unsigned)grid, BT, 0, s>>>(val, A->col, A->col_start, A->block_len,    \
-                                                                       A->perm, \
-                                                                  x, y, A->n_rows, A->b, k, lr)
+  // after spmm_quad_kernel: overlapping it, to take over or to leave at once
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)grid);
+  cfg.blockDim = dim3(BT);
+  cfg.stream = s;
+  int32_t fours = 0;
+  if constexpr (!std::is_same<TX, double>::value) {
+    if (offer_quads(A, k)) {
+      // rows of the first jagged diagonal: all but the empty ones, which follow it
+      fours = A->n_rows / 4 * 4;
+      if (small) {
+        if (sc) launch_quads<TV, TX, int32_t, true, PAT>(A, val, k, x, y, fours, s);
+        else launch_quads<TV, TX, int32_t, false, PAT>(A, val, k, x, y, fours, s);
+      } else {
+        if (sc) launch_quads<TV, TX, int64_t, true, PAT>(A, val, k, x, y, fours, s);
+        else launch_quads<TV, TX, int64_t, false, PAT>(A, val, k, x, y, fours, s);
+      }
+      cfg.attrs = &at;
+      cfg.numAttrs = 1;
+    }
+  }
+#define SPMM(IDX, SC, CH)                                                                                             \
+  cudaLaunchKernelEx(&cfg, spmm_kernel<TV, TX, IDX, SC, CH, PAT>, val, A->col, A->col_start, A->block_len, A->perm, x, \
+                     y, A->n_rows, A->b, k, lr, fours)
 #define SPMM_CH(IDX, SC) \
   do {                   \
     if (ch == 2)         \
@@ -373,10 +612,9 @@ static int launch_spmm(const pjds_dev *A, int32_t k, const void *X, void *Y, cud
     else                 \
       SPMM(IDX, SC, 1);  \
   } while (0)
-#define SPMMP(IDX, SC, CH, UU)                                                                                 \
-  spmm_pair_kernel<TV, TX, IDX, SC, CH, UU, PAT><<<(unsigned)grid, BT, 0, s>>>(val, A->col, A->col_start,        \
-                                                                            A->block_len, A->perm, x, y, A->n_rows, \
-                                                                            A->b, k, lr)
+#define SPMMP(IDX, SC, CH, UU)                                                                                     \
+  cudaLaunchKernelEx(&cfg, spmm_pair_kernel<TV, TX, IDX, SC, CH, UU, PAT>, val, A->col, A->col_start, A->block_len, \
+                     A->perm, x, y, A->n_rows, A->b, k, lr, fours)
 #define SPMMP_CH(IDX, SC)      \
   do {                         \
     if (pair_u == 2)           \

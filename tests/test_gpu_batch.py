@@ -285,3 +285,73 @@ def test_batch_degenerate_matrices(mods, oracle_lib):
                                   np.diff(A.row_ptr))
             assert r["ok"], (kw, r)
         B.destroy()
+
+
+def _block_rows(n_rows, n_brows, bs, nb, mixed, seed):
+    """CRS of n_rows rows in block rows of bs (their columns shared, nb blocks of
+    bs columns each, drawn from n_brows); `mixed` of the rows get a column of
+    their own, and the last rows are shorter."""
+    rng = np.random.default_rng(seed)
+    brow = np.arange(n_rows) // bs
+    first = np.sort(rng.integers(0, n_brows, size=(brow[-1] + 1, nb)), axis=1)
+    first += np.arange(nb)  # distinct: strictly ascending
+    col = (first[brow][:, :, None] * bs + np.arange(bs)).reshape(n_rows, nb * bs)
+    own = np.nonzero(rng.random(n_rows) < mixed)[0]
+    n_cols = (n_brows + nb) * bs + 8
+    col[own, -1] = n_cols - 1 - own % 8
+    lens = np.full(n_rows, nb * bs)
+    lens[-37:] = nb * bs - 3  # a kind of its own in the sorted order, and a remainder
+    keep = np.arange(nb * bs) < lens[:, None]
+    ptr = np.concatenate([[0], np.cumsum(lens)]).astype(np.int64)
+    val = rng.uniform(-1, 1, size=int(ptr[-1]))
+    return synth.Crs(n_rows, n_cols, ptr, col[keep].astype(np.int32), val)
+
+
+# four rows per thread (blocks of 4 and 8 rows, some rows with a column of their
+# own), the fall back from it (blocks of 2 and 6), both depths (2^18 threads
+# between k = 32 and 264 / 64 on 131,077 rows), row counts with every remainder
+# of 4, and just below the size from which it is offered (n k = 2^20)
+@pytest.mark.parametrize("dtype", ["f32", "bf16"])
+@pytest.mark.parametrize("n,k,bs,nb,mixed", [(32768, 32, 4, 5, 0.0), (32769, 32, 4, 5, 0.02), (32767, 32, 4, 5, 0.02),
+                                             (43691, 24, 8, 3, 0.02), (131074, 8, 4, 4, 0.02), (32771, 32, 2, 10, 0.0),
+                                             (34950, 32, 6, 4, 0.01), (131077, 64, 4, 4, 0.02)])
+def test_spmm_rows_sharing_their_columns_in_fours(mods, dtype, n, k, bs, nb, mixed):
+    torch, pjds, batch = mods
+    A = _block_rows(n, n // bs // 2, bs, nb, mixed, seed=n + k)
+    D = pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
+    assert D.pair_share >= 900
+    X = torch.rand(A.n_cols, k, device="cuda", generator=torch.Generator("cuda").manual_seed(n)) * 2 - 1
+    Y = torch.full((A.n_rows, k), float("nan"), device="cuda")
+    P = torch.full((A.n_rows, k), float("nan"), device="cuda")
+    batch.spmm(D, X, Y)
+    batch.spmm_pattern(D, X, P)
+    assert not torch.isnan(Y).any() and not torch.isnan(P).any()
+    # each column in the order and with the multiply-adds of the single product
+    y1, p1 = (torch.empty(A.n_rows, device="cuda") for _ in range(2))
+    for c in (0, 3, 4, 7, k - 1):
+        x = X[:, c].contiguous()
+        pjds.pjds_spmv_cfg(D, x, y1, threads_per_row=1, rows_per_thread=1)
+        pjds.pjds_spmv_pattern(D, x, p1, threads_per_row=1, rows_per_thread=1)
+        assert torch.equal(y1, Y[:, c].contiguous()) and torch.equal(p1, P[:, c].contiguous()), c
+
+
+def test_spmm_in_fours_in_a_captured_graph(mods):
+    # two overlapping launches and what follows them on the stream
+    torch, pjds, batch = mods
+    for bs, nb in ((4, 5), (2, 10)):
+        A = _block_rows(33_000, 8_000, bs, nb, 0.0, seed=bs)
+        D = pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype="f32").to_device("cuda")
+        X = torch.rand(A.n_cols, 32, device="cuda")
+        Y, Z = (torch.zeros(A.n_rows, 32, device="cuda") for _ in range(2))
+        batch.spmm(D, X, Y)
+        want = 2 * Y
+        g = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(g):
+            batch.spmm(D, X, Y)
+            torch.add(Y, Y, out=Z)
+            Y.zero_()
+        for _ in range(3):
+            Z.zero_()
+            g.replay()
+            torch.cuda.synchronize()
+            assert torch.equal(Z, want)
