@@ -7,6 +7,7 @@
 #include <type_traits>
 
 #include "common.h"
+#include "plan.h"
 #include "spmv_kernels.cuh"
 #include "spmv_staged.cuh"
 #include "tiles.cuh"
@@ -127,6 +128,36 @@ int launch_pjds_idx(const pjds_dev *A, const TX *x, TX *y, const LaunchCfg &c, c
   return check_launch("pjds_spmv launch");
 }
 
+// Plans of at most this many tiles (three times the CTAs that are resident at
+// once) run their long rows in a launch of their own: on a small plan one tile's
+// rows set the time, while on a large one all SMs are busy and that launch's fewer
+// warps cost more (fp64, Zipf s = 2, 3M rows, 4,558 tiles: 77 us without, 85
+// with; s = 1.6, 1M rows, 2,599 tiles: 74 and 68).
+constexpr int32_t k_plan_split_max_tiles = 3072;
+
+template <typename TV, typename TX, bool PAT>
+int launch_plan_kernels(const pjds_dev *A, const tiles::Desc &d, cudaStream_t s) {
+  const int4 *plan = reinterpret_cast<const int4 *>(A->plan);
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t cfg{};
+  cfg.gridDim = dim3((unsigned)A->n_plan);
+  cfg.blockDim = dim3(tiles::BT);
+  cfg.stream = s;
+  const int32_t split = A->n_plan <= k_plan_split_max_tiles && A->n_max >= k_plan_rule.min_len[1] ? 1 : 0;
+  if (split) {
+    cudaLaunchKernelEx(&cfg, tiles::pjds_plan_long_kernel<TV, TX, PAT>, d, plan, A->n_pad);
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+  }
+  if constexpr (std::is_same<TV, double>::value)
+    cudaLaunchKernelEx(&cfg, tiles::pjds_plan_kernel_f64<PAT>, d, plan, A->n_pad, split);
+  else
+    cudaLaunchKernelEx(&cfg, tiles::pjds_plan_kernel<TV, TX, PAT>, d, plan, A->n_pad, split);
+  return check_launch("pjds_spmv plan launch");
+}
+
 // Per-tile mapping: one CTA per plan entry (tiles.cuh).
 template <typename TV, typename TX>
 int launch_plan(const pjds_dev *A, const TX *x, TX *y, const LaunchCfg &c, cudaStream_t s) {
@@ -148,21 +179,12 @@ int launch_plan(const pjds_dev *A, const TX *x, TX *y, const LaunchCfg &c, cudaS
   d.n_blocks = A->n_blocks;
   d.n_diag = A->n_max + 1;
   d.reserved = 0;
-  const int4 *plan = reinterpret_cast<const int4 *>(A->plan);
-  if (c.pattern) {  // the pattern kernel reads its values from eight ones
+  if (c.pattern) {  // the pattern kernels read their values from eight ones
     const cudaError_t e = dev::pattern_ones_address<TV>(&d.val);
     if (e != cudaSuccess) return set_error(PJDS_ECUDA, "pattern values: %s", cudaGetErrorString(e));
-    if constexpr (std::is_same<TV, double>::value)
-      tiles::pjds_plan_kernel_f64<true><<<(unsigned)A->n_plan, tiles::BT, 0, s>>>(d, plan, A->n_pad);
-    else
-      tiles::pjds_plan_kernel<TV, TX, true><<<(unsigned)A->n_plan, tiles::BT, 0, s>>>(d, plan, A->n_pad);
-    return check_launch("pjds_spmv_pattern plan launch");
+    return launch_plan_kernels<TV, TX, true>(A, d, s);
   }
-  if constexpr (std::is_same<TV, double>::value)
-    tiles::pjds_plan_kernel_f64<><<<(unsigned)A->n_plan, tiles::BT, 0, s>>>(d, plan, A->n_pad);
-  else
-    tiles::pjds_plan_kernel<TV, TX><<<(unsigned)A->n_plan, tiles::BT, 0, s>>>(d, plan, A->n_pad);
-  return check_launch("pjds_spmv plan launch");
+  return launch_plan_kernels<TV, TX, false>(A, d, s);
 }
 
 template <typename TV, typename TX>

@@ -34,6 +34,19 @@ __device__ __forceinline__ void store_row(const Desc &d, TX *y, int64_t i, TA v)
   if (PJDS_IN(r, d.n_rows, dev::CHK_ROW)) y[r] = (TX)v;
 }
 
+// The same in two halves (EARLY below): the target row is read before the
+// product, whose loads do not depend on it, so that the store does not wait for
+// one more latency. For the plan kernels (Zipf s = 2, 1M rows fp64 34.6 -> 32.9
+// us); the batched launch, which hides it behind other tiles, keeps its registers.
+__device__ __forceinline__ int32_t early_target(const Desc &d, int64_t i) {
+  return d.scatter ? __ldcs(d.perm + i) : (int32_t)i;
+}
+template <typename TX, typename TA>
+__device__ __forceinline__ void store_early(const Desc &d, TX *y, int32_t r, TA v) {
+  asm volatile("" : "+r"(r));  // so that its address, which waits for it, is computed here
+  if (PJDS_IN(r, d.n_rows, dev::CHK_ROW)) y[r] = (TX)v;
+}
+
 // PAT (every routine below): the pattern product; d.val is then the address
 // of eight ones (dev::pattern_ones_address), read at
 // dev::pattern_slot(d.val + o) where the product reads d.val + o.
@@ -124,27 +137,37 @@ __device__ __forceinline__ void desc_rows(const Desc &d, int64_t i, typename dev
 
 // R adjacent rows per thread from the tile's first row; rows past the tile
 // or the matrix are not stored.
-template <typename TV, typename TX, int R, int U, bool PAT = false>
+template <typename TV, typename TX, int R, int U, bool PAT = false, bool EARLY = false>
 __device__ __forceinline__ void rows_tile(const Desc &d, const int4 &tl, TX *y) {
   const int32_t k = R * (int32_t)threadIdx.x;
   const int64_t i = (int64_t)tl.y + k;
   if (k >= tl.z || i >= d.n_rows) return;
   typename dev::Acc<TV>::T acc[R];
+  int32_t to[R];
+  if constexpr (EARLY) {
+#pragma unroll
+    for (int r = 0; r < R; ++r) to[r] = k + r < tl.z && i + r < d.n_rows ? early_target(d, i + r) : -1;
+  }
   if (d.idx64)
     desc_rows<TV, TX, int64_t, R, U, PAT>(d, i, acc);
   else
     desc_rows<TV, TX, int32_t, R, U, PAT>(d, i, acc);
 #pragma unroll
-  for (int r = 0; r < R; ++r)
-    if (k + r < tl.z && i + r < d.n_rows) store_row(d, y, i + r, acc[r]);
+  for (int r = 0; r < R; ++r) {
+    if constexpr (EARLY) {
+      if (to[r] >= 0) store_early(d, y, to[r], acc[r]);
+    } else {
+      if (k + r < tl.z && i + r < d.n_rows) store_row(d, y, i + r, acc[r]);
+    }
+  }
 }
 
 // LANES consecutive lanes share sorted row i: lane s takes jagged diagonals
-// s, s + LANES, ...; the partial sums are added with shuffles (fixed tree).
-template <typename TV, typename TX, typename IDX, int LANES, bool PAT = false>
+// s, s + LANES, ..., U of them a round; the partial sums are added with shuffles
+// (fixed tree).
+template <typename TV, typename TX, typename IDX, int LANES, bool PAT = false, int U = 4>
 __device__ __forceinline__ typename dev::Acc<TV>::T desc_row_lanes(const Desc &d, int64_t i, int32_t s, bool active) {
   using TA = typename dev::Acc<TV>::T;
-  constexpr int U = 4;
   const TV *__restrict__ val = static_cast<const TV *>(d.val);
   const TX *__restrict__ x = static_cast<const TX *>(d.x);
   const int32_t L =
@@ -182,26 +205,32 @@ __device__ __forceinline__ typename dev::Acc<TV>::T desc_row_lanes(const Desc &d
 
 // A tile of BT / LANES rows with LANES lanes each; the whole CTA stays for the
 // shuffles.
-template <typename TV, typename TX, int LANES, bool PAT = false>
+template <typename TV, typename TX, int LANES, bool PAT = false, int U = 4, bool EARLY = false>
 __device__ __forceinline__ void lanes_tile(const Desc &d, const int4 &tl, TX *y) {
   const int32_t r = threadIdx.x / LANES, s = threadIdx.x % LANES;
   const int64_t i = (int64_t)tl.y + r;
   const bool active = r < tl.z && i < d.n_rows;
-  const auto acc = d.idx64 ? desc_row_lanes<TV, TX, int64_t, LANES, PAT>(d, i, s, active)
-                           : desc_row_lanes<TV, TX, int32_t, LANES, PAT>(d, i, s, active);
-  if (active && s == 0) store_row(d, y, i, acc);
+  int32_t to = -1;
+  if constexpr (EARLY) to = active && s == 0 ? early_target(d, i) : -1;
+  const auto acc = d.idx64 ? desc_row_lanes<TV, TX, int64_t, LANES, PAT, U>(d, i, s, active)
+                           : desc_row_lanes<TV, TX, int32_t, LANES, PAT, U>(d, i, s, active);
+  if constexpr (EARLY) {
+    if (to >= 0) store_early(d, y, to, acc);
+  } else {
+    if (active && s == 0) store_row(d, y, i, acc);
+  }
 }
 
 // One plan entry tl = {matrix, first sorted row, rows, kind} of matrix d, by
 // the whole CTA: kind 0 two rows per thread, 3 four rows per thread, 1 one
 // row per thread, 2 / 4 / 8 lanes per row.
-template <typename TV, typename TX, bool PAT = false>
+template <typename TV, typename TX, bool PAT = false, bool EARLY = false>
 __device__ __forceinline__ void run_tile(const Desc &d, const int4 &tl) {
   TX *y = static_cast<TX *>(d.y);
   if (tl.w == 0) {
-    rows_tile<TV, TX, 2, 4, PAT>(d, tl, y);
+    rows_tile<TV, TX, 2, 4, PAT, EARLY>(d, tl, y);
   } else if (tl.w == 3) {  // blocks of at most 2 entries (PlanRule::quad_max_len)
-    rows_tile<TV, TX, 4, 1, PAT>(d, tl, y);
+    rows_tile<TV, TX, 4, 1, PAT, EARLY>(d, tl, y);
   } else if (tl.w == 1) {
     const int64_t i = (int64_t)tl.y + threadIdx.x;
     if ((int32_t)threadIdx.x < tl.z && i < d.n_rows) {
@@ -209,11 +238,11 @@ __device__ __forceinline__ void run_tile(const Desc &d, const int4 &tl) {
       store_row(d, y, i, acc);
     }
   } else if (tl.w == 2) {
-    lanes_tile<TV, TX, 2, PAT>(d, tl, y);
+    lanes_tile<TV, TX, 2, PAT, 4, EARLY>(d, tl, y);
   } else if (tl.w == 4) {
-    lanes_tile<TV, TX, 4, PAT>(d, tl, y);
+    lanes_tile<TV, TX, 4, PAT, 4, EARLY>(d, tl, y);
   } else {
-    lanes_tile<TV, TX, 8, PAT>(d, tl, y);
+    lanes_tile<TV, TX, 8, PAT, 4, EARLY>(d, tl, y);
   }
 }
 
@@ -237,12 +266,21 @@ __device__ __forceinline__ bool plan_entry_ok(const int4 &tl, int32_t n_pad) {
 // ordered by their work per lane, largest first, so the block scheduler
 // starts the long tiles first (on large matrices the short-row entries follow
 // in the original order of their first rows). Any order gives the same
-// results.
-template <typename TV, typename TX, bool PAT = false>
-__global__ void __launch_bounds__(BT) pjds_plan_kernel(const Desc d, const int4 *__restrict__ plan, int32_t n_pad) {
+// results. short_only: the tiles of 4 and 8 lanes per row are
+// pjds_plan_long_kernel's, the launch before, which this one overlaps (and whose
+// end is awaited here, for what follows on the stream).
+template <typename TV, typename TX, bool PAT>
+__device__ __forceinline__ void plan_body(const Desc &d, const int4 *__restrict__ plan, int32_t n_pad,
+                                          int32_t short_only) {
   const int4 tl = plan[blockIdx.x];
-  if (!plan_entry_ok(tl, n_pad)) return;
-  run_tile<TV, TX, PAT>(d, tl);
+  if (plan_entry_ok(tl, n_pad) && !(short_only && tl.w >= 4)) run_tile<TV, TX, PAT, true>(d, tl);
+  if (short_only && blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+}
+
+template <typename TV, typename TX, bool PAT = false>
+__global__ void __launch_bounds__(BT)
+    pjds_plan_kernel(const Desc d, const int4 *__restrict__ plan, int32_t n_pad, int32_t short_only) {
+  plan_body<TV, TX, PAT>(d, plan, n_pad, short_only);
 }
 
 // fp64 values: bounded to six resident CTAs per SM (40 registers; unbounded
@@ -250,10 +288,29 @@ __global__ void __launch_bounds__(BT) pjds_plan_kernel(const Desc d, const int4 
 // stay unbounded (40 and 34 registers).
 template <bool PAT = false>  // a template: instantiated only where it is launched
 __global__ void __launch_bounds__(BT, 6)
-    pjds_plan_kernel_f64(const Desc d, const int4 *__restrict__ plan, int32_t n_pad) {
+    pjds_plan_kernel_f64(const Desc d, const int4 *__restrict__ plan, int32_t n_pad, int32_t short_only) {
+  plan_body<double, double, PAT>(d, plan, n_pad, short_only);
+}
+
+// The plan's tiles of 4 and 8 lanes per row, 16 jagged diagonals a round: a row
+// of 512 entries is 4 rounds of two latencies instead of 16. The registers (72 in
+// fp64) leave two or three CTAs on an SM, so the short rows, whose many tiles need
+// the warps, are not part of it. Zipf s = 2, 1M / 300k / 100k rows fp64 41 / 30 /
+// 22 -> 33 / 23 / 18 us, 1M rows fp32 38 -> 30 us (4 diagonals a round in one
+// launch; 8 in a launch of its own 36 us on 1M rows fp64; a row's entries loaded
+// by four times as many threads and added by shuffles 38 us, as every one of them
+// takes part in the fp64 additions).
+template <typename TV, typename TX, bool PAT = false>
+__global__ void __launch_bounds__(BT, 2)
+    pjds_plan_long_kernel(const Desc d, const int4 *__restrict__ plan, int32_t n_pad) {
+  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
   const int4 tl = plan[blockIdx.x];
-  if (!plan_entry_ok(tl, n_pad)) return;
-  run_tile<double, double, PAT>(d, tl);
+  if (tl.w < 4 || !plan_entry_ok(tl, n_pad)) return;
+  TX *y = static_cast<TX *>(d.y);
+  if (tl.w == 8)
+    lanes_tile<TV, TX, 8, PAT, 16, true>(d, tl, y);
+  else
+    lanes_tile<TV, TX, 4, PAT, 16, true>(d, tl, y);
 }
 
 }  // namespace tiles

@@ -385,3 +385,40 @@ def test_plan_rows_bit_identical_to_uniform_mappings(P, name, make, permute, dty
     spread = H.n_max * A.n_rows > 4 * A.nnz
     big = A.n_rows >= {"f64": 1 << 16, "f32": 1 << 17, "bf16": 1 << 18}[dtype]
     assert P.pjds_spmv_resolve(D)["plan"] == (1 if spread and big else -1)
+
+
+# plans of a launch for the long rows and one for the short ones (up to 3,072
+# tiles and rows of 64 entries), with all kinds of tile, only long rows, only one
+# kind of them, and a plan too large for it: bit for bit the uniform mappings
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("name", ["zipf", "long", "eight", "many"])
+def test_plan_long_and_short_rows(P, name, dtype):
+    import torch
+    rng = np.random.default_rng(11)
+    if name == "many":
+        A = synth.zipf_rows(2_100_000, s=2.0, len_max=512, seed=3)
+    else:
+        lens = {"zipf": np.minimum(rng.zipf(1.7, size=9001), 700),
+                "long": rng.integers(64, 530, size=1237),
+                "eight": np.concatenate([np.full(33, 300), np.full(4000, 1)])}[name]
+        A = tiny.from_lengths(lens, 9001, seed=5)
+    H = P.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype)
+    assert (H.n_plan > 3072) == (name == "many") and H.n_max >= 64
+    D = H.to_device("cuda")
+    x = torch.from_numpy(synth.vector(A.n_cols, seed=2)).to("cuda", D.vec_dtype)
+    y = torch.full((A.n_rows,), float("nan"), dtype=D.vec_dtype, device="cuda")
+    P.pjds_spmv_cfg(D, x, y, plan=1)
+    twice = 2 * y  # (what follows on the stream sees both launches' rows)
+    s = torch.full_like(y, float("nan"))
+    P.pjds_spmv_pattern(D, x, s, plan=1)
+    lanes = np.zeros(H.n_pad, np.int64)
+    for _, row0, rows, kind in H.plan:
+        lanes[row0:row0 + rows] = 1 if kind in (0, 1, 3) else kind
+    by_row = torch.from_numpy(lanes[:A.n_rows][H.inv_perm]).cuda()  # H.inv_perm[original] = sorted
+    for t in (1, 2, 4, 8):
+        u, v = torch.empty_like(y), torch.empty_like(y)
+        P.pjds_spmv_cfg(D, x, u, plan=-1, threads_per_row=t, rows_per_thread=1)
+        P.pjds_spmv_pattern(D, x, v, plan=-1, threads_per_row=t, rows_per_thread=1)
+        at = by_row == t
+        assert torch.equal(y[at], u[at]) and torch.equal(s[at], v[at])
+        assert torch.equal(twice[at], 2 * u[at])
