@@ -187,6 +187,22 @@ __device__ __forceinline__ TX gather(const TX *__restrict__ x, int32_t c) {
   return c >= 0 ? __ldg(x + c) : TX(0);
 }
 
+// Programmatic dependent launch, for kernels of a few microseconds. A kernel that
+// is launched with it may be placed on the SMs when every CTA of the kernel before
+// has called let_next_start() or ended, and waits in after_previous() until that
+// kernel is completed and visible; so its launch is over by then. The kernel
+// before may have written any array that this one reads (the matrix too) while it
+// was already launched: every pointer goes through the wait, so that no load by it,
+// not even one of read-only memory, can be moved ahead, and x is read by ordinary
+// loads.
+__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename... P>
+__device__ __forceinline__ void after_previous(P *&...p) {
+  asm volatile("griddepcontrol.wait;" ::: "memory");
+  const auto hold = [](auto *&q) { asm volatile("" : "+l"(q)::"memory"); };
+  (hold(p), ...);
+}
+
 // ----------------------------------------------------------------------------- checked build
 
 // Built with PJDS_CHECKED (libpjds_checked.so, a test build), the product
@@ -328,21 +344,32 @@ __global__ void __launch_bounds__(512) pjds_rows_kernel(const TV *__restrict__ v
 
 // T consecutive lanes share one sorted row: lane s takes jagged diagonals
 // j = s, s+T, ...; the T partial sums are added with shuffles (fixed tree).
+// Used where the matrix is small against the GPU, so bound by latency: the block
+// length, the first diagonals' offsets (clamped to the last, which exists) and
+// the target row are read at once, and the offsets of a round during the round
+// before. The next launch may start at the end of the rows (a launch that started
+// with this one would be dealt to the SMs unevenly, as their CTAs end: banded, 20k
+// rows fp64, products one after another 8.2 us without, 9.3 with it at the start,
+// 5.8 us at the end; fp32 6.2 / 4.5 / 4.6, 120k HMEp-like rows 10.4 / 10.3 / 8.7).
 template <typename TV, typename TX, typename IDX, int T, int U, bool SCATTER, bool PAT = false>
-__global__ void __launch_bounds__(512) pjds_tpr_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col,
-                                                        const int64_t *__restrict__ col_start,
-                                                        const int32_t *__restrict__ block_len,
-                                                        const int32_t *__restrict__ perm,
-                                                        const int32_t *__restrict__ order, const TX *__restrict__ x,
-                                                        TX *__restrict__ y, int32_t n_rows, int32_t n_pad, int32_t b) {
+__global__ void __launch_bounds__(512) pjds_tpr_kernel(const TV *val, const int32_t *col,
+                                                        const int64_t *col_start, const int32_t *block_len,
+                                                        const int32_t *perm, const int32_t *order, const TX *x, TX *y, int32_t n_rows, int32_t n_pad, int32_t b,
+                                                        int32_t n_max) {
   using TA = typename Acc<TV>::T;
+  after_previous(val, col, col_start, block_len, perm, order, x);
   const int64_t g = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t i = g / T;
   const int32_t s = (int32_t)(g % T);
   bool active = i < n_pad;  // whole warps stay for the shuffles
   if (active && order) active = tile_row(order, n_pad, i);
   if (active) active = PJDS_IN(i / b, PJDS_EXT(n_blocks), CHK_BLOCK);
-  const int32_t L = active ? __ldg(block_len + (int32_t)(i / b)) : 0;
+  IDX start[U];
+#pragma unroll
+  for (int u = 0; u < U; ++u) start[u] = (IDX)__ldg(col_start + min(s + u * T, n_max));
+  const int32_t L = active ? __ldg(block_len + (uint32_t)i / (uint32_t)b) : 0;
+  int32_t to = (int32_t)i;
+  if (SCATTER && s == 0 && active && i < n_rows) to = __ldcs(perm + i);
   TA acc = TA(0);
   for (int32_t j = s; j < L; j += U * T) {
     int32_t c[U];
@@ -352,7 +379,7 @@ __global__ void __launch_bounds__(512) pjds_tpr_kernel(const TV *__restrict__ va
       bool live = j + u * T < L && PJDS_IN(j + u * T, PJDS_EXT(n_diag), CHK_DIAG);
       IDX o = 0;
       if (live) {
-        o = (IDX)__ldg(col_start + j + u * T) + (IDX)i;
+        o = start[u] + (IDX)i;
         live = PJDS_IN(o, PJDS_EXT(stored), CHK_OFFSET);
       }
       if (live) {
@@ -363,32 +390,29 @@ __global__ void __launch_bounds__(512) pjds_tpr_kernel(const TV *__restrict__ va
         v[u] = TV{};
       }
     }
+#pragma unroll
+    for (int u = 0; u < U; ++u) start[u] = (IDX)__ldg(col_start + min(j + (U + u) * T, n_max));
     TX xv[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) xv[u] = gather_n(x, c[u], PJDS_EXT(n_cols));
+    for (int u = 0; u < U; ++u)
+      xv[u] = c[u] >= 0 && PJDS_IN(c[u], PJDS_EXT(n_cols), CHK_COLUMN) ? x[c[u]] : TX(0);
 #pragma unroll
     for (int u = 0; u < U; ++u) acc = c[u] >= 0 ? fma_acc(to_acc(v[u]), (TA)xv[u], acc) : acc;
   }
+  let_next_start();
 #pragma unroll
   for (int off = T / 2; off >= 1; off /= 2) acc += __shfl_down_sync(0xffffffffu, acc, off, T);
-  if (s == 0 && active && i < n_rows) {
-    if constexpr (SCATTER) {
-      const int32_t p = __ldcs(perm + i);
-      if (PJDS_IN(p, PJDS_EXT(n_rows), CHK_ROW)) y[p] = (TX)acc;
-    } else {
-      y[i] = (TX)acc;
-    }
-  }
+  if (s == 0 && active && i < n_rows && PJDS_IN(to, PJDS_EXT(n_rows), CHK_ROW)) y[to] = (TX)acc;
 }
 
 // ----------------------------------------------------------------------------- ELLPACK-R (Listing 1)
 
 // One thread per row in the original order; loop to the row's own length.
 template <typename TV, typename TX, typename IDX, int U>
-__global__ void __launch_bounds__(512) ellr_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col,
-                                                    const int32_t *__restrict__ row_max, const TX *__restrict__ x,
-                                                    TX *__restrict__ y, int32_t n_rows, int32_t n_pad) {
+__global__ void __launch_bounds__(512) ellr_kernel(const TV *val, const int32_t *col, const int32_t *row_max, const TX *x, TX *y,
+                                                    int32_t n_rows, int32_t n_pad) {
   using TA = typename Acc<TV>::T;
+  after_previous(val, col, row_max, x);
   const int64_t i = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   if (i >= n_rows) return;
   const int32_t L = __ldcs(row_max + i);
@@ -409,7 +433,8 @@ __global__ void __launch_bounds__(512) ellr_kernel(const TV *__restrict__ val, c
     }
     TX xv[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) xv[u] = gather_n(x, c[u], PJDS_EXT(n_cols));
+    for (int u = 0; u < U; ++u)
+      xv[u] = c[u] >= 0 && PJDS_IN(c[u], PJDS_EXT(n_cols), CHK_COLUMN) ? x[c[u]] : TX(0);
 #pragma unroll
     for (int u = 0; u < U; ++u) acc = c[u] >= 0 ? fma_acc(to_acc(v[u]), (TA)xv[u], acc) : acc;
   }

@@ -33,6 +33,21 @@ inline int check_launch(const char *what) {
   return PJDS_OK;
 }
 
+// Launch with programmatic dependence on the kernel before (dev::after_previous).
+template <typename... P, typename... A>
+void launch_early(void (*kernel)(P...), unsigned grid, unsigned threads, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(threads);
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 template <typename TV, typename TX, typename IDX, bool SC>
 int launch_staged(const pjds_dev *A, const TX *x, TX *y, cudaStream_t s) {
   const TV *val = static_cast<const TV *>(A->val);
@@ -75,8 +90,10 @@ int launch_pjds_idx(const pjds_dev *A, const TX *x, TX *y, const LaunchCfg &c, c
   const int U = c.unroll;
 #define PJDS_ROWS(RR, UU) dev::pjds_rows_kernel<TV, TX, IDX, RR, UU, SC><<<g, blk, 0, s>>>(PJDS_ARGS)
 #define PJDS_PAT(RR, UU) dev::pjds_rows_kernel<TV, TX, IDX, RR, UU, SC, true><<<g, blk, 0, s>>>(PJDS_ARGS)
-#define PJDS_TPR(TT, UU) dev::pjds_tpr_kernel<TV, TX, IDX, TT, UU, SC><<<g, blk, 0, s>>>(PJDS_ARGS)
-#define PJDS_TPR_PAT(TT, UU) dev::pjds_tpr_kernel<TV, TX, IDX, TT, UU, SC, true><<<g, blk, 0, s>>>(PJDS_ARGS)
+#define PJDS_TPR(TT, UU) \
+  launch_early(dev::pjds_tpr_kernel<TV, TX, IDX, TT, UU, SC>, g.x, blk.x, s, PJDS_ARGS, A->n_max)
+#define PJDS_TPR_PAT(TT, UU) \
+  launch_early(dev::pjds_tpr_kernel<TV, TX, IDX, TT, UU, SC, true>, g.x, blk.x, s, PJDS_ARGS, A->n_max)
   if (c.pattern && T > 1) {
     if (U != 2 && U != 4) return set_error(PJDS_EINVAL, "unroll must be 2 or 4 with threads_per_row > 1");
     switch (T) {
@@ -201,13 +218,16 @@ int launch_pjds(const pjds_dev *A, const void *x, void *y, const LaunchCfg &c, c
                  : launch_pjds_idx<TV, TX, int64_t, false>(A, xx, yy, c, s);
 }
 
-// ELLPACK-R baseline: 4 diagonals per round of the j-loop, 128-thread CTAs
-// (the caller's nt). A GB300 sweep of U in 1, 2, 4, 8 x 128, 256, 512
-// threads put this configuration first or within 1% of the first on the
-// HMEp-like (6.2M rows, fp64), stencil (4.5M rows, fp64 / fp32) and
-// block-dense (280k rows, fp32) matrices, 10% behind U = 8 on the HMEp-like
-// matrix in fp32; U = 8 with 256 threads (52 registers in fp64, half the
-// warps resident) was 11-24% slower in fp64.
+// ELLPACK-R baseline: 128-thread CTAs (the caller's nt), 4 diagonals per round of
+// the j-loop, or 8 while the rows leave the GPU short of loads in flight: up to
+// 2^18 rows in fp64, 2^17 with bf16 values, always in fp32. Measured, 4 / 8 (us):
+// banded 20k rows fp64 8.9 / 7.9, fp32 6.9 / 5.4; HMEp-like 300k rows fp64 23.3 /
+// 21.3, fp32 15.3 / 14.6, bf16 15.0 / 16.9, 1M rows fp32 40.9 / 37.2; 27-point
+// stencil 405k rows fp64 28.9 / 33.0, 1M rows fp64 61.0 / 68.9, fp32 38.1 / 36.4,
+// bf16 37.1 / 43.1, 250k rows bf16 11.0 / 13.1; rows of 144 in dense blocks, 100k
+// fp32 36.0 / 24.6, bf16 41.4 / 33.4, 248k fp64 109 / 93, bf16 50 / 66, 600k fp64
+// 179 / 187. (256-thread CTAs with 8 were 11-24% slower in fp64 on millions of
+// rows.)
 template <typename TV, typename TX>
 int launch_ellr(const ellr_dev *A, const void *x, void *y, int nt, cudaStream_t s) {
   const int64_t grid = ((int64_t)A->n_rows + nt - 1) / nt;
@@ -218,12 +238,11 @@ int launch_ellr(const ellr_dev *A, const void *x, void *y, int nt, cudaStream_t 
 #endif
   const TX *xx = static_cast<const TX *>(x);
   TX *yy = static_cast<TX *>(y);
-  if (A->n_stored < 0x7fffffffLL)
-    dev::ellr_kernel<TV, TX, int32_t, 4>
-        <<<(unsigned)grid, nt, 0, s>>>(val, A->col, A->row_max, xx, yy, A->n_rows, A->n_pad);
-  else
-    dev::ellr_kernel<TV, TX, int64_t, 4>
-        <<<(unsigned)grid, nt, 0, s>>>(val, A->col, A->row_max, xx, yy, A->n_rows, A->n_pad);
+  const bool deep = sizeof(TV) == 4 || A->n_rows <= (sizeof(TV) == 8 ? 1 << 18 : 1 << 17);
+  const bool small = A->n_stored < 0x7fffffffLL;
+  auto *const kernel = small ? (deep ? dev::ellr_kernel<TV, TX, int32_t, 8> : dev::ellr_kernel<TV, TX, int32_t, 4>)
+                             : (deep ? dev::ellr_kernel<TV, TX, int64_t, 8> : dev::ellr_kernel<TV, TX, int64_t, 4>);
+  launch_early(kernel, (unsigned)grid, (unsigned)nt, s, val, A->col, A->row_max, xx, yy, A->n_rows, A->n_pad);
   return check_launch("ellr_spmv launch");
 }
 

@@ -422,3 +422,62 @@ def test_plan_long_and_short_rows(P, name, dtype):
         at = by_row == t
         assert torch.equal(y[at], u[at]) and torch.equal(s[at], v[at])
         assert torch.equal(twice[at], 2 * u[at])
+
+
+# products on the lanes of a row and the ELLPACK-R baseline, launched while the one
+# before runs: each reads what the one before has written (through the matrix
+# values too), one after another on a stream and in a graph, at the edges of a
+# round of 2, 4 or 8 lanes and of 8 diagonals, bit for bit the products one by one
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("lanes", [2, 4, 8, "ellr"])
+def test_products_one_after_another(P, lanes, dtype):
+    import torch
+    n = 6001
+    lens = np.tile([0, 1, 2, 3, 4, 5, 7, 8, 9, 15, 16, 17, 31, 32, 33, 63, 64, 65], n // 18 + 1)[:n]
+    A = tiny.from_lengths(lens, n, seed=7)
+    if lanes == "ellr":
+        D = P.ellr_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, dtype=dtype).to_device("cuda")
+        product = lambda x, y: P.ellr_spmv(D, x, y)
+    else:
+        D = P.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
+        product = lambda x, y: P.pjds_spmv_cfg(D, x, y, plan=-1, threads_per_row=lanes, rows_per_thread=1)
+    values = D.val.view(torch.bfloat16) if dtype == "bf16" else D.val
+    one = torch.from_numpy(synth.vector(n, seed=2)).to("cuda", D.vec_dtype)
+    v = [one] + [torch.full_like(one, float("nan")) for _ in range(6)]
+
+    def row():
+        for i in range(6):
+            product(v[i], v[i + 1])
+            if i == 2:
+                values.mul_(0.5)  # (a power of two: exact)
+        values.mul_(2.0)
+
+    def one_by_one():
+        u = [one]
+        for i in range(6):
+            u.append(torch.full_like(one, float("nan")))
+            torch.cuda.synchronize()
+            product(u[i], u[i + 1])
+            torch.cuda.synchronize()
+            if i == 2:
+                values.mul_(0.5)
+        values.mul_(2.0)
+        return u
+
+    want = one_by_one()
+    assert torch.isfinite(want[6]).all() and want[6].abs().max() > 0
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        row()
+        stream.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(v, want))
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            row()
+    for _ in range(3):
+        for a in v[1:]:
+            a.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(v, want))
