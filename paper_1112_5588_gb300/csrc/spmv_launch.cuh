@@ -88,8 +88,8 @@ int launch_pjds_idx(const pjds_dev *A, const TX *x, TX *y, const LaunchCfg &c, c
 #endif
 #define PJDS_ARGS val, A->col, A->col_start, A->block_len, A->perm, order, x, y, A->n_rows, A->n_pad, A->b
   const int U = c.unroll;
-#define PJDS_ROWS(RR, UU) dev::pjds_rows_kernel<TV, TX, IDX, RR, UU, SC><<<g, blk, 0, s>>>(PJDS_ARGS)
-#define PJDS_PAT(RR, UU) dev::pjds_rows_kernel<TV, TX, IDX, RR, UU, SC, true><<<g, blk, 0, s>>>(PJDS_ARGS)
+#define PJDS_ROWS(RR, UU) launch_early(dev::pjds_rows_kernel<TV, TX, IDX, RR, UU, SC>, g.x, blk.x, s, PJDS_ARGS)
+#define PJDS_PAT(RR, UU) launch_early(dev::pjds_rows_kernel<TV, TX, IDX, RR, UU, SC, true>, g.x, blk.x, s, PJDS_ARGS)
 #define PJDS_TPR(TT, UU) \
   launch_early(dev::pjds_tpr_kernel<TV, TX, IDX, TT, UU, SC>, g.x, blk.x, s, PJDS_ARGS, A->n_max)
 #define PJDS_TPR_PAT(TT, UU) \
@@ -155,23 +155,13 @@ constexpr int32_t k_plan_split_max_tiles = 3072;
 template <typename TV, typename TX, bool PAT>
 int launch_plan_kernels(const pjds_dev *A, const tiles::Desc &d, cudaStream_t s) {
   const int4 *plan = reinterpret_cast<const int4 *>(A->plan);
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)A->n_plan);
-  cfg.blockDim = dim3(tiles::BT);
-  cfg.stream = s;
+  const unsigned grid = (unsigned)A->n_plan;
   const int32_t split = A->n_plan <= k_plan_split_max_tiles && A->n_max >= k_plan_rule.min_len[1] ? 1 : 0;
-  if (split) {
-    cudaLaunchKernelEx(&cfg, tiles::pjds_plan_long_kernel<TV, TX, PAT>, d, plan, A->n_pad);
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
-  }
+  if (split) launch_early(tiles::pjds_plan_long_kernel<TV, TX, PAT>, grid, tiles::BT, s, d, plan, A->n_pad);
   if constexpr (std::is_same<TV, double>::value)
-    cudaLaunchKernelEx(&cfg, tiles::pjds_plan_kernel_f64<PAT>, d, plan, A->n_pad, split);
+    launch_early(tiles::pjds_plan_kernel_f64<PAT>, grid, tiles::BT, s, d, plan, A->n_pad, split);
   else
-    cudaLaunchKernelEx(&cfg, tiles::pjds_plan_kernel<TV, TX, PAT>, d, plan, A->n_pad, split);
+    launch_early(tiles::pjds_plan_kernel<TV, TX, PAT>, grid, tiles::BT, s, d, plan, A->n_pad, split);
   return check_launch("pjds_spmv plan launch");
 }
 

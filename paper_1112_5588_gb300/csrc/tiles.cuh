@@ -47,10 +47,18 @@ __device__ __forceinline__ void store_early(const Desc &d, TX *y, int32_t r, TA 
   if (PJDS_IN(r, d.n_rows, dev::CHK_ROW)) y[r] = (TX)v;
 }
 
+// x's element of column c, or 0 on a pad. The plan kernels (EARLY), launched while
+// the kernel before runs, read x by ordinary loads (index_after_previous).
+template <bool EARLY, typename TX>
+__device__ __forceinline__ TX gather_x(const TX *x, int32_t c, int32_t n_cols) {
+  if constexpr (EARLY) return c >= 0 && PJDS_IN(c, n_cols, dev::CHK_COLUMN) ? x[c] : TX(0);
+  return dev::gather_n(x, c, n_cols);
+}
+
 // PAT (every routine below): the pattern product; d.val is then the address
 // of eight ones (dev::pattern_ones_address), read at
 // dev::pattern_slot(d.val + o) where the product reads d.val + o.
-template <typename TV, typename TX, typename IDX, bool PAT = false>
+template <typename TV, typename TX, typename IDX, bool PAT = false, bool EARLY = false>
 __device__ __forceinline__ typename dev::Acc<TV>::T desc_row(const Desc &d, int64_t i) {
   using TA = typename dev::Acc<TV>::T;
   constexpr int U = 4;
@@ -79,7 +87,7 @@ __device__ __forceinline__ typename dev::Acc<TV>::T desc_row(const Desc &d, int6
     }
     TX xv[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) xv[u] = dev::gather_n(x, c[u], d.n_cols);
+    for (int u = 0; u < U; ++u) xv[u] = gather_x<EARLY>(x, c[u], d.n_cols);
 #pragma unroll
     for (int u = 0; u < U; ++u) acc = c[u] >= 0 ? dev::fma_acc(dev::to_acc(v[u]), (TA)xv[u], acc) : acc;
   }
@@ -89,7 +97,7 @@ __device__ __forceinline__ typename dev::Acc<TV>::T desc_row(const Desc &d, int6
 // R adjacent sorted rows i .. i+R-1 (i a multiple of R: one block) with one
 // vector load of col and of val per jagged diagonal, U diagonals per round;
 // each row's arithmetic as in desc_row.
-template <typename TV, typename TX, typename IDX, int R, int U, bool PAT = false>
+template <typename TV, typename TX, typename IDX, int R, int U, bool PAT = false, bool EARLY = false>
 __device__ __forceinline__ void desc_rows(const Desc &d, int64_t i, typename dev::Acc<TV>::T (&acc)[R]) {
   using TA = typename dev::Acc<TV>::T;
   const TV *__restrict__ val = static_cast<const TV *>(d.val);
@@ -126,7 +134,7 @@ __device__ __forceinline__ void desc_rows(const Desc &d, int64_t i, typename dev
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
-      for (int r = 0; r < R; ++r) xv[u][r] = dev::gather_n(x, c[u][r], d.n_cols);
+      for (int r = 0; r < R; ++r) xv[u][r] = gather_x<EARLY>(x, c[u][r], d.n_cols);
 #pragma unroll
     for (int u = 0; u < U; ++u)
 #pragma unroll
@@ -149,9 +157,9 @@ __device__ __forceinline__ void rows_tile(const Desc &d, const int4 &tl, TX *y) 
     for (int r = 0; r < R; ++r) to[r] = k + r < tl.z && i + r < d.n_rows ? early_target(d, i + r) : -1;
   }
   if (d.idx64)
-    desc_rows<TV, TX, int64_t, R, U, PAT>(d, i, acc);
+    desc_rows<TV, TX, int64_t, R, U, PAT, EARLY>(d, i, acc);
   else
-    desc_rows<TV, TX, int32_t, R, U, PAT>(d, i, acc);
+    desc_rows<TV, TX, int32_t, R, U, PAT, EARLY>(d, i, acc);
 #pragma unroll
   for (int r = 0; r < R; ++r) {
     if constexpr (EARLY) {
@@ -165,7 +173,7 @@ __device__ __forceinline__ void rows_tile(const Desc &d, const int4 &tl, TX *y) 
 // LANES consecutive lanes share sorted row i: lane s takes jagged diagonals
 // s, s + LANES, ..., U of them a round; the partial sums are added with shuffles
 // (fixed tree).
-template <typename TV, typename TX, typename IDX, int LANES, bool PAT = false, int U = 4>
+template <typename TV, typename TX, typename IDX, int LANES, bool PAT = false, int U = 4, bool EARLY = false>
 __device__ __forceinline__ typename dev::Acc<TV>::T desc_row_lanes(const Desc &d, int64_t i, int32_t s, bool active) {
   using TA = typename dev::Acc<TV>::T;
   const TV *__restrict__ val = static_cast<const TV *>(d.val);
@@ -194,7 +202,7 @@ __device__ __forceinline__ typename dev::Acc<TV>::T desc_row_lanes(const Desc &d
     }
     TX xv[U];
 #pragma unroll
-    for (int u = 0; u < U; ++u) xv[u] = dev::gather_n(x, c[u], d.n_cols);
+    for (int u = 0; u < U; ++u) xv[u] = gather_x<EARLY>(x, c[u], d.n_cols);
 #pragma unroll
     for (int u = 0; u < U; ++u) acc = c[u] >= 0 ? dev::fma_acc(dev::to_acc(v[u]), (TA)xv[u], acc) : acc;
   }
@@ -212,8 +220,8 @@ __device__ __forceinline__ void lanes_tile(const Desc &d, const int4 &tl, TX *y)
   const bool active = r < tl.z && i < d.n_rows;
   int32_t to = -1;
   if constexpr (EARLY) to = active && s == 0 ? early_target(d, i) : -1;
-  const auto acc = d.idx64 ? desc_row_lanes<TV, TX, int64_t, LANES, PAT, U>(d, i, s, active)
-                           : desc_row_lanes<TV, TX, int32_t, LANES, PAT, U>(d, i, s, active);
+  const auto acc = d.idx64 ? desc_row_lanes<TV, TX, int64_t, LANES, PAT, U, EARLY>(d, i, s, active)
+                           : desc_row_lanes<TV, TX, int32_t, LANES, PAT, U, EARLY>(d, i, s, active);
   if constexpr (EARLY) {
     if (to >= 0) store_early(d, y, to, acc);
   } else {
@@ -234,7 +242,8 @@ __device__ __forceinline__ void run_tile(const Desc &d, const int4 &tl) {
   } else if (tl.w == 1) {
     const int64_t i = (int64_t)tl.y + threadIdx.x;
     if ((int32_t)threadIdx.x < tl.z && i < d.n_rows) {
-      const auto acc = d.idx64 ? desc_row<TV, TX, int64_t, PAT>(d, i) : desc_row<TV, TX, int32_t, PAT>(d, i);
+      const auto acc = d.idx64 ? desc_row<TV, TX, int64_t, PAT, EARLY>(d, i)
+                                 : desc_row<TV, TX, int32_t, PAT, EARLY>(d, i);
       store_row(d, y, i, acc);
     }
   } else if (tl.w == 2) {
@@ -268,11 +277,14 @@ __device__ __forceinline__ bool plan_entry_ok(const int4 &tl, int32_t n_pad) {
 // in the original order of their first rows). Any order gives the same
 // results. short_only: the tiles of 4 and 8 lanes per row are
 // pjds_plan_long_kernel's, the launch before, which this one overlaps (and whose
-// end is awaited here, for what follows on the stream).
+// end is awaited here, for what follows on the stream; that launch itself waits
+// for the kernels before it and only then lets this one start).
 template <typename TV, typename TX, bool PAT>
 __device__ __forceinline__ void plan_body(const Desc &d, const int4 *__restrict__ plan, int32_t n_pad,
                                           int32_t short_only) {
-  const int4 tl = plan[blockIdx.x];
+  unsigned k = blockIdx.x;
+  if (!short_only) dev::index_after_previous(k);
+  const int4 tl = plan[k];
   if (plan_entry_ok(tl, n_pad) && !(short_only && tl.w >= 4)) run_tile<TV, TX, PAT, true>(d, tl);
   if (short_only && blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
 }
@@ -303,8 +315,10 @@ __global__ void __launch_bounds__(BT, 6)
 template <typename TV, typename TX, bool PAT = false>
 __global__ void __launch_bounds__(BT, 2)
     pjds_plan_long_kernel(const Desc d, const int4 *__restrict__ plan, int32_t n_pad) {
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
-  const int4 tl = plan[blockIdx.x];
+  unsigned k = blockIdx.x;
+  dev::index_after_previous(k);
+  dev::let_next_start();
+  const int4 tl = plan[k];
   if (tl.w < 4 || !plan_entry_ok(tl, n_pad)) return;
   TX *y = static_cast<TX *>(d.y);
   if (tl.w == 8)

@@ -424,12 +424,12 @@ def test_plan_long_and_short_rows(P, name, dtype):
         assert torch.equal(twice[at], 2 * u[at])
 
 
-# products on the lanes of a row and the ELLPACK-R baseline, launched while the one
-# before runs: each reads what the one before has written (through the matrix
+# products of all mappings and of the ELLPACK-R baseline, launched while the one
+# before runs (the plan's: two launches): each reads what the one before has written (through the matrix
 # values too), one after another on a stream and in a graph, at the edges of a
 # round of 2, 4 or 8 lanes and of 8 diagonals, bit for bit the products one by one
 @pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
-@pytest.mark.parametrize("lanes", [2, 4, 8, "ellr"])
+@pytest.mark.parametrize("lanes", [1, 2, 4, 8, "plan", "ellr"])
 def test_products_one_after_another(P, lanes, dtype):
     import torch
     n = 6001
@@ -440,7 +440,8 @@ def test_products_one_after_another(P, lanes, dtype):
         product = lambda x, y: P.ellr_spmv(D, x, y)
     else:
         D = P.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
-        product = lambda x, y: P.pjds_spmv_cfg(D, x, y, plan=-1, threads_per_row=lanes, rows_per_thread=1)
+        cfg = {"plan": 1} if lanes == "plan" else {"plan": -1, "threads_per_row": lanes, "rows_per_thread": 1}
+        product = lambda x, y: P.pjds_spmv_cfg(D, x, y, **cfg)
     values = D.val.view(torch.bfloat16) if dtype == "bf16" else D.val
     one = torch.from_numpy(synth.vector(n, seed=2)).to("cuda", D.vec_dtype)
     v = [one] + [torch.full_like(one, float("nan")) for _ in range(6)]
