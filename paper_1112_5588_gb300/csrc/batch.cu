@@ -18,14 +18,14 @@ namespace bat {
 
 using pjds::tiles::BT;  // threads per CTA
 
-// 16-byte vectors of the vector type
+// 16-byte vectors of the vector type (read by ordinary loads: dev::after_previous)
 template <typename TX>
 struct V16;
 template <>
 struct V16<float> {
   static constexpr int W = 4;
   __device__ static void load(const float *p, float (&v)[4]) {
-    const float4 a = __ldg(reinterpret_cast<const float4 *>(p));
+    const float4 a = *reinterpret_cast<const float4 *>(p);
     v[0] = a.x, v[1] = a.y, v[2] = a.z, v[3] = a.w;
   }
   __device__ static void store(float *p, const float (&v)[4]) {
@@ -36,7 +36,7 @@ template <>
 struct V16<double> {
   static constexpr int W = 2;
   __device__ static void load(const double *p, double (&v)[2]) {
-    const double2 a = __ldg(reinterpret_cast<const double2 *>(p));
+    const double2 a = *reinterpret_cast<const double2 *>(p);
     v[0] = a.x, v[1] = a.y;
   }
   __device__ static void store(double *p, const double (&v)[2]) {
@@ -62,12 +62,16 @@ __device__ __forceinline__ bool in_fours(const int32_t *__restrict__ col, int32_
   return __popc(__ballot_sync(0xffffffffu, same)) >= 28;
 }
 
-// For the kernel that a block product falls back to (fours = the rows of the
-// first jagged diagonal, 0 when spmm_quad_kernel was not launched): true when
-// spmm_quad_kernel, which this launch overlaps, does the work. The launch's end
-// is that kernel's too.
-__device__ __forceinline__ bool left_to_quads(const int32_t *__restrict__ col, int32_t n_rows, int32_t fours) {
-  if (fours == 0) return false;
+// Start of spmm_kernel and spmm_pair_kernel for thread t. Without spmm_quad_kernel
+// before it (fours = 0) the launch overlaps the end of whatever is before it, and
+// waits for it. Else (fours = the rows of the first jagged diagonal) it overlaps
+// spmm_quad_kernel, which has waited: true when that one does the work. The
+// launch's end is that kernel's too.
+__device__ __forceinline__ bool left_to_quads(const int32_t *__restrict__ col, int32_t n_rows, int32_t fours, int64_t &t) {
+  if (fours == 0) {
+    dev::index_after_previous(t);
+    return false;
+  }
   const bool yes = in_fours(col, n_rows, fours);
   if (!yes || blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   return yes;
@@ -86,12 +90,12 @@ __device__ __forceinline__ bool left_to_quads(const int32_t *__restrict__ col, i
 template <typename TV, typename TX, typename IDX, bool SCATTER, int CH, bool PAT = false>
 __global__ void __launch_bounds__(BT)
     spmm_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
-                const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *__restrict__ X,
-                TX *__restrict__ Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
+                const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X,
+                TX *Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
   using TA = typename dev::Acc<TV>::T;
   constexpr int VW = V16<TX>::W, W = VW * CH, U = 4;
-  if (left_to_quads(col, n_rows, fours)) return;
-  const int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
+  int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
+  if (left_to_quads(col, n_rows, fours, t)) return;
   const int64_t i = t / lr;
   const int32_t q = (int32_t)(t % lr);
   if (i >= n_rows) return;
@@ -195,12 +199,12 @@ __device__ __forceinline__ void ld_ones(const TV *p, TV (&v)[R]) {
 template <typename TV, typename TX, typename IDX, bool SCATTER, int CH, int U, bool PAT = false>
 __global__ void __launch_bounds__(BT)
     spmm_pair_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
-                     const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *__restrict__ X,
-                     TX *__restrict__ Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
+                     const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X,
+                     TX *Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
   using TA = typename dev::Acc<TV>::T;
   constexpr int VW = V16<TX>::W, W = VW * CH;
-  if (left_to_quads(col, n_rows, fours)) return;
-  const int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
+  int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
+  if (left_to_quads(col, n_rows, fours, t)) return;
   const int64_t i = 2 * (t / lr);
   const int32_t q = (int32_t)(t % lr);
   if (i >= n_rows) return;
@@ -284,7 +288,7 @@ __global__ void __launch_bounds__(BT)
 // multiply-adds of spmm_kernel.
 template <typename TV, typename TX, typename IDX, int R, int CH, int U, bool PAT>
 __device__ __forceinline__ void shared_rows(const TV *__restrict__ val, const int32_t *__restrict__ col,
-                                            const int64_t *__restrict__ col_start, const TX *__restrict__ X,
+                                            const int64_t *__restrict__ col_start, const TX *X,
                                             int32_t k, int32_t i, int32_t L,
                                             typename dev::Acc<TV>::T (&acc)[R][V16<TX>::W * CH]) {
   using TA = typename dev::Acc<TV>::T;
@@ -378,17 +382,18 @@ __device__ __forceinline__ void shared_rows(const TV *__restrict__ val, const in
 template <typename TV, typename TX, typename IDX, bool SCATTER, int U, int MB, bool PAT>
 __global__ void __launch_bounds__(BT, MB)
     spmm_quad_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
-                     const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *__restrict__ X,
-                     TX *__restrict__ Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
+                     const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X,
+                     TX *Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
   using TA = typename dev::Acc<TV>::T;
   constexpr int CH = 2, VW = V16<TX>::W, W = VW * CH;
-  asm volatile("griddepcontrol.launch_dependents;" ::: "memory");
+  dev::index_after_previous(fours);
+  dev::let_next_start();
   if (!in_fours(col, n_rows, fours)) return;
   const uint32_t t = blockIdx.x * (uint32_t)BT + threadIdx.x, p = t / (uint32_t)lr, q = t - p * (uint32_t)lr;
   if (p >= ((uint32_t)n_rows + 3) / 4) return;
   const int32_t i = 4 * (int32_t)p;
   const int32_t L = PJDS_IN(i / b, PJDS_EXT(n_blocks), dev::CHK_BLOCK) ? __ldg(block_len + (uint32_t)i / (uint32_t)b) : 0;
-  const TX *__restrict__ Xq = X + q * W;
+  const TX *Xq = X + q * W;
   auto store = [&](int32_t row, const TA (&a)[W]) {
     if (row >= n_rows) return;
     TX out[W];
@@ -541,11 +546,11 @@ static void launch_quads(const pjds_dev *A, const TV *val, int32_t k, const TX *
   const int64_t threads = ((int64_t)A->n_rows + 3) / 4 * lr;
   const unsigned grid = (unsigned)((threads + BT - 1) / BT);
   if (threads < (1 << 18))
-    spmm_quad_kernel<TV, TX, IDX, SC, 4, 2, PAT><<<grid, BT, 0, s>>>(val, A->col, A->col_start, A->block_len, A->perm, x,
-                                                                  y, A->n_rows, A->b, k, lr, fours);
+    dev::launch_early(spmm_quad_kernel<TV, TX, IDX, SC, 4, 2, PAT>, grid, BT, s, val, A->col, A->col_start, A->block_len,
+                 A->perm, x, y, A->n_rows, A->b, k, lr, fours);
   else
-    spmm_quad_kernel<TV, TX, IDX, SC, 2, 3, PAT><<<grid, BT, 0, s>>>(val, A->col, A->col_start, A->block_len, A->perm, x,
-                                                                  y, A->n_rows, A->b, k, lr, fours);
+    dev::launch_early(spmm_quad_kernel<TV, TX, IDX, SC, 2, 3, PAT>, grid, BT, s, val, A->col, A->col_start, A->block_len,
+                 A->perm, x, y, A->n_rows, A->b, k, lr, fours);
 }
 
 template <typename TV, typename TX, bool PAT = false>
@@ -578,14 +583,6 @@ static int launch_spmm(const pjds_dev *A, int32_t k, const void *X, void *Y, cud
 #ifdef PJDS_CHECKED
   dev::set_extents(dev::Extents{A->n_stored, A->n_cols, A->n_rows, A->n_blocks, A->n_max + 1}, s);
 #endif
-  // after spmm_quad_kernel: overlapping it, to take over or to leave at once
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t cfg{};
-  cfg.gridDim = dim3((unsigned)grid);
-  cfg.blockDim = dim3(BT);
-  cfg.stream = s;
   int32_t fours = 0;
   if constexpr (!std::is_same<TX, double>::value) {
     if (offer_quads(A, k)) {
@@ -598,13 +595,11 @@ static int launch_spmm(const pjds_dev *A, int32_t k, const void *X, void *Y, cud
         if (sc) launch_quads<TV, TX, int64_t, true, PAT>(A, val, k, x, y, fours, s);
         else launch_quads<TV, TX, int64_t, false, PAT>(A, val, k, x, y, fours, s);
       }
-      cfg.attrs = &at;
-      cfg.numAttrs = 1;
     }
   }
 #define SPMM(IDX, SC, CH)                                                                                             \
-  cudaLaunchKernelEx(&cfg, spmm_kernel<TV, TX, IDX, SC, CH, PAT>, val, A->col, A->col_start, A->block_len, A->perm, x, \
-                     y, A->n_rows, A->b, k, lr, fours)
+  dev::launch_early(spmm_kernel<TV, TX, IDX, SC, CH, PAT>, (unsigned)grid, BT, s, val, A->col, A->col_start, A->block_len, \
+               A->perm, x, y, A->n_rows, A->b, k, lr, fours)
 #define SPMM_CH(IDX, SC) \
   do {                   \
     if (ch == 2)         \
@@ -613,8 +608,8 @@ static int launch_spmm(const pjds_dev *A, int32_t k, const void *X, void *Y, cud
       SPMM(IDX, SC, 1);  \
   } while (0)
 #define SPMMP(IDX, SC, CH, UU)                                                                                     \
-  cudaLaunchKernelEx(&cfg, spmm_pair_kernel<TV, TX, IDX, SC, CH, UU, PAT>, val, A->col, A->col_start, A->block_len, \
-                     A->perm, x, y, A->n_rows, A->b, k, lr, fours)
+  dev::launch_early(spmm_pair_kernel<TV, TX, IDX, SC, CH, UU, PAT>, (unsigned)grid, BT, s, val, A->col, A->col_start,   \
+               A->block_len, A->perm, x, y, A->n_rows, A->b, k, lr, fours)
 #define SPMMP_CH(IDX, SC)      \
   do {                         \
     if (pair_u == 2)           \

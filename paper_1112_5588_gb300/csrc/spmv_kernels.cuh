@@ -215,6 +215,22 @@ __device__ __forceinline__ void index_after_previous(I &i) {
     asm volatile("" : "+r"(i)::"memory");
 }
 
+// Launch with programmatic dependence on the kernel before (after_previous,
+// index_after_previous).
+template <typename... P, typename... A>
+void launch_early(void (*kernel)(P...), unsigned grid, unsigned threads, cudaStream_t s, A... args) {
+  cudaLaunchAttribute at{};
+  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+  at.val.programmaticStreamSerializationAllowed = 1;
+  cudaLaunchConfig_t c{};
+  c.gridDim = dim3(grid);
+  c.blockDim = dim3(threads);
+  c.stream = s;
+  c.attrs = &at;
+  c.numAttrs = 1;
+  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
+}
+
 // ----------------------------------------------------------------------------- checked build
 
 // Built with PJDS_CHECKED (libpjds_checked.so, a test build), the product

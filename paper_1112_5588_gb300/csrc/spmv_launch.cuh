@@ -33,21 +33,6 @@ inline int check_launch(const char *what) {
   return PJDS_OK;
 }
 
-// Launch with programmatic dependence on the kernel before (dev::after_previous).
-template <typename... P, typename... A>
-void launch_early(void (*kernel)(P...), unsigned grid, unsigned threads, cudaStream_t s, A... args) {
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t c{};
-  c.gridDim = dim3(grid);
-  c.blockDim = dim3(threads);
-  c.stream = s;
-  c.attrs = &at;
-  c.numAttrs = 1;
-  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
-}
-
 template <typename TV, typename TX, typename IDX, bool SC>
 int launch_staged(const pjds_dev *A, const TX *x, TX *y, cudaStream_t s) {
   const TV *val = static_cast<const TV *>(A->val);
@@ -88,12 +73,12 @@ int launch_pjds_idx(const pjds_dev *A, const TX *x, TX *y, const LaunchCfg &c, c
 #endif
 #define PJDS_ARGS val, A->col, A->col_start, A->block_len, A->perm, order, x, y, A->n_rows, A->n_pad, A->b
   const int U = c.unroll;
-#define PJDS_ROWS(RR, UU) launch_early(dev::pjds_rows_kernel<TV, TX, IDX, RR, UU, SC>, g.x, blk.x, s, PJDS_ARGS)
-#define PJDS_PAT(RR, UU) launch_early(dev::pjds_rows_kernel<TV, TX, IDX, RR, UU, SC, true>, g.x, blk.x, s, PJDS_ARGS)
+#define PJDS_ROWS(RR, UU) dev::launch_early(dev::pjds_rows_kernel<TV, TX, IDX, RR, UU, SC>, g.x, blk.x, s, PJDS_ARGS)
+#define PJDS_PAT(RR, UU) dev::launch_early(dev::pjds_rows_kernel<TV, TX, IDX, RR, UU, SC, true>, g.x, blk.x, s, PJDS_ARGS)
 #define PJDS_TPR(TT, UU) \
-  launch_early(dev::pjds_tpr_kernel<TV, TX, IDX, TT, UU, SC>, g.x, blk.x, s, PJDS_ARGS, A->n_max)
+  dev::launch_early(dev::pjds_tpr_kernel<TV, TX, IDX, TT, UU, SC>, g.x, blk.x, s, PJDS_ARGS, A->n_max)
 #define PJDS_TPR_PAT(TT, UU) \
-  launch_early(dev::pjds_tpr_kernel<TV, TX, IDX, TT, UU, SC, true>, g.x, blk.x, s, PJDS_ARGS, A->n_max)
+  dev::launch_early(dev::pjds_tpr_kernel<TV, TX, IDX, TT, UU, SC, true>, g.x, blk.x, s, PJDS_ARGS, A->n_max)
   if (c.pattern && T > 1) {
     if (U != 2 && U != 4) return set_error(PJDS_EINVAL, "unroll must be 2 or 4 with threads_per_row > 1");
     switch (T) {
@@ -157,11 +142,11 @@ int launch_plan_kernels(const pjds_dev *A, const tiles::Desc &d, cudaStream_t s)
   const int4 *plan = reinterpret_cast<const int4 *>(A->plan);
   const unsigned grid = (unsigned)A->n_plan;
   const int32_t split = A->n_plan <= k_plan_split_max_tiles && A->n_max >= k_plan_rule.min_len[1] ? 1 : 0;
-  if (split) launch_early(tiles::pjds_plan_long_kernel<TV, TX, PAT>, grid, tiles::BT, s, d, plan, A->n_pad);
+  if (split) dev::launch_early(tiles::pjds_plan_long_kernel<TV, TX, PAT>, grid, tiles::BT, s, d, plan, A->n_pad);
   if constexpr (std::is_same<TV, double>::value)
-    launch_early(tiles::pjds_plan_kernel_f64<PAT>, grid, tiles::BT, s, d, plan, A->n_pad, split);
+    dev::launch_early(tiles::pjds_plan_kernel_f64<PAT>, grid, tiles::BT, s, d, plan, A->n_pad, split);
   else
-    launch_early(tiles::pjds_plan_kernel<TV, TX, PAT>, grid, tiles::BT, s, d, plan, A->n_pad, split);
+    dev::launch_early(tiles::pjds_plan_kernel<TV, TX, PAT>, grid, tiles::BT, s, d, plan, A->n_pad, split);
   return check_launch("pjds_spmv plan launch");
 }
 
@@ -232,7 +217,7 @@ int launch_ellr(const ellr_dev *A, const void *x, void *y, int nt, cudaStream_t 
   const bool small = A->n_stored < 0x7fffffffLL;
   auto *const kernel = small ? (deep ? dev::ellr_kernel<TV, TX, int32_t, 8> : dev::ellr_kernel<TV, TX, int32_t, 4>)
                              : (deep ? dev::ellr_kernel<TV, TX, int64_t, 8> : dev::ellr_kernel<TV, TX, int64_t, 4>);
-  launch_early(kernel, (unsigned)grid, (unsigned)nt, s, val, A->col, A->row_max, xx, yy, A->n_rows, A->n_pad);
+  dev::launch_early(kernel, (unsigned)grid, (unsigned)nt, s, val, A->col, A->row_max, xx, yy, A->n_rows, A->n_pad);
   return check_launch("ellr_spmv launch");
 }
 

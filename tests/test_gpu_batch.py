@@ -355,3 +355,40 @@ def test_spmm_in_fours_in_a_captured_graph(mods):
             g.replay()
             torch.cuda.synchronize()
             assert torch.equal(Z, want)
+
+
+# block products launched while the one before runs, each on what that one has
+# written (one row, pairs, fours and the fall back from fours), in a row on a
+# stream and in a graph: bit for bit the products one by one
+@pytest.mark.parametrize("dtype,k,bs,nb", [("f64", 2, 4, 5), ("f32", 4, 2, 8), ("bf16", 8, 2, 8), ("f32", 32, 4, 5),
+                                           ("f32", 32, 2, 10), ("bf16", 32, 6, 4)])
+def test_spmm_one_after_another(mods, dtype, k, bs, nb):
+    torch, pjds, batch = mods
+    A = _block_rows(33_001, 33_001 // bs // 2, bs, nb, 0.01, seed=bs)
+    D = pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
+    one = torch.rand(A.n_rows, k, device="cuda", generator=torch.Generator("cuda").manual_seed(k)).to(D.vec_dtype) - 0.5
+    v = [one] + [torch.full_like(one, float("nan")) for _ in range(5)]
+    want = [one]
+    for _ in range(5):
+        want.append(torch.full_like(one, float("nan")))
+        torch.cuda.synchronize()
+        batch.spmm(D, want[-2][:A.n_cols], want[-1])
+        torch.cuda.synchronize()
+    assert torch.isfinite(want[-1]).all()
+    stream = torch.cuda.Stream()
+    stream.wait_stream(torch.cuda.current_stream())
+    with torch.cuda.stream(stream):
+        for i in range(5):
+            batch.spmm(D, v[i][:A.n_cols], v[i + 1])
+        stream.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(v, want))
+        graph = torch.cuda.CUDAGraph()
+        with torch.cuda.graph(graph, stream=stream):
+            for i in range(5):
+                batch.spmm(D, v[i][:A.n_cols], v[i + 1])
+    for _ in range(3):
+        for a in v[1:]:
+            a.fill_(float("nan"))
+        graph.replay()
+        torch.cuda.synchronize()
+        assert all(torch.equal(a, b) for a, b in zip(v, want))
