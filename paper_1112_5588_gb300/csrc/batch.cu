@@ -62,18 +62,26 @@ __device__ __forceinline__ bool in_fours(const int32_t *__restrict__ col, int32_
   return __popc(__ballot_sync(0xffffffffu, same)) >= 28;
 }
 
-// Start of spmm_kernel and spmm_pair_kernel for thread t. Without spmm_quad_kernel
-// before it (fours = 0) the launch overlaps the end of whatever is before it, and
-// waits for it. Else (fours = the rows of the first jagged diagonal) it overlaps
-// spmm_quad_kernel, which has waited: true when that one does the work. The
-// launch's end is that kernel's too.
+constexpr int LONG_BT = 64;           // threads of spmm_long_kernel's CTAs
+constexpr int LONG_U = 16;            // its jagged diagonals a round
+constexpr int32_t k_long_len = 64;    // and the shortest rows it takes
+// Lanes up to which it is launched (every lane a 16-byte chunk of a long row; on
+// more, the GPU is full without it): Zipf 400k rows s = 2 fp64 k = 64, 830,000 lanes
+// 342 us without, 314 with; s = 1.6 fp32 k = 128, 2.5 million lanes 319 and 448.
+constexpr int64_t k_long_max_lanes = 1 << 20;
+
+// Start of spmm_kernel and spmm_pair_kernel for thread t. Alone (fours = 0) the
+// launch overlaps the end of whatever is before it, and waits for it. Else it
+// overlaps the launch before that belongs to the same product and has waited, and
+// its end is that one's too: spmm_quad_kernel (fours = the rows of the first jagged
+// diagonal; true when that one does the work) or spmm_long_kernel (fours < 0).
 __device__ __forceinline__ bool left_to_quads(const int32_t *__restrict__ col, int32_t n_rows, int32_t fours, int64_t &t) {
   if (fours == 0) {
     dev::index_after_previous(t);
     return false;
   }
-  const bool yes = in_fours(col, n_rows, fours);
-  if (!yes || blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  const bool yes = fours > 0 && in_fours(col, n_rows, fours);
+  if ((fours > 0 && !yes) || blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
   return yes;
 }
 
@@ -100,6 +108,7 @@ __global__ void __launch_bounds__(BT)
   const int32_t q = (int32_t)(t % lr);
   if (i >= n_rows) return;
   const int32_t L = PJDS_IN(i / b, PJDS_EXT(n_blocks), dev::CHK_BLOCK) ? __ldg(block_len + (int32_t)(i / b)) : 0;
+  if (fours < 0 && L >= -fours) return;  // spmm_long_kernel's
   TA acc[W];
 #pragma unroll
   for (int w = 0; w < W; ++w) acc[w] = TA(0);
@@ -431,6 +440,86 @@ __global__ void __launch_bounds__(BT, MB)
   }
 }
 
+// The rows of min_len entries or more of a matrix with widely spread lengths (the
+// first sorted rows), one chunk of the k columns per lane. Bound by latency: a long
+// row is one serial sum, in the order of spmm_kernel, on a GPU that the few long
+// rows leave idle. U jagged diagonals a round; their columns and values are loaded
+// one round ahead and their offsets two, so that a round is one latency (and in
+// fp64 the sum's additions) instead of three. Zipf, against the rows in spmm_kernel:
+// 100k rows s = 2 fp64 k = 8 176 -> 88 us, 400k rows fp32 k = 4 176 -> 71, s = 1.6
+// fp64 k = 4 289 -> 106, 20k rows bf16 k = 32 132 -> 39, 3k rows fp64 k = 2 110 ->
+// 69 (8 diagonals a round 133, 127, 156, 71, 84; rows from 32 or 128 entries on
+// within 5%).
+template <typename TV, typename TX, typename IDX, bool SCATTER, int U, bool PAT>
+__global__ void __launch_bounds__(LONG_BT)
+    spmm_long_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
+                     const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X, TX *Y,
+                     int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t min_len) {
+  using TA = typename dev::Acc<TV>::T;
+  constexpr int W = V16<TX>::W;
+  int64_t t = (int64_t)blockIdx.x * LONG_BT + threadIdx.x;
+  dev::index_after_previous(t);
+  dev::let_next_start();
+  const int64_t i = t / lr;
+  const int32_t q = (int32_t)(t % lr);
+  if (i >= n_rows) return;
+  const int32_t L = PJDS_IN(i / b, PJDS_EXT(n_blocks), dev::CHK_BLOCK) ? __ldg(block_len + (int32_t)(i / b)) : 0;
+  if (L < min_len) return;
+  const int64_t r = SCATTER ? (int64_t)__ldcs(perm + i) : i;
+  const TX *Xq = X + (int64_t)q * W;
+  IDX start[U];  // of the round after the next one's columns and values
+  int32_t next[U];
+  TV next_v[U];
+  auto starts = [&](int32_t j) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) start[u] = (IDX)__ldg(col_start + min(j + u, L));  // (entry L exists)
+  };
+  auto entries = [&](int32_t j) {
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      const IDX o = start[u] + (IDX)i;
+      const bool live = j + u < L && PJDS_IN(j + u, PJDS_EXT(n_diag), dev::CHK_DIAG) &&
+                        PJDS_IN(o, PJDS_EXT(stored), dev::CHK_OFFSET);
+      next[u] = live ? __ldcs(col + o) : -1;
+      next_v[u] = live ? dev::ld_stream1(PAT ? val + dev::pattern_slot(val + o) : val + o) : TV{};
+    }
+  };
+  TA acc[W];
+#pragma unroll
+  for (int w = 0; w < W; ++w) acc[w] = TA(0);
+  starts(0);
+  entries(0);
+  starts(U);
+  for (int32_t j = 0; j < L; j += U) {
+    int32_t c[U];
+    TV v[U];
+    TX x[U][W];
+#pragma unroll
+    for (int u = 0; u < U; ++u) {
+      c[u] = next[u];
+      v[u] = next_v[u];
+      if (c[u] >= 0 && PJDS_IN(c[u], PJDS_EXT(n_cols), dev::CHK_COLUMN)) {
+        V16<TX>::load(Xq + (int64_t)c[u] * k, x[u]);
+      } else {
+#pragma unroll
+        for (int w = 0; w < W; ++w) x[u][w] = TX(0);
+      }
+    }
+    entries(j + U);
+    starts(j + 2 * U);
+#pragma unroll
+    for (int u = 0; u < U; ++u)
+#pragma unroll
+      for (int w = 0; w < W; ++w)
+        acc[w] = c[u] >= 0 ? dev::fma_acc(dev::to_acc(v[u]), (TA)x[u][w], acc[w]) : acc[w];
+  }
+  if (!PJDS_IN(r, PJDS_EXT(n_rows), dev::CHK_ROW)) return;
+  TX out[W];
+#pragma unroll
+  for (int w = 0; w < W; ++w) out[w] = (TX)acc[w];
+  V16<TX>::store(Y + r * k + (int64_t)q * W, out);
+}
+
 // ----------------------------------------------------------------------------- persistent batch
 
 using namespace pjds::tiles;
@@ -597,6 +686,25 @@ static int launch_spmm(const pjds_dev *A, int32_t k, const void *X, void *Y, cud
       }
     }
   }
+#define SPMML(IDX, SC)                                                                                              \
+  dev::launch_early(spmm_long_kernel<TV, TX, IDX, SC, LONG_U, PAT>, (unsigned)long_grid, LONG_BT, s, val, A->col, A->col_start, \
+                    A->block_len, A->perm, x, y, A->n_rows, A->b, k, lr, k_long_len)
+  if (!pair_u && fours == 0 && ch == 1 && A->n_max >= k_long_len && (int64_t)A->n_max * A->n_rows > 4 * A->nnz) {
+    // a row in a block of that length takes that many stored entries
+    const int64_t most = std::min<int64_t>(A->n_rows, A->n_stored / k_long_len);
+    const int64_t long_grid = (most * lr + LONG_BT - 1) / LONG_BT;
+    if (most > 0 && most * lr <= k_long_max_lanes) {
+      fours = -k_long_len;
+      if (small) {
+        if (sc) SPMML(int32_t, true);
+        else SPMML(int32_t, false);
+      } else {
+        if (sc) SPMML(int64_t, true);
+        else SPMML(int64_t, false);
+      }
+    }
+  }
+#undef SPMML
 #define SPMM(IDX, SC, CH)                                                                                             \
   dev::launch_early(spmm_kernel<TV, TX, IDX, SC, CH, PAT>, (unsigned)grid, BT, s, val, A->col, A->col_start, A->block_len, \
                A->perm, x, y, A->n_rows, A->b, k, lr, fours)

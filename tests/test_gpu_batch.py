@@ -392,3 +392,32 @@ def test_spmm_one_after_another(mods, dtype, k, bs, nb):
         graph.replay()
         torch.cuda.synchronize()
         assert all(torch.equal(a, b) for a, b in zip(v, want))
+
+
+# long rows in a launch of their own (widely spread lengths, rows of 64 entries or
+# more): lengths at the edges of its rounds of 16, only long rows and a few, one
+# long row, and past the lanes up to which it is launched; each column in the order
+# and with the multiply-adds of the single product
+@pytest.mark.parametrize("dtype,k", [("f64", 2), ("f64", 6), ("f32", 4), ("bf16", 24), ("f32", 128)])
+@pytest.mark.parametrize("name", ["edges", "one", "many"])
+def test_spmm_long_rows(mods, dtype, k, name):
+    torch, pjds, batch = mods
+    lens = {"edges": [64, 65, 79, 80, 81, 63, 95, 96, 97, 111, 112, 113, 128, 700] + [3] * 4001,
+            "one": [64] + [1] * 900,
+            "many": list(np.minimum(np.random.default_rng(3).zipf(1.5, size=9000), 600))}[name]
+    A = tiny.from_lengths(np.array(lens), 9001, seed=k)
+    rng = np.random.default_rng(5)
+    D = pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
+    assert D.n_max * A.n_rows > 4 * A.nnz
+    X = torch.from_numpy(rng.uniform(-1, 1, size=(A.n_cols, k))).to("cuda", D.vec_dtype)
+    Y, P = (torch.full((A.n_rows, k), float("nan"), dtype=D.vec_dtype, device="cuda") for _ in range(2))
+    batch.spmm(D, X, Y)
+    twice = 2 * Y  # (what follows on the stream sees both launches' rows)
+    batch.spmm_pattern(D, X, P)
+    y1, p1 = (torch.empty(A.n_rows, dtype=D.vec_dtype, device="cuda") for _ in range(2))
+    for c in (0, 1, k - 1):
+        x = X[:, c].contiguous()
+        pjds.pjds_spmv_cfg(D, x, y1, plan=-1, threads_per_row=1, rows_per_thread=1)
+        pjds.pjds_spmv_pattern(D, x, p1, plan=-1, threads_per_row=1, rows_per_thread=1)
+        assert torch.equal(y1, Y[:, c].contiguous()) and torch.equal(p1, P[:, c].contiguous()), c
+        assert torch.equal(2 * y1, twice[:, c].contiguous()), c
