@@ -567,6 +567,23 @@ __global__ void __launch_bounds__(BT, 6)
   batch_body<double, double, PAT>(descs, tiles, n_tiles, counter, ones);
 }
 
+// The same with tile blockIdx.x: for batches whose tiles are all resident at once
+// (pjds_batch::n_ctas = n_tiles), where nothing is left to distribute and the
+// counter, its reset and its graph are most of the time. 8 bf16 matrices of 3k to 13k
+// rows 17.3 -> 13.0 us, 5 fp32 ones of 1.5k to 4k 12.9 -> 7.7, 20 fp64 ones of 8k to
+// 20k 33.3 -> 29.3. (Larger batches: the same launch mode and a counter that the last
+// CTA resets made the fp32 kernel 5% slower, 179 -> 188 us, and fp64 no faster.)
+template <typename TV, typename TX, bool PAT = false>
+__global__ void __launch_bounds__(BT)
+    batch_once_kernel(const Desc *__restrict__ descs, const int4 *__restrict__ tiles, const void *ones) {
+  unsigned k = blockIdx.x;
+  dev::index_after_previous(k);
+  const int4 tl = tiles[k];
+  Desc d = descs[tl.x];
+  if constexpr (PAT) d.val = ones;
+  run_tile<TV, TX, PAT, true>(d, tl);
+}
+
 static inline size_t a256(size_t b) { return (b + 255) & ~(size_t)255; }
 
 }  // namespace bat
@@ -948,7 +965,8 @@ extern "C" int pjds_batch_create_rule(int32_t n_mats, const pjds_dev *mats, cons
 
 template <bool PAT = false>
 static int batch_issue(pjds_batch *h, cudaStream_t s) {
-  cudaError_t e = cudaMemsetAsync(h->counter, 0, sizeof(int32_t), s);
+  const bool once = h->n_ctas == h->n_tiles;
+  cudaError_t e = once ? cudaSuccess : cudaMemsetAsync(h->counter, 0, sizeof(int32_t), s);
   if (e != cudaSuccess) return set_error(PJDS_ECUDA, "reset counter: %s", cudaGetErrorString(e));
   const void *ones = nullptr;
   if constexpr (PAT) {
@@ -957,7 +975,14 @@ static int batch_issue(pjds_batch *h, cudaStream_t s) {
                                : dev::pattern_ones_address<dev::bf16_t>(&ones);
     if (e != cudaSuccess) return set_error(PJDS_ECUDA, "pattern values: %s", cudaGetErrorString(e));
   }
-  if (h->dtype == PJDS_F64)
+  const unsigned grid = (unsigned)h->n_ctas;
+  if (once && h->dtype == PJDS_F64)
+    dev::launch_early(batch_once_kernel<double, double, PAT>, grid, BT, s, h->descs, h->tiles, ones);
+  else if (once && h->dtype == PJDS_F32)
+    dev::launch_early(batch_once_kernel<float, float, PAT>, grid, BT, s, h->descs, h->tiles, ones);
+  else if (once)
+    dev::launch_early(batch_once_kernel<dev::bf16_t, float, PAT>, grid, BT, s, h->descs, h->tiles, ones);
+  else if (h->dtype == PJDS_F64)
     batch_kernel_f64<PAT><<<h->n_ctas, BT, 0, s>>>(h->descs, h->tiles, h->n_tiles, h->counter, ones);
   else if (h->dtype == PJDS_F32)
     batch_kernel<float, float, PAT><<<h->n_ctas, BT, 0, s>>>(h->descs, h->tiles, h->n_tiles, h->counter, ones);
@@ -973,7 +998,7 @@ extern "C" int pjds_batch_run(pjds_batch *h, int32_t use_graph, void *stream) {
   if (!h) return set_error(PJDS_EINVAL, "h is NULL");
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   if (h->n_tiles == 0) return PJDS_OK;
-  if (!use_graph) return batch_issue(h, s);
+  if (!use_graph || h->n_ctas == h->n_tiles) return batch_issue(h, s);  // (one launch needs no graph)
   if (!h->exec) {
     cudaStream_t cap = nullptr;
     cudaGraph_t g = nullptr;

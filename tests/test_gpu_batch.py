@@ -421,3 +421,41 @@ def test_spmm_long_rows(mods, dtype, k, name):
         pjds.pjds_spmv_pattern(D, x, p1, plan=-1, threads_per_row=1, rows_per_thread=1)
         assert torch.equal(y1, Y[:, c].contiguous()) and torch.equal(p1, P[:, c].contiguous()), c
         assert torch.equal(2 * y1, twice[:, c].contiguous()), c
+
+
+# batches of which every tile has its CTA: run after run, each reading what the one
+# before wrote (x and y change places), with and without use_graph and in a captured
+# graph, bit for bit the single products of the same plan
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+def test_small_batches_one_after_another(mods, dtype):
+    torch, pjds, batch = mods
+    mats = [synth.zipf_rows(n, s=2.0, len_max=300, seed=n) for n in (33, 1000, 2047)]
+    devs = [pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
+            for A in mats]
+    a = [torch.from_numpy(synth.vector(A.n_cols, seed=2)).to("cuda", D.vec_dtype) for A, D in zip(mats, devs)]
+    b = [torch.empty_like(v) for v in a]
+    there, back = batch.Batch(devs, a, b), batch.Batch(devs, b, a)
+    assert there.info()["n_ctas"] == there.info()["n_tiles"]
+    first, want = [v.clone() for v in a], [v.clone() for v in a]
+    for _ in range(6):
+        for q, D in enumerate(devs):
+            y = torch.empty_like(want[q])
+            torch.cuda.synchronize()
+            pjds.pjds_spmv_cfg(D, want[q], y, plan=1)
+            torch.cuda.synchronize()
+            want[q] = y
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        for k in range(6):
+            (back if k % 2 else there).run()
+
+    def runs(use_graph):
+        for k in range(6):
+            (back if k % 2 else there).run(use_graph=use_graph)
+
+    for go in (lambda: runs(True), lambda: runs(False), graph.replay, graph.replay):
+        for v, u in zip(a, first):
+            v.copy_(u)
+        go()
+        torch.cuda.synchronize()
+        assert all(torch.equal(v, w) for v, w in zip(a, want))
