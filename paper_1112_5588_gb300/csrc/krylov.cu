@@ -1157,9 +1157,7 @@ extern "C" int pjds_cg_solve_static(const pjds_dev *A_hi, const pjds_dev *A_lo, 
     if (o.inner_iters <= 0) o.inner_iters = 50;
   }
   if (o.inner_iters > 100000 || o.max_outer > 100000) return set_error(PJDS_EINVAL, "iteration counts too large");
-  // The inner steps are always launched one by one on the caller's stream:
-  // recording them into a CUDA graph would create a stream and an executable
-  // graph, driver objects this entry point promises not to create.
+  // No stream, graph or other driver object is created, as this entry point promises.
   o.use_graph = 0;
   const bool low = A_lo->dtype != PJDS_F64;
   const size_t need = cg_bytes(A_hi->n_rows, low ? 4 : 8);

@@ -7,7 +7,8 @@
 //     L1 and L2 (ld.global.cs) so they do not push x out of the caches;
 //   - a warp reads one jagged diagonal as one contiguous run (Listing 2
 //     addressing col_start[j] + i), with optional 2- or 4-row vector loads;
-//   - the gather x[col] goes through the read-only L1 path (ld.global.nc);
+//   - the gather x[col] is cached in L1 (ordinary loads: the kernel before may
+//     have written x while this one was already launched);
 //   - the j-loop is unrolled so each thread issues U independent val/col
 //     loads, then U gathers, before the dependent fused multiply-adds;
 //   - the accumulator stays in a register and y is written once (scattered
@@ -181,7 +182,8 @@ __device__ __forceinline__ bool tile_row(const int32_t *__restrict__ order, int3
   return true;
 }
 
-// Gather through the read-only L1 path; pads (c < 0) read nothing.
+// Gather through the read-only L1 path (kernels launched normally); pads (c < 0) read
+// nothing.
 template <typename TX>
 __device__ __forceinline__ TX gather(const TX *__restrict__ x, int32_t c) {
   return c >= 0 ? __ldg(x + c) : TX(0);
