@@ -68,7 +68,7 @@ struct Dot<float> {
       const float e = __fmaf_rn(a, b, -p), t = __fadd_rn(s, p), z = __fsub_rn(t, s);
       c = __fadd_rn(c, __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z))));
       s = t;
-    } else if (a != 0.0f && b != 0.0f) {
+    } else if (p != 0.0f || (a != 0.0f && b != 0.0f)) {  // (also a NaN: 0 times an infinity)
       far = far_product(a, b, far);
     }
   }

@@ -269,3 +269,35 @@ def test_reduction_of_many_partial_sums_keeps_fp64(mods, oracle_lib):
     # two sums of 1.1M products, each in fp64 within a few ulps of the exact one (they are added in trees),
     # and the products' own rounding: 2^-53 on average over the rows, far below 1e-14
     assert theta == pytest.approx(want, rel=1e-14)
+
+
+# a NaN or an infinity of a matrix row reaches the inner product that this row is part of, also where the other
+# factor is zero (0 * inf is NaN), in every value type and on one CTA's rows as on many
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("bad", [np.nan, np.inf, -np.inf])
+@pytest.mark.parametrize("n", [5, 4097])
+def test_lanczos_keeps_a_nan_beside_a_zero(mods, dtype, bad, n):
+    torch, pjds, krylov = mods
+    A = _spd("tri", n)
+    row = 3
+    val = A.val.copy()
+    val[A.row_ptr[row]] = bad  # its coupling with row 2
+    D, perm = _dev(pjds, A._replace(val=val), dtype)
+    v0 = np.ones(n)
+    v0[row] = 0.0
+    alpha, beta, _ = krylov.lanczos(D, torch.from_numpy(v0[perm]).to("cuda", D.vec_dtype), 1)
+    assert np.isnan(alpha[0]) and np.isnan(beta[1])
+
+
+# a NaN in the start vector reaches every coefficient, and every element of the next vector
+@pytest.mark.parametrize("dtype", ["f64", "f32"])
+def test_lanczos_from_a_nan(mods, dtype):
+    torch, pjds, krylov = mods
+    A = _spd("tri", 1029)
+    D, perm = _dev(pjds, A, dtype)
+    v0 = torch.ones(A.n_rows, dtype=D.vec_dtype, device="cuda")
+    v0[::2] = 0.0
+    v0[77] = float("nan")
+    alpha, beta, V = krylov.lanczos(D, v0, 2, keep_basis=True)
+    assert np.isnan(alpha).all() and np.isnan(beta[1:]).all()
+    assert bool(torch.isnan(V[1]).all())
