@@ -344,7 +344,9 @@ struct Work {
   GridSlots *slots;
 };
 
-static size_t carve(void *w, int32_t n, int32_t batch, Work *k) {
+// train: with what only a training run uses (its steps' constants and the slots of
+// its grid-wide waits); prediction takes any training workspace of as many samples.
+static size_t carve(void *w, int32_t n, int32_t batch, bool train, Work *k) {
   char *const base = static_cast<char *>(w);
   size_t at = 0;
   auto take = [&](size_t bytes) {
@@ -361,14 +363,15 @@ static size_t carve(void *w, int32_t n, int32_t batch, Work *k) {
   k->Y = reinterpret_cast<float *>(take(sizeof(float) * (size_t)n));
   k->out = reinterpret_cast<float *>(take(sizeof(float) * (size_t)n));
   k->idx = reinterpret_cast<int32_t *>(take(sizeof(int32_t) * (size_t)n));
+  if (!train) return at;
   k->c = reinterpret_cast<float2 *>(take(sizeof(float2) * (size_t)steps));
   k->slots = reinterpret_cast<GridSlots *>(take(sizeof(GridSlots)));
   return at;
 }
 
-static size_t work_bytes(int32_t n, int32_t batch) {
+static size_t work_bytes(int32_t n, int32_t batch, bool train) {
   Work k;
-  return carve(nullptr, n, batch, &k);
+  return carve(nullptr, n, batch, train, &k);
 }
 
 static void pack(const pjds_mlp &m, float *P) {
@@ -492,7 +495,7 @@ extern "C" int pjds_mlp_fit_scaling(pjds_mlp *m, const float *X, const float *y,
 extern "C" int pjds_mlp_workspace_bytes(int32_t n, int32_t batch, size_t *bytes) {
   clear_error();
   if (n <= 0 || batch <= 0 || !bytes) return set_error(PJDS_EINVAL, "bad arguments");
-  *bytes = work_bytes(n, batch);
+  *bytes = work_bytes(n, batch, true);
   return PJDS_OK;
 }
 
@@ -501,7 +504,7 @@ extern "C" int pjds_mlp_train(pjds_mlp *m, const float *X, const float *y, int32
   clear_error();
   if (!m || !X || !y || !work || n <= 0 || epochs < 0 || batch <= 0 || !(lr > 0.0f))
     return set_error(PJDS_EINVAL, "bad arguments");
-  if (wbytes < work_bytes(n, batch)) return set_error(PJDS_EINVAL, "workspace too small");
+  if (wbytes < work_bytes(n, batch, true)) return set_error(PJDS_EINVAL, "workspace too small");
   int rc = set_smem_limits();
   if (rc) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
@@ -509,7 +512,7 @@ extern "C" int pjds_mlp_train(pjds_mlp *m, const float *X, const float *y, int32
   if ((rc = sm_count(&sms))) return rc;
   const int32_t bsz = std::min(batch, n);
   Work w;
-  carve(work, n, batch, &w);
+  carve(work, n, batch, true, &w);
   std::vector<float> P(NP);
   pack(*m, P.data());
   cudaError_t e = upload(*m, X, y, n, w, s);
@@ -583,12 +586,12 @@ extern "C" int pjds_mlp_predict(const pjds_mlp *m, const float *X, int32_t n, fl
                                 void *stream) {
   clear_error();
   if (!m || !X || !out || !work || n <= 0) return set_error(PJDS_EINVAL, "bad arguments");
-  if (wbytes < work_bytes(n, 1)) return set_error(PJDS_EINVAL, "workspace too small");
+  if (wbytes < work_bytes(n, 1, false)) return set_error(PJDS_EINVAL, "workspace too small");
   int rc = set_smem_limits();
   if (rc) return rc;
   cudaStream_t s = static_cast<cudaStream_t>(stream);
   Work w;
-  carve(work, n, 1, &w);
+  carve(work, n, 1, false, &w);
   std::vector<float> P(NP);
   pack(*m, P.data());
   cudaError_t e = upload(*m, X, nullptr, n, w, s);

@@ -116,3 +116,23 @@ def test_training_in_batches_matches_oracle(L, n, batch, epochs):
         q = _to_oracle(m)
         for k in p:
             assert np.mean(np.abs(q[k] - p[k])) <= 2e-5, k
+
+
+# the size that pjds_mlp_workspace_bytes gives for any batch serves pjds_mlp_predict on as many inputs, and no
+# byte beyond it is written
+@pytest.mark.parametrize("n,batch", [(1, 1), (17, 1), (100, 1000), (21600, 16), (21600, 21600), (200_000, 1024)])
+def test_predict_in_a_training_workspace(L, n, batch):
+    import ctypes
+
+    import torch
+    m = L.init(5)
+    X, _ = _data(n, 8)
+    need = ctypes.c_size_t()
+    assert L._lib.pjds_mlp_workspace_bytes(n, batch, ctypes.byref(need)) == 0
+    work = torch.full((need.value + 4096,), 0x5A, dtype=torch.uint8, device="cuda")
+    out = np.full(n, np.nan, np.float32)
+    rc = L._lib.pjds_mlp_predict(ctypes.byref(m), X.ctypes.data, n, out.ctypes.data, work.data_ptr(), need.value,
+                                 torch.cuda.current_stream().cuda_stream)
+    assert rc == 0, L._p._lib.pjds_last_error()
+    assert bool((work[need.value:] == 0x5A).all())
+    assert np.array_equal(out, L.predict(m, X))
