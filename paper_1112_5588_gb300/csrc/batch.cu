@@ -472,7 +472,10 @@ __global__ void __launch_bounds__(LONG_BT)
   TV next_v[U];
   auto starts = [&](int32_t j) {
 #pragma unroll
-    for (int u = 0; u < U; ++u) start[u] = (IDX)__ldg(col_start + min(j + u, L));  // (entry L exists)
+    for (int u = 0; u < U; ++u) {
+      const int32_t at = min(j + u, L);  // (entry L of a matrix exists)
+      start[u] = PJDS_IN(at, PJDS_EXT(n_diag), dev::CHK_DIAG) ? (IDX)__ldg(col_start + at) : (IDX)0;
+    }
   };
   auto entries = [&](int32_t j) {
 #pragma unroll

@@ -10,8 +10,9 @@ match the oracle (fp64; fp32 bounds for the paired block product).
 
 Planted: an index put out of range in a device copy of a matrix (a column
 beyond n_cols, a perm entry beyond n_rows, a jagged-diagonal offset beyond
-the stored entries, a block longer than the longest row) must be recorded
-with its code and skipped: the kernels check each index before the access.
+the stored entries, a block longer than the longest row; also in the block
+product's launch for long rows) must be recorded with its code and skipped:
+the kernels check each index before the access.
 
 Prints one JSON line.
 """
@@ -211,6 +212,19 @@ def main():
     batch.spmm(D, torch.rand(A.n_cols, 4, dtype=torch.float64, device="cuda"), Y)
     torch.cuda.synchronize()
     res["planted"]["spmm_column"] = [[{}, *split(pjds.pjds_check_word(clear=True))]]
+    # SpMM's launch for long rows (widely spread lengths): a column beyond n_cols, a block longer than the longest row
+    Z = mats["zipf"]
+    Hz = pjds.pjds_create(Z.n_rows, Z.n_cols, Z.row_ptr, Z.col, Z.val, b=32)
+    assert Hz.n_max >= 64 and Hz.n_max * Z.n_rows > 4 * Z.nnz
+    res["zipf"] = {"n_cols": Z.n_cols, "n_stored": Hz.n_stored, "n_max": Hz.n_max}
+    for name, mutate in (("long_column", lambda D: D.col.__setitem__(0, Z.n_cols + 13)),
+                         ("long_block", lambda D: D.block_len.__setitem__(0, Hz.n_max + 3))):
+        D = Hz.to_device("cuda")
+        mutate(D)
+        Y = torch.empty(Z.n_rows, 4, dtype=torch.float64, device="cuda")
+        batch.spmm(D, torch.rand(Z.n_cols, 4, dtype=torch.float64, device="cuda"), Y)
+        torch.cuda.synchronize()
+        res["planted"][name] = [[{}, *split(pjds.pjds_check_word(clear=True))]]
     print(json.dumps(res))
 
 

@@ -67,3 +67,11 @@ def test_paired_block_product_column_is_recorded(res):
     for cfg, code, idx in res["planted"]["paired_column"]:
         assert (code, idx) == (COLUMN, res["paired_n_cols"] + 11), (cfg, code, idx)
     assert any(c[0] == "paired" for c in res["clean"])
+
+
+def test_long_rows_of_a_block_product_are_checked(res):
+    n = res["zipf"]
+    for cfg, code, idx in res["planted"]["long_column"]:
+        assert (code, idx) == (COLUMN, n["n_cols"] + 13), (code, idx)
+    for cfg, code, idx in res["planted"]["long_block"]:
+        assert (code == DIAG and idx >= n["n_max"] + 1) or (code == OFFSET and idx >= n["n_stored"]), (code, idx)
