@@ -135,8 +135,7 @@ typedef struct pjds_host {
  * its first sorted row), so that the short rows in flight lie close together
  * in the original numbering. A row gives the same bits as with the same lanes per row in
  * the uniform mappings (one thread per row for kinds 0 and 3). The plan
- * kernel runs one CTA per entry (up to 3,072 entries and rows of 64 or more: two
- * overlapping launches, the kinds 4 and 8 first); it needs plan, val and col 16-byte aligned
+ * kernel runs one CTA per entry; it needs plan, val and col 16-byte aligned
  * and skips an entry that does not describe a tile of the matrix.
  * val must be 16-byte aligned; all other pointers 4-byte aligned.
  */

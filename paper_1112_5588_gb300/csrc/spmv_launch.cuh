@@ -130,23 +130,24 @@ int launch_pjds_idx(const pjds_dev *A, const TX *x, TX *y, const LaunchCfg &c, c
   return check_launch("pjds_spmv launch");
 }
 
-// Plans of at most this many tiles (three times the CTAs that are resident at
-// once) run their long rows in a launch of their own: on a small plan one tile's
-// rows set the time, while on a large one all SMs are busy and that launch's fewer
-// warps cost more (fp64, Zipf s = 2, 3M rows, 4,558 tiles: 77 us without, 85
-// with; s = 1.6, 1M rows, 2,599 tiles: 74 and 68).
-constexpr int32_t k_plan_split_max_tiles = 3072;
+// Plans of at most this many tiles with rows of 4 or 8 lanes run more diagonals a
+// round: on a small plan one tile's rows set the time, while on a large one all
+// SMs are busy and fewer warps cost more (Zipf, 4 diagonals a round / 16: fp64 s =
+// 2, 2.2M rows, 3,341 tiles 55.8 / 55.7 us, 3M rows, 4,554 tiles 72.5 / 74.1, s =
+// 1.6, 1.5M rows, 3,901 tiles 98.1 / 99.1; bf16 s = 2, 2.2M rows 48.9 / 51.3; below
+// the line tiles.cuh).
+constexpr int32_t k_plan_deep_max_tiles = 3072;
 
 template <typename TV, typename TX, bool PAT>
-int launch_plan_kernels(const pjds_dev *A, const tiles::Desc &d, cudaStream_t s) {
+int launch_plan_kernel(const pjds_dev *A, const tiles::Desc &d, cudaStream_t s) {
   const int4 *plan = reinterpret_cast<const int4 *>(A->plan);
   const unsigned grid = (unsigned)A->n_plan;
-  const int32_t split = A->n_plan <= k_plan_split_max_tiles && A->n_max >= k_plan_rule.min_len[1] ? 1 : 0;
-  if (split) dev::launch_early(tiles::pjds_plan_long_kernel<TV, TX, PAT>, grid, tiles::BT, s, d, plan, A->n_pad);
-  if constexpr (std::is_same<TV, double>::value)
-    dev::launch_early(tiles::pjds_plan_kernel_f64<PAT>, grid, tiles::BT, s, d, plan, A->n_pad, split);
+  if (A->n_plan <= k_plan_deep_max_tiles && A->n_max >= k_plan_rule.min_len[1])
+    dev::launch_early(tiles::pjds_plan_deep_kernel<TV, TX, PAT>, grid, tiles::BT, s, d, plan, A->n_pad);
+  else if constexpr (std::is_same<TV, double>::value)
+    dev::launch_early(tiles::pjds_plan_kernel_f64<PAT>, grid, tiles::BT, s, d, plan, A->n_pad);
   else
-    dev::launch_early(tiles::pjds_plan_kernel<TV, TX, PAT>, grid, tiles::BT, s, d, plan, A->n_pad, split);
+    dev::launch_early(tiles::pjds_plan_kernel<TV, TX, PAT>, grid, tiles::BT, s, d, plan, A->n_pad);
   return check_launch("pjds_spmv plan launch");
 }
 
@@ -174,9 +175,9 @@ int launch_plan(const pjds_dev *A, const TX *x, TX *y, const LaunchCfg &c, cudaS
   if (c.pattern) {  // the pattern kernels read their values from eight ones
     const cudaError_t e = dev::pattern_ones_address<TV>(&d.val);
     if (e != cudaSuccess) return set_error(PJDS_ECUDA, "pattern values: %s", cudaGetErrorString(e));
-    return launch_plan_kernels<TV, TX, true>(A, d, s);
+    return launch_plan_kernel<TV, TX, true>(A, d, s);
   }
-  return launch_plan_kernels<TV, TX, false>(A, d, s);
+  return launch_plan_kernel<TV, TX, false>(A, d, s);
 }
 
 template <typename TV, typename TX>

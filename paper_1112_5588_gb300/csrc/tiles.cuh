@@ -231,8 +231,9 @@ __device__ __forceinline__ void lanes_tile(const Desc &d, const int4 &tl, TX *y)
 
 // One plan entry tl = {matrix, first sorted row, rows, kind} of matrix d, by
 // the whole CTA: kind 0 two rows per thread, 3 four rows per thread, 1 one
-// row per thread, 2 / 4 / 8 lanes per row.
-template <typename TV, typename TX, bool PAT = false, bool EARLY = false>
+// row per thread, 2 / 4 / 8 lanes per row (4 and 8 with U jagged diagonals a
+// round).
+template <typename TV, typename TX, bool PAT = false, bool EARLY = false, int U = 4>
 __device__ __forceinline__ void run_tile(const Desc &d, const int4 &tl) {
   TX *y = static_cast<TX *>(d.y);
   if (tl.w == 0) {
@@ -249,9 +250,9 @@ __device__ __forceinline__ void run_tile(const Desc &d, const int4 &tl) {
   } else if (tl.w == 2) {
     lanes_tile<TV, TX, 2, PAT, 4, EARLY>(d, tl, y);
   } else if (tl.w == 4) {
-    lanes_tile<TV, TX, 4, PAT, 4, EARLY>(d, tl, y);
+    lanes_tile<TV, TX, 4, PAT, U, EARLY>(d, tl, y);
   } else {
-    lanes_tile<TV, TX, 8, PAT, 4, EARLY>(d, tl, y);
+    lanes_tile<TV, TX, 8, PAT, U, EARLY>(d, tl, y);
   }
 }
 
@@ -275,56 +276,45 @@ __device__ __forceinline__ bool plan_entry_ok(const int4 &tl, int32_t n_pad) {
 // ordered by their work per lane, largest first, so the block scheduler
 // starts the long tiles first (on large matrices the short-row entries follow
 // in the original order of their first rows). Any order gives the same
-// results. short_only: the tiles of 4 and 8 lanes per row are
-// pjds_plan_long_kernel's, the launch before, which this one overlaps (and whose
-// end is awaited here, for what follows on the stream; that launch itself waits
-// for the kernels before it and only then lets this one start).
-template <typename TV, typename TX, bool PAT>
-__device__ __forceinline__ void plan_body(const Desc &d, const int4 *__restrict__ plan, int32_t n_pad,
-                                          int32_t short_only) {
+// results.
+template <typename TV, typename TX, bool PAT, int U = 4>
+__device__ __forceinline__ void plan_body(const Desc &d, const int4 *__restrict__ plan, int32_t n_pad) {
   unsigned k = blockIdx.x;
-  if (!short_only) dev::index_after_previous(k);
+  dev::index_after_previous(k);
   const int4 tl = plan[k];
-  if (plan_entry_ok(tl, n_pad) && !(short_only && tl.w >= 4)) run_tile<TV, TX, PAT, true>(d, tl);
-  if (short_only && blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
+  if (plan_entry_ok(tl, n_pad)) run_tile<TV, TX, PAT, true, U>(d, tl);
 }
 
 template <typename TV, typename TX, bool PAT = false>
 __global__ void __launch_bounds__(BT)
-    pjds_plan_kernel(const Desc d, const int4 *__restrict__ plan, int32_t n_pad, int32_t short_only) {
-  plan_body<TV, TX, PAT>(d, plan, n_pad, short_only);
+    pjds_plan_kernel(const Desc d, const int4 *__restrict__ plan, int32_t n_pad) {
+  plan_body<TV, TX, PAT>(d, plan, n_pad);
 }
 
 // fp64 values: bounded to six resident CTAs per SM (40 registers; unbounded
 // the instance takes 42, allocated as 48: five CTAs per SM). fp32 and bf16
-// stay unbounded (40 and 34 registers).
+// stay unbounded (32 and 40 registers).
 template <bool PAT = false>  // a template: instantiated only where it is launched
 __global__ void __launch_bounds__(BT, 6)
-    pjds_plan_kernel_f64(const Desc d, const int4 *__restrict__ plan, int32_t n_pad, int32_t short_only) {
-  plan_body<double, double, PAT>(d, plan, n_pad, short_only);
+    pjds_plan_kernel_f64(const Desc d, const int4 *__restrict__ plan, int32_t n_pad) {
+  plan_body<double, double, PAT>(d, plan, n_pad);
 }
 
-// The plan's tiles of 4 and 8 lanes per row, 16 jagged diagonals a round: a row
-// of 512 entries is 4 rounds of two latencies instead of 16. The registers (72 in
-// fp64) leave two or three CTAs on an SM, so the short rows, whose many tiles need
-// the warps, are not part of it. Zipf s = 2, 1M / 300k / 100k rows fp64 41 / 30 /
-// 22 -> 33 / 23 / 18 us, 1M rows fp32 38 -> 30 us (4 diagonals a round in one
-// launch; 8 in a launch of its own 36 us on 1M rows fp64; a row's entries loaded
-// by four times as many threads and added by shuffles 38 us, as every one of them
-// takes part in the fp64 additions).
+// The same for small plans with long rows, where one tile's rows set the time:
+// the tiles of 4 and 8 lanes per row with 16 jagged diagonals a round, so that a
+// row of 512 entries is 4 rounds of two latencies instead of 16, on registers
+// that leave four CTAs on an SM. Zipf s = 2, 4 diagonals a round -> 16: 1M / 300k
+// / 100k rows fp64 38.5 / 26.1 / 20.0 -> 33.6 / 21.3 / 15.9 us, 1M rows fp32 36.0
+// -> 29.7, bf16 34.0 -> 31.5; s = 1.6, 1M rows fp64 74.3 -> 70.3, fp32 71.0 ->
+// 63.4 (12 a round within 7% either way; 16 with three CTAs within 5%; a row's
+// entries loaded by four times as many threads and added by shuffles was slower,
+// as every one of them takes part in the fp64 additions). The long tiles in a
+// launch of their own, which the short ones' overlaps, would be 5-10% faster, but
+// the second launch could not wait for the kernels before the first by itself.
 template <typename TV, typename TX, bool PAT = false>
-__global__ void __launch_bounds__(BT, 2)
-    pjds_plan_long_kernel(const Desc d, const int4 *__restrict__ plan, int32_t n_pad) {
-  unsigned k = blockIdx.x;
-  dev::index_after_previous(k);
-  dev::let_next_start();
-  const int4 tl = plan[k];
-  if (tl.w < 4 || !plan_entry_ok(tl, n_pad)) return;
-  TX *y = static_cast<TX *>(d.y);
-  if (tl.w == 8)
-    lanes_tile<TV, TX, 8, PAT, 16, true>(d, tl, y);
-  else
-    lanes_tile<TV, TX, 4, PAT, 16, true>(d, tl, y);
+__global__ void __launch_bounds__(BT, 4)
+    pjds_plan_deep_kernel(const Desc d, const int4 *__restrict__ plan, int32_t n_pad) {
+  plan_body<TV, TX, PAT, 16>(d, plan, n_pad);
 }
 
 }  // namespace tiles

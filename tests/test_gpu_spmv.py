@@ -387,9 +387,9 @@ def test_plan_rows_bit_identical_to_uniform_mappings(P, name, make, permute, dty
     assert P.pjds_spmv_resolve(D)["plan"] == (1 if spread and big else -1)
 
 
-# plans of a launch for the long rows and one for the short ones (up to 3,072
-# tiles and rows of 64 entries), with all kinds of tile, only long rows, only one
-# kind of them, and a plan too large for it: bit for bit the uniform mappings
+# plans with long rows of up to 3,072 tiles (pjds_plan_deep_kernel), with all kinds
+# of tile, only long rows, only one kind of them, and a plan too large for it: bit
+# for bit the uniform mappings
 @pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
 @pytest.mark.parametrize("name", ["zipf", "long", "eight", "many"])
 def test_plan_long_and_short_rows(P, name, dtype):
@@ -408,7 +408,7 @@ def test_plan_long_and_short_rows(P, name, dtype):
     x = torch.from_numpy(synth.vector(A.n_cols, seed=2)).to("cuda", D.vec_dtype)
     y = torch.full((A.n_rows,), float("nan"), dtype=D.vec_dtype, device="cuda")
     P.pjds_spmv_cfg(D, x, y, plan=1)
-    twice = 2 * y  # (what follows on the stream sees both launches' rows)
+    twice = 2 * y  # (what follows on the stream sees all rows)
     s = torch.full_like(y, float("nan"))
     P.pjds_spmv_pattern(D, x, s, plan=1)
     lanes = np.zeros(H.n_pad, np.int64)
@@ -425,7 +425,7 @@ def test_plan_long_and_short_rows(P, name, dtype):
 
 
 # products of all mappings and of the ELLPACK-R baseline, launched while the one
-# before runs (the plan's: two launches): each reads what the one before has written (through the matrix
+# before runs: each reads what the one before has written (through the matrix
 # values too), one after another on a stream and in a graph, at the edges of a
 # round of 2, 4 or 8 lanes and of 8 diagonals, bit for bit the products one by one
 @pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
@@ -482,3 +482,51 @@ def test_products_one_after_another(P, lanes, dtype):
         graph.replay()
         torch.cuda.synchronize()
         assert all(torch.equal(a, b) for a, b in zip(v, want))
+
+
+# the same with x and y changing places from product to product and new data before every run, so that a
+# vector left in a cache from an earlier product would show: rows of 1 to 700 entries (the plan with more
+# diagonals a round and the one without, every number of lanes, ELLPACK-R), on a stream and in a graph
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+@pytest.mark.parametrize("lanes", [1, 4, 8, "plan", "plan of short rows", "ellr"])
+def test_products_back_and_forth(P, lanes, dtype):
+    import torch
+    n = 20_001
+    lens = np.minimum(np.random.default_rng(2).zipf(1.7, size=n), 60 if lanes == "plan of short rows" else 700)
+    A = tiny.from_lengths(lens, n, seed=8)
+    A = A._replace(val=A.val / np.repeat(np.maximum(lens, 1), lens))  # row sums below 1: products stay in range
+    if lanes == "ellr":
+        D = P.ellr_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, dtype=dtype).to_device("cuda")
+        product = lambda x, y: P.ellr_spmv(D, x, y)
+    else:
+        D = P.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
+        cfg = {"plan": -1, "threads_per_row": lanes, "rows_per_thread": 1} if isinstance(lanes, int) else {"plan": 1}
+        product = lambda x, y: P.pjds_spmv_cfg(D, x, y, **cfg)
+    a, b, first = (torch.empty(n, dtype=D.vec_dtype, device="cuda") for _ in range(3))
+    add = torch.from_numpy(synth.vector(n, seed=4)).to("cuda", D.vec_dtype)
+
+    def run(between=lambda: None):
+        for i in range(6):
+            between()
+            product(*((b, a) if i % 2 else (a, b)))
+            between()
+            if i == 2:
+                b.add_(add)
+
+    def check(go):
+        for seed in range(4):
+            first.copy_(torch.from_numpy(synth.vector(n, seed=10 + seed)))
+            a.copy_(first), b.zero_()
+            run(torch.cuda.synchronize)
+            want = a.clone(), b.clone()
+            a.copy_(first), b.zero_()
+            go()
+            torch.cuda.synchronize()
+            assert torch.equal(a, want[0]) and torch.equal(b, want[1]), seed
+        assert torch.isfinite(a).all() and a.abs().max() > 0
+
+    check(run)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run()
+    check(graph.replay)
