@@ -39,7 +39,8 @@ extern "C" {
  * n_rows k >= 2^20, val and col 16-byte aligned, and 28 of 32 sampled sets of four
  * rows found equal on the device) fp32 and bf16 products take four rows per thread.
  * On matrices of widely spread row lengths (longest row more than 4 times the mean)
- * rows of 64 entries or more run in an overlapping launch of their own. Column c of Y is
+ * rows of 64 entries or more run 16 entries a round, in the same launch as the others or,
+ * on large products, in one before it. Column c of Y is
  * computed in the same order and with the same fused multiply-adds as
  * pjds_spmv with one thread per row on column c of X. Original basis (permute_cols = 0): row i of
  * the sorted matrix is written to row perm[i] of Y; permuted basis: to row i.

@@ -62,27 +62,27 @@ __device__ __forceinline__ bool in_fours(const int32_t *__restrict__ col, int32_
   return __popc(__ballot_sync(0xffffffffu, same)) >= 28;
 }
 
-constexpr int LONG_BT = 64;           // threads of spmm_long_kernel's CTAs
-constexpr int LONG_U = 16;            // its jagged diagonals a round
-constexpr int32_t k_long_len = 64;    // and the shortest rows it takes
-// Lanes up to which it is launched (every lane a 16-byte chunk of a long row; on
-// more, the GPU is full without it): Zipf 400k rows s = 2 fp64 k = 64, 830,000 lanes
-// 342 us without, 314 with; s = 1.6 fp32 k = 128, 2.5 million lanes 319 and 448.
-constexpr int64_t k_long_max_lanes = 1 << 20;
+constexpr int LONG_BT = 64;           // threads of spmm_spread_kernel's CTAs
+constexpr int LONG_U = 16;            // jagged diagonals a round of a long row
+constexpr int32_t k_long_len = 64;    // and the shortest rows that are long
+// Lanes (every lane a 16-byte chunk of a row) up to which the long rows run apart
+// from the others, all lanes and those of long rows, and up to which one launch
+// takes both: the long rows' 128 registers leave the short ones few warps. Zipf, us
+// with all rows in spmm_kernel / long rows in the launch before it / both in one
+// launch: s = 2 fp64 400k rows k = 8 (1.6M lanes) 290 / 152 / 91, k = 16 306 / 173 /
+// 147, k = 24 313 / 201 / 217, k = 32 319 / 228 / 279, k = 48 (9.6M) 336 / 295 / 415,
+// k = 64 345 / 355 / 530; 400k rows fp32 k = 32 (3.2M) 204 / 94 / 116, k = 64 218 /
+// 126 / 220, k = 128 243 / 231 / 420; s = 1.6 100k rows fp32 k = 64 (1.6M) 156 / 85 /
+// 80, k = 128 154 / 87 / 151. Long rows' lanes: s = 1.6 400k rows fp32 k = 128 2.5
+// million 319 with all rows in spmm_kernel, 448 apart.
+constexpr int64_t k_one_launch_lanes = 1 << 21, k_apart_lanes = 10 << 20, k_long_max_lanes = 1 << 20;
 
-// Start of spmm_kernel and spmm_pair_kernel for thread t. Alone (fours = 0) the
-// launch overlaps the end of whatever is before it, and waits for it. Else it
-// overlaps the launch before that belongs to the same product and has waited, and
-// its end is that one's too: spmm_quad_kernel (fours = the rows of the first jagged
-// diagonal; true when that one does the work) or spmm_long_kernel (fours < 0).
+// Start of spmm_kernel and spmm_pair_kernel for thread t: the launch overlaps the
+// end of the one before and waits for it. Whether that one has done the work:
+// spmm_quad_kernel (fours = the rows of the first jagged diagonal).
 __device__ __forceinline__ bool left_to_quads(const int32_t *__restrict__ col, int32_t n_rows, int32_t fours, int64_t &t) {
-  if (fours == 0) {
-    dev::index_after_previous(t);
-    return false;
-  }
-  const bool yes = fours > 0 && in_fours(col, n_rows, fours);
-  if ((fours > 0 && !yes) || blockIdx.x == 0) asm volatile("griddepcontrol.wait;" ::: "memory");
-  return yes;
+  dev::index_after_previous(t);
+  return fours > 0 && in_fours(col, n_rows, fours);
 }
 
 // Thread t: sorted row i = t / lr and, of its k columns, the CH 16-byte chunks
@@ -95,20 +95,19 @@ __device__ __forceinline__ bool left_to_quads(const int32_t *__restrict__ col, i
 // (dev::pattern_ones_address), read where the product reads its values, so
 // the kernel keeps the product's instructions, registers and occupancy and
 // only the value stream is missing; fma(1, x, acc) is acc + x rounded once.
-template <typename TV, typename TX, typename IDX, bool SCATTER, int CH, bool PAT = false>
-__global__ void __launch_bounds__(BT)
-    spmm_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
-                const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X,
-                TX *Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
+// short_only: rows of k_long_len entries or more are left out.
+template <typename TV, typename TX, typename IDX, bool SCATTER, int CH, bool PAT>
+__device__ __forceinline__ void spmm_row(const TV *__restrict__ val, const int32_t *__restrict__ col,
+                                         const int64_t *__restrict__ col_start, const int32_t *__restrict__ block_len,
+                                         const int32_t *__restrict__ perm, const TX *X, TX *Y, int32_t n_rows,
+                                         int32_t b, int32_t k, int32_t lr, int64_t t, bool short_only) {
   using TA = typename dev::Acc<TV>::T;
   constexpr int VW = V16<TX>::W, W = VW * CH, U = 4;
-  int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
-  if (left_to_quads(col, n_rows, fours, t)) return;
   const int64_t i = t / lr;
   const int32_t q = (int32_t)(t % lr);
   if (i >= n_rows) return;
   const int32_t L = PJDS_IN(i / b, PJDS_EXT(n_blocks), dev::CHK_BLOCK) ? __ldg(block_len + (int32_t)(i / b)) : 0;
-  if (fours < 0 && L >= -fours) return;  // spmm_long_kernel's
+  if (short_only && L >= k_long_len) return;
   TA acc[W];
 #pragma unroll
   for (int w = 0; w < W; ++w) acc[w] = TA(0);
@@ -160,6 +159,18 @@ __global__ void __launch_bounds__(BT)
 #pragma unroll
   for (int h = 0; h < CH; ++h)
     V16<TX>::store(Y + r * k + (int64_t)q * W + h * VW, *reinterpret_cast<const TX(*)[VW]>(&out[h * VW]));
+}
+
+// fours: left_to_quads; below 0, the rows of k_long_len entries or more are the
+// launch before's (spmm_spread_kernel).
+template <typename TV, typename TX, typename IDX, bool SCATTER, int CH, bool PAT = false>
+__global__ void __launch_bounds__(BT)
+    spmm_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
+                const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X,
+                TX *Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
+  int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
+  if (left_to_quads(col, n_rows, fours, t)) return;
+  spmm_row<TV, TX, IDX, SCATTER, CH, PAT>(val, col, col_start, block_len, perm, X, Y, n_rows, b, k, lr, t, fours < 0);
 }
 
 // The pattern product's value address reduced to a slot of the ones (0 for
@@ -440,31 +451,26 @@ __global__ void __launch_bounds__(BT, MB)
   }
 }
 
-// The rows of min_len entries or more of a matrix with widely spread lengths (the
-// first sorted rows), one chunk of the k columns per lane. Bound by latency: a long
-// row is one serial sum, in the order of spmm_kernel, on a GPU that the few long
-// rows leave idle. U jagged diagonals a round; their columns and values are loaded
-// one round ahead and their offsets two, so that a round is one latency (and in
-// fp64 the sum's additions) instead of three. Zipf, against the rows in spmm_kernel:
-// 100k rows s = 2 fp64 k = 8 176 -> 88 us, 400k rows fp32 k = 4 176 -> 71, s = 1.6
-// fp64 k = 4 289 -> 106, 20k rows bf16 k = 32 132 -> 39, 3k rows fp64 k = 2 110 ->
-// 69 (8 diagonals a round 133, 127, 156, 71, 84; rows from 32 or 128 entries on
+// A long row (k_long_len entries or more; thread t as in spmm_kernel, one chunk of
+// the k columns). Bound by latency: it is one serial sum, in the order of
+// spmm_kernel, on a GPU that the few long rows leave idle. U jagged diagonals a
+// round; their columns and values are loaded one round ahead and their offsets
+// two, so that a round is one latency (and in fp64 the sum's additions) instead of
+// three (8 diagonals a round take 5-80% longer; rows from 32 or 128 entries on
 // within 5%).
 template <typename TV, typename TX, typename IDX, bool SCATTER, int U, bool PAT>
-__global__ void __launch_bounds__(LONG_BT)
-    spmm_long_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
-                     const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X, TX *Y,
-                     int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t min_len) {
+__device__ __forceinline__ void spmm_long_row(const TV *__restrict__ val, const int32_t *__restrict__ col,
+                                              const int64_t *__restrict__ col_start,
+                                              const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm,
+                                              const TX *X, TX *Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr,
+                                              int64_t t) {
   using TA = typename dev::Acc<TV>::T;
   constexpr int W = V16<TX>::W;
-  int64_t t = (int64_t)blockIdx.x * LONG_BT + threadIdx.x;
-  dev::index_after_previous(t);
-  dev::let_next_start();
   const int64_t i = t / lr;
   const int32_t q = (int32_t)(t % lr);
   if (i >= n_rows) return;
   const int32_t L = PJDS_IN(i / b, PJDS_EXT(n_blocks), dev::CHK_BLOCK) ? __ldg(block_len + (int32_t)(i / b)) : 0;
-  if (L < min_len) return;
+  if (L < k_long_len) return;
   const int64_t r = SCATTER ? (int64_t)__ldcs(perm + i) : i;
   const TX *Xq = X + (int64_t)q * W;
   IDX start[U];  // of the round after the next one's columns and values
@@ -521,6 +527,27 @@ __global__ void __launch_bounds__(LONG_BT)
 #pragma unroll
   for (int w = 0; w < W; ++w) out[w] = (TX)acc[w];
   V16<TX>::store(Y + r * k + (int64_t)q * W, out);
+}
+
+// Matrices of widely spread row lengths: the long rows by the first n_long CTAs,
+// the others by the CTAs after them, or, if there are none, by the next launch
+// (spmm_kernel), which may then be placed early. Zipf, against all rows in
+// spmm_kernel: s = 2 400k rows fp32 k = 4 176 -> 46 us, 100k rows fp64 k = 8 211 ->
+// 79, 3k rows fp64 k = 2 104 -> 52, 20k rows bf16 k = 32 135 -> 27, s = 1.6 400k rows
+// fp64 k = 4 292 -> 95.
+template <typename TV, typename TX, typename IDX, bool SCATTER, bool PAT>
+__global__ void __launch_bounds__(LONG_BT, 8)
+    spmm_spread_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
+                       const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X, TX *Y,
+                       int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t n_long) {
+  int64_t t = (int64_t)blockIdx.x * LONG_BT + threadIdx.x;
+  dev::index_after_previous(t);
+  if (gridDim.x == (unsigned)n_long) dev::let_next_start();
+  if (blockIdx.x < (unsigned)n_long)
+    spmm_long_row<TV, TX, IDX, SCATTER, LONG_U, PAT>(val, col, col_start, block_len, perm, X, Y, n_rows, b, k, lr, t);
+  else
+    spmm_row<TV, TX, IDX, SCATTER, 1, PAT>(val, col, col_start, block_len, perm, X, Y, n_rows, b, k, lr,
+                                           t - (int64_t)n_long * LONG_BT, true);
 }
 
 // ----------------------------------------------------------------------------- persistent batch
@@ -642,7 +669,8 @@ static int spmm_chunks(const pjds_dev *A, int32_t k, int vw) {
 // 2^20 elements of Y (60,000 rows of 80: k = 8 33 us against 38, not taken, k = 32
 // 62 against 36; 280,000 rows of 40: k = 8 42 against 36), and val and col aligned
 // for 16-byte loads. If the rows turn out not to share in fours, the other kernel
-// runs, 2 us later.
+// runs, 2 us later; if they do, its CTAs wait for spmm_quad_kernel and leave, 1 to
+// 3 us after it.
 static bool offer_quads(const pjds_dev *A, int32_t k) {
   return A->dtype != PJDS_F64 && A->pair_share >= 900 && A->nnz >= 16 * (int64_t)A->n_rows && k % 8 == 0 &&
          (int64_t)A->n_rows * k >= (1 << 20) && (int64_t)A->n_rows * k < (1ll << 36) && A->n_rows >= 128 &&
@@ -692,6 +720,10 @@ static int launch_spmm(const pjds_dev *A, int32_t k, const void *X, void *Y, cud
 #ifdef PJDS_CHECKED
   dev::set_extents(dev::Extents{A->n_stored, A->n_cols, A->n_rows, A->n_blocks, A->n_max + 1}, s);
 #endif
+  auto launched = [] {
+    const cudaError_t e = cudaGetLastError();
+    return e == cudaSuccess ? PJDS_OK : set_error(PJDS_ECUDA, "pjds_spmm launch: %s", cudaGetErrorString(e));
+  };
   int32_t fours = 0;
   if constexpr (!std::is_same<TX, double>::value) {
     if (offer_quads(A, k)) {
@@ -706,25 +738,27 @@ static int launch_spmm(const pjds_dev *A, int32_t k, const void *X, void *Y, cud
       }
     }
   }
-#define SPMML(IDX, SC)                                                                                              \
-  dev::launch_early(spmm_long_kernel<TV, TX, IDX, SC, LONG_U, PAT>, (unsigned)long_grid, LONG_BT, s, val, A->col, A->col_start, \
-                    A->block_len, A->perm, x, y, A->n_rows, A->b, k, lr, k_long_len)
+#define SPMMS(IDX, SC)                                                                                               \
+  dev::launch_early(spmm_spread_kernel<TV, TX, IDX, SC, PAT>, (unsigned)(n_long + n_short), LONG_BT, s, val, A->col, \
+                    A->col_start, A->block_len, A->perm, x, y, A->n_rows, A->b, k, lr, (int32_t)n_long)
   if (!pair_u && fours == 0 && ch == 1 && A->n_max >= k_long_len && (int64_t)A->n_max * A->n_rows > 4 * A->nnz) {
     // a row in a block of that length takes that many stored entries
     const int64_t most = std::min<int64_t>(A->n_rows, A->n_stored / k_long_len);
-    const int64_t long_grid = (most * lr + LONG_BT - 1) / LONG_BT;
-    if (most > 0 && most * lr <= k_long_max_lanes) {
-      fours = -k_long_len;
+    if (most > 0 && most * lr <= k_long_max_lanes && threads <= k_apart_lanes) {
+      const bool one = threads <= k_one_launch_lanes;
+      const int64_t n_long = (most * lr + LONG_BT - 1) / LONG_BT, n_short = one ? (threads + LONG_BT - 1) / LONG_BT : 0;
       if (small) {
-        if (sc) SPMML(int32_t, true);
-        else SPMML(int32_t, false);
+        if (sc) SPMMS(int32_t, true);
+        else SPMMS(int32_t, false);
       } else {
-        if (sc) SPMML(int64_t, true);
-        else SPMML(int64_t, false);
+        if (sc) SPMMS(int64_t, true);
+        else SPMMS(int64_t, false);
       }
+      if (one) return launched();
+      fours = -1;
     }
   }
-#undef SPMML
+#undef SPMMS
 #define SPMM(IDX, SC, CH)                                                                                             \
   dev::launch_early(spmm_kernel<TV, TX, IDX, SC, CH, PAT>, (unsigned)grid, BT, s, val, A->col, A->col_start, A->block_len, \
                A->perm, x, y, A->n_rows, A->b, k, lr, fours)
@@ -764,8 +798,7 @@ static int launch_spmm(const pjds_dev *A, int32_t k, const void *X, void *Y, cud
 #undef SPMMP
 #undef SPMM_CH
 #undef SPMM
-  cudaError_t e = cudaGetLastError();
-  return e == cudaSuccess ? PJDS_OK : set_error(PJDS_ECUDA, "pjds_spmm launch: %s", cudaGetErrorString(e));
+  return launched();
 }
 
 template <bool PAT>

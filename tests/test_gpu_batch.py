@@ -394,17 +394,19 @@ def test_spmm_one_after_another(mods, dtype, k, bs, nb):
         assert all(torch.equal(a, b) for a, b in zip(v, want))
 
 
-# long rows in a launch of their own (widely spread lengths, rows of 64 entries or
-# more): lengths at the edges of its rounds of 16, only long rows and a few, one
-# long row, and past the lanes up to which it is launched; each column in the order
-# and with the multiply-adds of the single product
-@pytest.mark.parametrize("dtype,k", [("f64", 2), ("f64", 6), ("f32", 4), ("bf16", 24), ("f32", 128)])
-@pytest.mark.parametrize("name", ["edges", "one", "many"])
+# long rows apart from the others (widely spread lengths, rows of 64 entries or more), in one launch (up to 2^21
+# 16-byte chunks of Y) and in two ("two": 2,112,000 of them at k = 64 fp64 and 128 fp32): lengths at the edges of a
+# round of 16, only long rows and a few, one long row; each column in the order and with the multiply-adds of the
+# single product
+@pytest.mark.parametrize("name,dtype,k", [(name, dtype, k) for name in ("edges", "one", "many") for dtype, k in
+                                          (("f64", 2), ("f64", 6), ("f32", 4), ("bf16", 24), ("f32", 128))] +
+                         [("two", "f64", 64), ("two", "f32", 128), ("two", "bf16", 128)])
 def test_spmm_long_rows(mods, dtype, k, name):
     torch, pjds, batch = mods
     lens = {"edges": [64, 65, 79, 80, 81, 63, 95, 96, 97, 111, 112, 113, 128, 700] + [3] * 4001,
             "one": [64] + [1] * 900,
-            "many": list(np.minimum(np.random.default_rng(3).zipf(1.5, size=9000), 600))}[name]
+            "many": list(np.minimum(np.random.default_rng(3).zipf(1.5, size=9000), 600)),
+            "two": list(np.minimum(np.random.default_rng(4).zipf(1.9, size=66_000), 300))}[name]
     A = tiny.from_lengths(np.array(lens), 9001, seed=k)
     rng = np.random.default_rng(5)
     D = pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
@@ -412,7 +414,7 @@ def test_spmm_long_rows(mods, dtype, k, name):
     X = torch.from_numpy(rng.uniform(-1, 1, size=(A.n_cols, k))).to("cuda", D.vec_dtype)
     Y, P = (torch.full((A.n_rows, k), float("nan"), dtype=D.vec_dtype, device="cuda") for _ in range(2))
     batch.spmm(D, X, Y)
-    twice = 2 * Y  # (what follows on the stream sees both launches' rows)
+    twice = 2 * Y  # (what follows on the stream sees all rows)
     batch.spmm_pattern(D, X, P)
     y1, p1 = (torch.empty(A.n_rows, dtype=D.vec_dtype, device="cuda") for _ in range(2))
     for c in (0, 1, k - 1):
@@ -459,3 +461,57 @@ def test_small_batches_one_after_another(mods, dtype):
         go()
         torch.cuda.synchronize()
         assert all(torch.equal(v, w) for v, w in zip(a, want))
+
+
+# block products with X and Y changing places and new data before every run, so that an element left in a cache
+# from an earlier product would show: one row a thread, long rows in one launch and in two, fours and the fall back
+# from them, on a stream and in a graph
+@pytest.mark.parametrize("name,dtype,k", [("rows", "f64", 2), ("rows", "f32", 8), ("spread", "f64", 4),
+                                          ("spread", "bf16", 16), ("spread", "f32", 128), ("fours", "f32", 32),
+                                          ("fours", "bf16", 32), ("twos", "f32", 32), ("sixes", "bf16", 32)])
+def test_block_products_back_and_forth(mods, name, dtype, k):
+    torch, pjds, batch = mods
+    if name == "spread":
+        n = 66_000 if k == 128 else 20_001  # two launches and one
+        A = tiny.from_lengths(np.minimum(np.random.default_rng(2).zipf(1.9, size=n), 300), n, seed=6)
+    elif name == "rows":
+        n = 20_001
+        A = tiny.from_lengths(np.full(n, 7), n, seed=6)
+    else:
+        bs, nb = {"fours": (4, 5), "twos": (2, 10), "sixes": (6, 4)}[name]
+        n = 34_950
+        A = _block_rows(n, n // bs // 2, bs, nb, 0.01, seed=bs)
+    lens = np.maximum(np.diff(A.row_ptr), 1)
+    A = A._replace(val=A.val / np.repeat(lens, np.diff(A.row_ptr)))  # row sums below 1: products stay in range
+    D = pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
+    m = max(A.n_rows, A.n_cols)
+    a, b, first, add = (torch.empty(m, k, dtype=D.vec_dtype, device="cuda") for _ in range(4))
+    g = torch.Generator("cuda").manual_seed(k)
+    add.uniform_(-1, 1, generator=g)
+
+    def run(between=lambda: None):
+        for i in range(6):
+            x, y = (b, a) if i % 2 else (a, b)
+            between()
+            batch.spmm(D, x[:A.n_cols], y[:A.n_rows])
+            between()
+            if i == 2:
+                b.add_(add)
+
+    def check(go):
+        for _ in range(4):
+            first.uniform_(-1, 1, generator=g)
+            a.copy_(first), b.zero_()
+            run(torch.cuda.synchronize)
+            want = a.clone(), b.clone()
+            a.copy_(first), b.zero_()
+            go()
+            torch.cuda.synchronize()
+            assert torch.equal(a, want[0]) and torch.equal(b, want[1])
+        assert torch.isfinite(a).all() and a.abs().max() > 0
+
+    check(run)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        run()
+    check(graph.replay)
