@@ -53,7 +53,8 @@ struct V16<double> {
 // of two or six rows from blocks of four.
 __device__ __forceinline__ bool in_fours(const int32_t *__restrict__ col, int32_t n_rows, int32_t n_stored0) {
   const uint32_t l = threadIdx.x & 31;
-  const int64_t i = (int64_t)(n_rows / 4 - 1) * l / 31 * 4;
+  int64_t i = (int64_t)(n_rows / 4 - 1) * l / 31 * 4;
+  asm volatile("" : "+l"(i)::"memory");  // after the wait (dev::index_after_previous)
   bool same = false;
   if (i + 4 <= n_stored0) {
     const int4 a = __ldg(reinterpret_cast<const int4 *>(col + i));
@@ -80,8 +81,9 @@ constexpr int64_t k_one_launch_lanes = 1 << 21, k_apart_lanes = 10 << 20, k_long
 // Start of spmm_kernel and spmm_pair_kernel for thread t: the launch overlaps the
 // end of the one before and waits for it. Whether that one has done the work:
 // spmm_quad_kernel (fours = the rows of the first jagged diagonal).
-__device__ __forceinline__ bool left_to_quads(const int32_t *__restrict__ col, int32_t n_rows, int32_t fours, int64_t &t) {
-  dev::index_after_previous(t);
+__device__ __forceinline__ bool left_to_quads(const int32_t *__restrict__ col, const int64_t *&col_start, int32_t n_rows,
+                                              int32_t fours, int64_t &t) {
+  dev::index_after_previous(t, col_start);
   return fours > 0 && in_fours(col, n_rows, fours);
 }
 
@@ -165,11 +167,11 @@ __device__ __forceinline__ void spmm_row(const TV *__restrict__ val, const int32
 // launch before's (spmm_spread_kernel).
 template <typename TV, typename TX, typename IDX, bool SCATTER, int CH, bool PAT = false>
 __global__ void __launch_bounds__(BT)
-    spmm_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
+    spmm_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *col_start,
                 const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X,
                 TX *Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
   int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
-  if (left_to_quads(col, n_rows, fours, t)) return;
+  if (left_to_quads(col, col_start, n_rows, fours, t)) return;
   spmm_row<TV, TX, IDX, SCATTER, CH, PAT>(val, col, col_start, block_len, perm, X, Y, n_rows, b, k, lr, t, fours < 0);
 }
 
@@ -218,13 +220,13 @@ __device__ __forceinline__ void ld_ones(const TV *p, TV (&v)[R]) {
 // a pad of the first is a pad of the second.
 template <typename TV, typename TX, typename IDX, bool SCATTER, int CH, int U, bool PAT = false>
 __global__ void __launch_bounds__(BT)
-    spmm_pair_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
+    spmm_pair_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *col_start,
                      const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X,
                      TX *Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
   using TA = typename dev::Acc<TV>::T;
   constexpr int VW = V16<TX>::W, W = VW * CH;
   int64_t t = (int64_t)blockIdx.x * BT + threadIdx.x;
-  if (left_to_quads(col, n_rows, fours, t)) return;
+  if (left_to_quads(col, col_start, n_rows, fours, t)) return;
   const int64_t i = 2 * (t / lr);
   const int32_t q = (int32_t)(t % lr);
   if (i >= n_rows) return;
@@ -401,15 +403,16 @@ __device__ __forceinline__ void shared_rows(const TV *__restrict__ val, const in
 // (k = 64: 326 against 386).
 template <typename TV, typename TX, typename IDX, bool SCATTER, int U, int MB, bool PAT>
 __global__ void __launch_bounds__(BT, MB)
-    spmm_quad_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
+    spmm_quad_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *col_start,
                      const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X,
                      TX *Y, int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t fours) {
   using TA = typename dev::Acc<TV>::T;
   constexpr int CH = 2, VW = V16<TX>::W, W = VW * CH;
-  dev::index_after_previous(fours);
+  uint32_t t = blockIdx.x * (uint32_t)BT + threadIdx.x;
+  dev::index_after_previous(t, col_start);
   dev::let_next_start();
   if (!in_fours(col, n_rows, fours)) return;
-  const uint32_t t = blockIdx.x * (uint32_t)BT + threadIdx.x, p = t / (uint32_t)lr, q = t - p * (uint32_t)lr;
+  const uint32_t p = t / (uint32_t)lr, q = t - p * (uint32_t)lr;
   if (p >= ((uint32_t)n_rows + 3) / 4) return;
   const int32_t i = 4 * (int32_t)p;
   const int32_t L = PJDS_IN(i / b, PJDS_EXT(n_blocks), dev::CHK_BLOCK) ? __ldg(block_len + (uint32_t)i / (uint32_t)b) : 0;
@@ -537,11 +540,11 @@ __device__ __forceinline__ void spmm_long_row(const TV *__restrict__ val, const 
 // fp64 k = 4 292 -> 95.
 template <typename TV, typename TX, typename IDX, bool SCATTER, bool PAT>
 __global__ void __launch_bounds__(LONG_BT, 8)
-    spmm_spread_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *__restrict__ col_start,
+    spmm_spread_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col, const int64_t *col_start,
                        const int32_t *__restrict__ block_len, const int32_t *__restrict__ perm, const TX *X, TX *Y,
                        int32_t n_rows, int32_t b, int32_t k, int32_t lr, int32_t n_long) {
   int64_t t = (int64_t)blockIdx.x * LONG_BT + threadIdx.x;
-  dev::index_after_previous(t);
+  dev::index_after_previous(t, col_start);
   if (gridDim.x == (unsigned)n_long) dev::let_next_start();
   if (blockIdx.x < (unsigned)n_long)
     spmm_long_row<TV, TX, IDX, SCATTER, LONG_U, PAT>(val, col, col_start, block_len, perm, X, Y, n_rows, b, k, lr, t);

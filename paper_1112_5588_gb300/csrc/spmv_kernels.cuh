@@ -200,21 +200,26 @@ __device__ __forceinline__ TX gather(const TX *__restrict__ x, int32_t c) {
 // not even one of read-only memory, can be moved ahead, and x is read by ordinary
 // loads.
 __device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+template <typename P>
+__device__ __forceinline__ void hold(P *&p) {
+  asm volatile("" : "+l"(p)::"memory");
+}
 template <typename... P>
 __device__ __forceinline__ void after_previous(P *&...p) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
-  const auto hold = [](auto *&q) { asm volatile("" : "+l"(q)::"memory"); };
   (hold(p), ...);
 }
-// The same for a kernel whose addresses all come from one index: the index goes
-// through the wait (no registers for the pointers; x without __restrict__).
-template <typename I>
-__device__ __forceinline__ void index_after_previous(I &i) {
+// The same for a kernel whose addresses come from one index: the index goes
+// through the wait (no registers for those pointers; x without __restrict__), and
+// the pointers whose addresses it does not enter (the offsets', col_start + j).
+template <typename I, typename... P>
+__device__ __forceinline__ void index_after_previous(I &i, P *&...p) {
   asm volatile("griddepcontrol.wait;" ::: "memory");
   if constexpr (sizeof(I) == 8)
     asm volatile("" : "+l"(i)::"memory");
   else
     asm volatile("" : "+r"(i)::"memory");
+  (hold(p), ...);
 }
 
 // Launch with programmatic dependence on the kernel before (after_previous,
@@ -305,7 +310,7 @@ __device__ __forceinline__ TX gather_n(const TX *__restrict__ x, int32_t c, int3
 // pattern_ones, L1 hits) and y stores.
 template <typename TV, typename TX, typename IDX, int R, int U, bool SCATTER, bool PAT = false>
 __global__ void __launch_bounds__(512) pjds_rows_kernel(const TV *__restrict__ val, const int32_t *__restrict__ col,
-                                                        const int64_t *__restrict__ col_start,
+                                                        const int64_t *col_start,
                                                         const int32_t *__restrict__ block_len,
                                                         const int32_t *__restrict__ perm,
                                                         const int32_t *__restrict__ order, const TX *x,
@@ -313,7 +318,7 @@ __global__ void __launch_bounds__(512) pjds_rows_kernel(const TV *__restrict__ v
   using TA = typename Acc<TV>::T;
   const int64_t t = (int64_t)blockIdx.x * blockDim.x + threadIdx.x;
   int64_t i0 = t * R;
-  index_after_previous(i0);
+  index_after_previous(i0, col_start);
   if (i0 >= n_pad) return;
   if (order && !tile_row(order, n_pad, i0)) return;
   if (!PJDS_IN(i0 / b, PJDS_EXT(n_blocks), CHK_BLOCK)) return;

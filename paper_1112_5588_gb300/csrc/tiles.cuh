@@ -278,9 +278,9 @@ __device__ __forceinline__ bool plan_entry_ok(const int4 &tl, int32_t n_pad) {
 // in the original order of their first rows). Any order gives the same
 // results.
 template <typename TV, typename TX, bool PAT, int U = 4>
-__device__ __forceinline__ void plan_body(const Desc &d, const int4 *__restrict__ plan, int32_t n_pad) {
+__device__ __forceinline__ void plan_body(Desc d, const int4 *__restrict__ plan, int32_t n_pad) {
   unsigned k = blockIdx.x;
-  dev::index_after_previous(k);
+  dev::index_after_previous(k, d.col_start);
   const int4 tl = plan[k];
   if (plan_entry_ok(tl, n_pad)) run_tile<TV, TX, PAT, true, U>(d, tl);
 }
