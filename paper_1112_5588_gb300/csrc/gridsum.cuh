@@ -1,13 +1,17 @@
-// fp64 sums over a warp and over all CTAs of a cooperative launch (cg.cu,
-// lanczos.cu): every CTA gives its threads' values and every thread gets the
-// total, with no return to the host and no second launch.
+// fp64 sums over a warp, a CTA and all CTAs of a cooperative launch (cg.cu, mlp.cu)
+// or over the partial sums of a launch (krylov.cu). Over a grid every CTA gives its
+// threads' values and every thread gets the total, with no return to the host and
+// no second launch.
 //
 // A dependent fp64 add takes 70 cycles here and a warp's fp64 add holds the
 // SM's fp64 pipe for 16, so that a shuffle tree of fp64 adds over 1024 threads
 // costs 5000 cycles (2.5 us). The sums are therefore taken in integers: each
-// level finds the largest exponent, shifts its values to it as 58-bit fixed
-// point and adds them as 64-bit integers, which is exact (the shift keeps 56
-// bits or more below the largest value; a tree of fp64 adds keeps 53).
+// level finds the largest exponent, shifts its values to it as fixed point,
+// rounded to nearest, and adds them as integers, which is exact. A warp's values
+// are each rounded at 2^-57 of the largest one or less, 160 CTAs' at 2^-60, and the
+// sum at 2^-57 of itself: a warp's sum and the CTAs' are off by less than 2^-51 of
+// the largest value and 2^-56 of the sum, trees of fp64 adds by up to 5 2^-53 and 8
+// 2^-53 of the sum of the magnitudes.
 //
 // Between CTAs: a CTA writes its sum into a slot of its own as two words, each
 // with the number of the sum (its epoch); one warp of every CTA reads all slots
@@ -48,8 +52,8 @@ struct GridSlots {
   uint32_t pad2[31];
 };
 
-// A sum in fixed point: f 2^(e - 1078); e = 0x7ff: f holds the bits of an
-// infinity or a NaN.
+// A sum in fixed point: f 2^(e - 1079), |f| at most 2^57, e from 1 on; e = 0x7ff: f
+// holds the bits of an infinity or a NaN.
 struct Fixed {
   long long f;
   uint32_t e;
@@ -62,7 +66,7 @@ __device__ __forceinline__ Fixed fixed_of(double v) {
   if (a.e == 0x7ffu) {
     a.f = (long long)b;
   } else {
-    const unsigned long long m = ((b & 0xfffffffffffffull) | (a.e ? 0x10000000000000ull : 0ull)) << 3;
+    const unsigned long long m = ((b & 0xfffffffffffffull) | (a.e ? 0x10000000000000ull : 0ull)) << 4;
     a.f = (long long)b < 0 ? -(long long)m : (long long)m;
     a.e = a.e ? a.e : 1u;
   }
@@ -75,8 +79,8 @@ __device__ __forceinline__ double double_of(const Fixed &a) {
   const bool neg = a.f < 0;
   unsigned long long m = neg ? 0ull - (unsigned long long)a.f : (unsigned long long)a.f;
   const int lz = __clzll((long long)m);
-  const int e = (int)a.e + 8 - lz;  // biased exponent of the result (m has bit 63 - lz as its highest)
-  if (e < 1 || e > 2045) return ldexp((double)a.f, (int)a.e - 1078);
+  const int e = (int)a.e + 7 - lz;  // biased exponent of the result (m has bit 63 - lz as its highest)
+  if (e < 1 || e > 2045) return ldexp((double)a.f, (int)a.e - 1079);
   m <<= lz;
   // 53 bits, to nearest even; a carry runs into the exponent as it should
   const unsigned long long keep = m >> 11, low = m & 0x7ffull;
@@ -85,50 +89,50 @@ __device__ __forceinline__ double double_of(const Fixed &a) {
   return __longlong_as_double((long long)(b | (neg ? 0x8000000000000000ull : 0ull)));
 }
 
-// Sum over the warp of N values a lane, in every lane; |f| of the inputs below 2^57.
+// Sum over the warp of N values a lane, in every lane.
 template <int N>
 __device__ __forceinline__ Fixed warp_sum(const Fixed (&a)[N]) {
+  static_assert(N <= 7, "a lane's sum beyond 63 bits");
+  constexpr int G = N > 1 ? 3 : 0;  // bits kept below a value's: N 2^(57 + G) is below 2^63
   uint32_t em = a[0].e;
 #pragma unroll
   for (int q = 1; q < N; ++q) em = max(em, a[q].e);
   em = __reduce_max_sync(0xffffffffu, em);
   Fixed s;
-  s.e = em;
   if (em == 0x7ffu) {  // an infinity or a NaN: finite values do not matter beside it
     double v = 0.0;
 #pragma unroll
     for (int q = 0; q < N; ++q)
       if (a[q].e == 0x7ffu) v += __longlong_as_double(a[q].f);
     for (int o = 16; o > 0; o >>= 1) v += __shfl_xor_sync(0xffffffffu, v, o);
+    s.e = 0x7ffu;
     s.f = __double_as_longlong(v);
     return s;
   }
-  // up to 6 bits of carry for 5 x 32 values of 57 bits and a sign: 3 bits fewer first
-  constexpr int drop = N > 1 ? 3 : 0;
-  static_assert(N <= 8, "carries beyond 63 bits");
   long long f = 0;
 #pragma unroll
-  for (int q = 0; q < N; ++q) {
-    const uint32_t d = min(em - a[q].e + drop, 62u);
-    // to nearest where many are cut: 160 of them would add up to 80 units
-    f += N > 1 ? (a[q].f + ((1ll << d) >> 1)) >> d : a[q].f >> d;
-  }
+  for (int q = 0; q < N; ++q)  // (G + 1 bits more, and the last one rounded)
+    f += (((long long)((unsigned long long)a[q].f << (G + 1)) >> min(em - a[q].e, 63u)) + 1) >> 1;
   // in three parts, whose sums over 32 lanes fit 32 bits
   const uint32_t s0 = __reduce_add_sync(0xffffffffu, (uint32_t)f & 0x3ffffffu);
   const uint32_t s1 = __reduce_add_sync(0xffffffffu, (uint32_t)(f >> 26) & 0x3ffffffu);
   const int32_t s2 = __reduce_add_sync(0xffffffffu, (int32_t)(f >> 52));
-  f = (long long)s0 + ((long long)s1 << 26) + ((long long)s2 << 52);
-  // back to 57 bits: below 2^57, and up to it, so that the next sum's shifts drop zeros
-  const unsigned long long m = f < 0 ? 0ull - (unsigned long long)f : (unsigned long long)f;
-  int sh = m ? 7 - __clzll((long long)m) : 0;  // > 0: too large by sh bits
-  if (sh > 0) {
-    f >>= sh;
-  } else {
-    sh = -min(-sh, (int)em + drop - 1);
-    f = (long long)((unsigned long long)f << -sh);
+  int e = (int)em - G;
+  if constexpr (N == 1) {  // below 2^62
+    f = (long long)s0 + ((long long)s1 << 26) + ((long long)s2 << 52);
+  } else {  // hi 2^26 + low, hi below 2^42
+    const long long hi = ((long long)s2 << 26) + s1 + (s0 >> 26);
+    const uint32_t low = s0 & 0x3ffffffu;
+    const bool far = hi < -(1ll << 36) || hi >= (1ll << 36);
+    f = far ? (hi << 20) + ((low + 32u) >> 6) : (hi << 26) + low;
+    e += far ? 6 : 0;
   }
-  s.f = f;
-  s.e = (uint32_t)((int)em + drop + sh);
+  // to 57 bits, from where the next sum's shifts drop nothing that a double holds, and e from 1 on
+  const unsigned long long m = f < 0 ? 0ull - (unsigned long long)f : (unsigned long long)f;
+  const int sh = max(m ? 7 - __clzll((long long)m) : 0, 1 - e);  // > 0: too large by sh bits
+  s.f = sh > 0 ? (f + ((1u << sh) >> 1)) >> sh : (long long)((unsigned long long)f << -sh);
+  s.e = (uint32_t)(e + sh);
+  if (f == 0) s.e = 1u;
   if (s.e >= 0x7ffu) {  // the sum overflows
     s.e = 0x7ffu;
     s.f = f < 0 ? (long long)0xfff0000000000000ull : 0x7ff0000000000000ll;

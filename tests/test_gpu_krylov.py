@@ -16,6 +16,8 @@ Tolerances:
     fp64 oracle on the exact matrix, and its residual equal to the oracle's
     recomputation within 1e-6.
 """
+import math
+
 import numpy as np
 import pytest
 
@@ -301,3 +303,26 @@ def test_lanczos_from_a_nan(mods, dtype):
     alpha, beta, V = krylov.lanczos(D, v0, 2, keep_basis=True)
     assert np.isnan(alpha).all() and np.isnan(beta[1:]).all()
     assert bool(torch.isnan(V[1]).all())
+
+
+def _diagonal(pjds, d, dtype):
+    n = len(d)
+    A = synth.Crs(n, n, np.arange(n + 1, dtype=np.int64), np.arange(n, dtype=np.int32), np.asarray(d, np.float64))
+    return _dev(pjds, A, dtype)[0]  # rows of one length: the sort keeps their order
+
+
+# sums whose terms differ much in size are rounded to nearest at every level: a warp's, a CTA's and all CTAs' sums
+# of one large term and many small negative ones, each below half of the large one's last bit (rounded down, 31 of
+# them would take 4 of its last bits)
+@pytest.mark.parametrize("n", [32, 250, 4096, 70_001])
+@pytest.mark.parametrize("small", [2.0 ** -54, 2.0 ** -58, 2.0 ** -70, 2.0 ** -300])
+def test_fp64_sums_of_terms_of_mixed_size(mods, n, small):
+    torch, pjds, krylov = mods
+    d = np.full(n, -small / n)
+    d[n // 2] = 1.0
+    alpha, _, V = krylov.lanczos(_diagonal(pjds, d, "f64"), torch.ones(n, dtype=torch.float64, device="cuda"), 1,
+                                 keep_basis=True)
+    v = V[0].cpu().numpy()
+    terms = v * (d * v)
+    # a few roundings of the sum itself at 2^-53 and of a warp's and the CTAs' terms below that
+    assert abs(alpha[0] - math.fsum(terms)) <= 2 * 2.0 ** -53 * math.fsum(np.abs(terms))
