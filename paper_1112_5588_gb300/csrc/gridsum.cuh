@@ -73,6 +73,16 @@ __device__ __forceinline__ Fixed fixed_of(double v) {
   return a;
 }
 
+// of a finite float, without the fp64 pipe
+__device__ __forceinline__ Fixed fixed_of(float v) {
+  const uint32_t b = __float_as_uint(v), k = (b >> 23) & 0xffu, m = (b & 0x7fffffu) | (k ? 0x800000u : 0u);
+  Fixed a;
+  a.f = (long long)m << 33;
+  if ((int32_t)b < 0) a.f = -a.f;
+  a.e = m ? max(k, 1u) + 896u : 1u;
+  return a;
+}
+
 __device__ __forceinline__ double double_of(const Fixed &a) {
   if (a.e == 0x7ffu) return __longlong_as_double(a.f);
   if (a.f == 0) return 0.0;

@@ -42,38 +42,74 @@ enum { F_ALPHA = 0, F_BETA, F_RR, F_NORM, F_LALPHA, F_LBETA, F_STORE };
 // Whether fp32 holds a product p and its rounding error, and sums of some of them.
 __device__ __forceinline__ bool in_range(float p) { return fabsf(p) >= 0x1p-96f && fabsf(p) <= 0x1p100f; }
 
-__device__ __noinline__ double far_product(float a, float b, double c) { return __fma_rn((double)a, (double)b, c); }
+// a + b as its rounded sum, and what the rounding left out added to err (Knuth, "The Art of Computer
+// Programming", vol. 2, 4.2.2; exact whatever the operands' sizes).
+__device__ __forceinline__ float two_sum(float a, float b, float &err) {
+  const float t = __fadd_rn(a, b), z = __fsub_rn(t, a);
+  err = __fadd_rn(__fsub_rn(a, __fsub_rn(t, z)), __fsub_rn(b, z));
+  return t;
+}
 
 // Running inner product of one thread. Vectors of floats: products and sums in
-// twice the working precision (Ogita, Rump, Oishi, "Accurate sum and dot
-// product", 2005, Dot2: error-free products and sums in fp32, their errors added
-// up beside), since an fp64 multiply-add and its conversions take 16 cycles of
-// the SM's fp64 pipe a warp: with them the two inner products of a CG step on
-// 2M rows alone take 20 us.
+// three times the working precision (Ogita, Rump, Oishi, "Accurate sum and dot
+// product", 2005, DotK with K = 3: error-free products and sums in fp32, their
+// errors added up the same way, and the errors of that beside), as an fp64
+// multiply-add and its conversions take 16 cycles of the SM's fp64 pipe a warp:
+// with them the two inner products of a CG step on 2M rows alone take 20 us. A
+// thread adds at most KEEP products (launch_dot). What is lost is the rounding of
+// the last part: of the sum P of KEEP products' magnitudes, the second part's 2 KEEP
+// terms are at most 2^-24 P each, their errors 2 KEEP 2^-48 P each, and the 4 KEEP
+// roundings in the sum of those below 16 KEEP^3 2^-72 P = 2^-53 P, against KEEP 2^-53
+// P for multiply-adds in fp64. A thread with a product outside that range takes all
+// of its products again, in fp64, after its loop (again(); with fp64 products inside
+// the loop the product kernel took 3 us longer).
+constexpr int KEEP = 32;
 template <typename TX>
 struct Dot;
 template <>
 struct Dot<double> {
   double s = 0.0;
   __device__ __forceinline__ void add(double a, double b) { s = __fma_rn(a, b, s); }
-  __device__ __forceinline__ double value() const { return s; }
+  template <typename F>
+  __device__ __forceinline__ Fixed warp(F) const {
+    const Fixed a[1] = {fixed_of(s)};
+    return warp_sum<1>(a);
+  }
 };
 template <>
 struct Dot<float> {
-  float s = 0.0f, c = 0.0f;
-  double far = 0.0;  // products too small or too large for an error-free fp32 product
+  float s = 0.0f, c = 0.0f, l = 0.0f;
+  bool far = false;  // a product too small or too large (or a NaN, as 0 times an infinity)
   __device__ __forceinline__ void add(float a, float b) {
     const float p = __fmul_rn(a, b);
-    if (in_range(p)) {
-      const float e = __fmaf_rn(a, b, -p), t = __fadd_rn(s, p), z = __fsub_rn(t, s);
-      c = __fadd_rn(c, __fadd_rn(e, __fadd_rn(__fsub_rn(s, __fsub_rn(t, z)), __fsub_rn(p, z))));
-      s = t;
-    } else if (p != 0.0f || (a != 0.0f && b != 0.0f)) {  // (also a NaN: 0 times an infinity)
-      far = far_product(a, b, far);
-    }
+    far = far || !(in_range(p) || (p == 0.0f && (a == 0.0f || b == 0.0f)));
+    float q, r, t;
+    s = two_sum(s, p, q);
+    c = two_sum(c, q, r);
+    c = two_sum(c, __fmaf_rn(a, b, -p), t);
+    l = __fadd_rn(l, __fadd_rn(r, t));
   }
-  __device__ __forceinline__ double value() const { return ((double)s + (double)c) + far; }
+  template <typename F>
+  __device__ __forceinline__ Fixed warp(F again) const {
+    Fixed a[3] = {fixed_of(s), fixed_of(c), fixed_of(l)};
+    if (far) a[0] = fixed_of(again()), a[1] = a[2] = Fixed{0, 1};
+    return warp_sum<3>(a);
+  }
 };
+
+// sum of a_i b_i in fp64 over the elements i0 + q stride + r below n, q from 0 to most - 1, r from 0 to width - 1
+__device__ __forceinline__ double products(const float *a, const float *b, int64_t i0, int64_t stride, int width, int most,
+                                           int64_t n) {
+  double d = 0.0;
+#pragma unroll 1
+  for (; i0 < n && most > 0; i0 += stride, --most)
+#pragma unroll 1
+    for (int64_t i = i0; i < min(i0 + width, n); ++i) d = __fma_rn((double)a[i], (double)b[i], d);
+  return d;
+}
+__device__ __forceinline__ double products(const double *, const double *, int64_t, int64_t, int, int, int64_t) {
+  return 0.0;  // (Dot<double> does not ask)
+}
 
 // Where a reduction's result goes: the scalar block and the update.
 struct Fin {
@@ -144,11 +180,11 @@ __device__ __forceinline__ void apply_op(double v, const Fin &f) {
 // reduce_kernel, the next launch, adds the slots. With an arrival counter, and so
 // a gpu-scope fence, in every CTA the product on 2M rows took 123 us in place of
 // 112 (a fence holds up the SM's other CTAs).
-__device__ __forceinline__ void store_partial(double v, double *partial) {
+template <typename TX, typename F>
+__device__ __forceinline__ void store_partial(const Dot<TX> &dot, double *partial, F again) {
   __shared__ Fixed sh[KT / 32];
   const int w = threadIdx.x >> 5, l = threadIdx.x & 31;
-  const Fixed a[1] = {fixed_of(v)};
-  const Fixed s = warp_sum<1>(a);
+  const Fixed s = dot.warp(again);
   if (l == 0) sh[w] = s;
   __syncthreads();
   if (w != 0) return;
@@ -282,13 +318,17 @@ __global__ void __launch_bounds__(KT)
     }
     y[i] = yi;
   }
-  store_partial(dot.value(), partial);
+  store_partial(dot, partial, [&] {
+    return products(MODE == 0 ? x : y, y, (int64_t)blockIdx.x * KT + threadIdx.x, (int64_t)gridDim.x * KT, 1, KEEP, n_rows);
+  });
 }
 
 // y = A x and the reduction of sum x_i y_i with two adjacent rows per thread
-// (row pair p: rows 2p, 2p+1; the second is a padding row when n_rows is odd)
+// (row pair p: rows 2p, 2p+1; the second is a padding row when n_rows is odd).
+// Six CTAs on an SM, 40 registers: five, 48, are up to 4% faster on half a million
+// to a million rows and up to 4% slower from 1.3M on.
 template <typename TV, typename TX, typename IDX>
-__global__ void __launch_bounds__(KT)
+__global__ void __launch_bounds__(KT, 6)
     spmv_dot2_kernel(const void *__restrict__ val_, const int32_t *__restrict__ col,
                      const int64_t *__restrict__ col_start, const int32_t *__restrict__ block_len,
                      const TX *__restrict__ x, TX *__restrict__ y, const TX *__restrict__ bv,
@@ -308,7 +348,9 @@ __global__ void __launch_bounds__(KT)
         y[i + r] = yi;
       }
   }
-  store_partial(dot.value(), partial);
+  store_partial(dot, partial, [&] {
+    return products(x, y, 2 * ((int64_t)blockIdx.x * KT + threadIdx.x), 2 * (int64_t)gridDim.x * KT, 2, KEEP, n_rows);
+  });
 }
 
 // 16-byte groups of workspace vectors (the workspace is 256-byte aligned):
@@ -343,6 +385,16 @@ __device__ __forceinline__ void groups(int32_t n, FL load, FU use, FT tail) {
   for (int q = 0; q < VG; ++q)
     if (k + q * KT < ng) use(q, (k + q * KT) * W);
   if (blockIdx.x == 0 && threadIdx.x < n - ng * W) tail(ng * W + threadIdx.x);
+}
+
+// sum of v_e^2 over this thread's elements of groups()
+template <typename TX>
+__device__ __forceinline__ double squares(const TX *v, int32_t n) {
+  constexpr int W = G16<TX>::W;
+  const int64_t whole = n / W * W;
+  double d = products(v, v, ((int64_t)blockIdx.x * (VG * KT) + threadIdx.x) * W, (int64_t)KT * W, W, VG, whole);
+  if (blockIdx.x == 0) d += products(v, v, whole + threadIdx.x, 1, 1, 1, n);
+  return d;
 }
 
 template <typename TX>
@@ -380,7 +432,7 @@ __global__ void __launch_bounds__(KT)
         r[i] = ri;
         dot.add(ri, ri);
       });
-  store_partial(dot.value(), partial);
+  store_partial(dot, partial, [&] { return squares(r, n); });
 }
 
 // d += alpha p (here, where p is read anyway), p = r + beta p.
@@ -431,7 +483,7 @@ __global__ void __launch_bounds__(KT)
     d[i] = TL(0);
     dot.add(ri, ri);
   }
-  store_partial(dot.value(), partial);
+  store_partial(dot, partial, [&] { return products(r, r, i, 1, 1, 1, n); });
 }
 
 // x += ||r64|| d (fp64)
@@ -449,7 +501,7 @@ __global__ void __launch_bounds__(KT) sumsq_kernel(const TX *v, double *partial,
   Dot<TX> dot;
   const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
   if (i < n) dot.add(v[i], v[i]);
-  store_partial(dot.value(), partial);
+  store_partial(dot, partial, [&] { return products(v, v, i, 1, 1, 1, n); });
 }
 
 // v = v0 / ||v0||
@@ -554,7 +606,7 @@ __global__ void __launch_bounds__(KT)
         w[i] = x;
         dot.add(x, x);
       });
-  store_partial(dot.value(), partial);
+  store_partial(dot, partial, [&] { return squares(w, n); });
 }
 
 // v = w / beta_{j+1}: the next vector, in its row of the basis if there is one.
@@ -587,15 +639,15 @@ __global__ void __launch_bounds__(KT)
     ritz_combine_kernel(const TB *basis, const double *s, int32_t k, int32_t n,
                         double *y, double *partial) {
   begin();
-  double contrib = 0.0;
+  Dot<double> dot;
   const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
   if (i < n) {
     double acc = 0.0;
     for (int32_t j = 0; j < k; ++j) acc = fma(s[j], (double)__ldcs(basis + (int64_t)j * n + i), acc);
     y[i] = acc;
-    contrib = acc * acc;
+    dot.add(acc, acc);
   }
-  store_partial(contrib, partial);
+  store_partial(dot, partial, [] { return 0.0; });
 }
 
 // reduces sum (w_i - theta y_i)^2 with theta = scal[S_AUX1] / scal[S_AUX0]
@@ -604,13 +656,13 @@ __global__ void __launch_bounds__(KT)
                          double *partial, int32_t n) {
   begin();
   const double theta = scal[S_AUX1] / scal[S_AUX0];
-  double contrib = 0.0;
+  Dot<double> dot;
   const int64_t i = (int64_t)blockIdx.x * KT + threadIdx.x;
   if (i < n) {
     const double e = w[i] - theta * y[i];
-    contrib = e * e;
+    dot.add(e, e);
   }
-  store_partial(contrib, partial);
+  store_partial(dot, partial, [] { return 0.0; });
 }
 
 // ----------------------------------------------------------------------------- host helpers
@@ -739,7 +791,9 @@ template <typename TX, int MODE>
 static void launch_dot(const DotKernel<TX, MODE> &d, const pjds_dev *A, const typename Same<TX>::type *x,
                        typename Same<TX>::type *y, const typename Same<TX>::type *bv, const Reduce &red, cudaStream_t s,
                        int32_t op, int32_t j = 0, double *out = nullptr) {
-  const int64_t grid = std::min<int64_t>(((int64_t)A->n_rows + d.rows - 1) / d.rows, d.resident);
+  // no more CTAs than fit at once, but no more rows of a thread than KEEP (from 7.5M rows on in fp32)
+  const int64_t all = ((int64_t)A->n_rows + d.rows - 1) / d.rows;
+  const int64_t grid = std::min<int64_t>(all, std::max<int64_t>(d.resident, (all * (d.rows / KT) + KEEP - 1) / KEEP));
   launch<false>(d.fn, grid, KT, s, A->val, A->col, A->col_start, A->block_len, x, y, bv, red.partial, A->n_rows, A->b);
   red.sum(grid, s, op, j, out);
 }

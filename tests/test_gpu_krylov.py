@@ -326,3 +326,21 @@ def test_fp64_sums_of_terms_of_mixed_size(mods, n, small):
     terms = v * (d * v)
     # a few roundings of the sum itself at 2^-53 and of a warp's and the CTAs' terms below that
     assert abs(alpha[0] - math.fsum(terms)) <= 2 * 2.0 ** -53 * math.fsum(np.abs(terms))
+
+
+# fp32 inner products are as good as sums in fp64: alpha = (v, A v) of a diagonal A, whose elements v_i (d_i v_i)
+# are known to the last bit. Few rows (two products a thread, where a sum in twice fp32's precision alone errs by
+# up to 2^-48 of the terms) and so many that a thread adds more than it keeps before it moves the sum to fp64
+@pytest.mark.parametrize("n,runs", [(2, 200), (7, 100), (700, 20), (9_000_001, 1)])
+def test_fp32_inner_products_keep_fp64_sums(mods, n, runs):
+    torch, pjds, krylov = mods
+    for seed in range(runs):
+        rng = np.random.default_rng(seed)
+        d = (rng.uniform(0.5, 1.5, n) * np.where(rng.random(n) < 0.5, -1, 1)).astype(np.float32)
+        v0 = torch.from_numpy(rng.uniform(-1, 1, n).astype(np.float32)).cuda()
+        alpha, _, V = krylov.lanczos(_diagonal(pjds, d, "f32"), v0, 1, keep_basis=True)
+        v = V[0].cpu().numpy()
+        terms = v.astype(np.float64) * (d * v).astype(np.float64)  # exact: 48 bits
+        # roundings: a thread's three floats to a double, its warp's, CTA's and the launch's sums, each within
+        # a few 2^-53 of the terms
+        assert abs(alpha[0] - math.fsum(terms)) <= 8 * 2.0 ** -53 * math.fsum(np.abs(terms)), seed
