@@ -515,13 +515,20 @@ __global__ void __launch_bounds__(KT)
 
 // The fp64 arithmetic of the Lanczos vectors, for floats without the fp64 pipe
 // (six conversions and multiply-adds an element took 20 us a step on 1M rows):
-// error-free products and sums in fp32, rounded once at the end, as good as the
-// fp64 expression to 2^-45 before that rounding; fp64 outside the range where
-// fp32 holds the products' errors.
+// error-free products and sums in fp32 give r, the result rounded once, and d, what
+// that rounding left out, within a bound E that covers their own errors and those of
+// the fp64 expression. Where r + d - E and r + d + E both round to r, so does the
+// fp64 expression; else (a few elements in 2^16 and those outside the range where
+// fp32 holds the products' errors) it is evaluated. So the vectors are those of the
+// fp64 arithmetic, bit for bit.
 // (not inlined, so that the fp64 operations are not speculated on every element)
 __device__ __noinline__ float far_times(float w, double a) { return (float)((double)w * a); }
 __device__ __noinline__ float far_orth(float w, double a, float v, double b, float p) {
   return (float)((double)w - a * (double)v - b * (double)p);
+}
+// whether every value within E of r + d rounds to r
+__device__ __forceinline__ bool certain(float r, float d, float E) {
+  return __fadd_rn(r, __fadd_rn(d, E)) == r && __fadd_rn(r, __fsub_rn(d, E)) == r;
 }
 template <typename TX>
 struct Coef;
@@ -540,22 +547,31 @@ struct Coef<float> {
   const double *wide;
   float2 h;
   __device__ __forceinline__ Coef(const double *w, const double *two)
-      : wide(w), h(*reinterpret_cast<const float2 *>(two)) {}
-  __device__ __forceinline__ float times(float w) const {
-    const float p = __fmul_rn(w, h.x);
-    if (!in_range(p)) return far_times(w, *wide);
-    return __fadd_rn(p, __fmaf_rn(w, h.y, __fmaf_rn(w, h.x, -p)));
+      : wide(w), h(*reinterpret_cast<const float2 *>(two)) {
+    // a lower half that fp32 does not hold to 2^-48 of the whole: no product is then in range
+    if (h.x != 0.0f && fabsf(h.x) < 0x1p-100f) h.x = __int_as_float(0x7fffffff);
   }
+  // errors: fma(w, h.y, e) 2^-47 of p, the halves of the factor 2^-48, the sum in certain() 2^-48, the fp64
+  // product 2^-53
+  __device__ __forceinline__ float times(float w) const {
+    const float p = __fmul_rn(w, h.x), c = __fmaf_rn(w, h.y, __fmaf_rn(w, h.x, -p)), r = __fadd_rn(p, c);
+    if ((p == 0.0f && w == 0.0f) ||
+        (in_range(p) && certain(r, __fadd_rn(__fsub_rn(p, r), c), 0x1p-45f * fabsf(p))))
+      return r;
+    return far_times(w, *wide);
+  }
+  // errors: ex 1.5 2^-47 of x, ey of y, et + eu 2^-47 of the sum M of the magnitudes, ex + ey 2^-47, their difference
+  // 2^-46, the sum in certain() 2^-48, the fp64 expression 2^-52: below 2^-44.4 M
   __device__ __forceinline__ static float orth(float w, const Coef &a, float v, const Coef &b, float p) {
     const float x = __fmul_rn(a.h.x, v), y = __fmul_rn(b.h.x, p);
-    if (!((x == 0.0f && v == 0.0f) || in_range(x)) || !((y == 0.0f && p == 0.0f) || in_range(y)) ||
-        !(w == 0.0f || in_range(w)))
-      return far_orth(w, *a.wide, v, *b.wide, p);
     const float ex = __fmaf_rn(a.h.y, v, __fmaf_rn(a.h.x, v, -x)), ey = __fmaf_rn(b.h.y, p, __fmaf_rn(b.h.x, p, -y));
-    // w - x = t + et, t - y = u + eu
-    const float t = __fsub_rn(w, x), zt = __fsub_rn(t, w), et = __fsub_rn(__fsub_rn(w, __fsub_rn(t, zt)), __fadd_rn(x, zt));
-    const float u = __fsub_rn(t, y), zu = __fsub_rn(u, t), eu = __fsub_rn(__fsub_rn(t, __fsub_rn(u, zu)), __fadd_rn(y, zu));
-    return __fadd_rn(u, __fsub_rn(__fadd_rn(et, eu), __fadd_rn(ex, ey)));
+    float et, eu, d;
+    const float t = two_sum(w, -x, et), u = two_sum(t, -y, eu);
+    const float r = two_sum(u, __fsub_rn(__fadd_rn(et, eu), __fadd_rn(ex, ey)), d);
+    if (((x == 0.0f && v == 0.0f) || in_range(x)) && ((y == 0.0f && p == 0.0f) || in_range(y)) &&
+        (w == 0.0f || in_range(w)) && certain(r, d, 0x1p-44f * (fabsf(w) + fabsf(x) + fabsf(y))))
+      return r;
+    return far_orth(w, *a.wide, v, *b.wide, p);
   }
 };
 

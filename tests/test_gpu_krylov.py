@@ -344,3 +344,26 @@ def test_fp32_inner_products_keep_fp64_sums(mods, n, runs):
         # roundings: a thread's three floats to a double, its warp's, CTA's and the launch's sums, each within
         # a few 2^-53 of the terms
         assert abs(alpha[0] - math.fsum(terms)) <= 8 * 2.0 ** -53 * math.fsum(np.abs(terms)), seed
+
+
+# the Lanczos vectors of floats are the fp64 expressions rounded once, also where that rounding is decided by the
+# last bits: with a diagonal A every element can be computed again (scaled, 1 / beta is near the end of fp32's range)
+@pytest.mark.parametrize("scale", [1.0, 2.0 ** 112])
+def test_fp32_lanczos_vectors_are_rounded_once(mods, scale):
+    torch, pjds, krylov = mods
+    n = 4_200_001
+    g = torch.Generator("cuda").manual_seed(5)
+    d = (torch.rand(n, generator=g, device="cuda") + 0.5) * scale
+    v0 = torch.rand(n, generator=g, device="cuda") - 0.5
+    steps = 4
+    alpha, beta, V = krylov.lanczos(_diagonal(pjds, d.cpu().numpy(), "f32"), v0, steps, keep_basis=True)
+    off = 0
+    for j in range(steps - 1):
+        w = (d * V[j]).double() - alpha[j] * V[j].double()
+        if j:
+            w -= beta[j] * V[j - 1].double()
+        nxt = (w.float().double() * (1.0 / beta[j + 1])).float()
+        off += int((nxt != V[j + 1]).sum())
+    # torch rounds the two products of the first expression, the kernel does not: that can decide about 2^-26 of
+    # the 12.6 million roundings (a difference of 2^-52 of the terms at a boundary of 2^-24)
+    assert off <= 1
