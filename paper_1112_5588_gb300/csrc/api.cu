@@ -3,6 +3,7 @@
 #include <stdint.h>
 
 #include "common.h"
+#include "cooperative.h"
 #include "spmv_launch.cuh"
 
 namespace pjds {
@@ -244,6 +245,11 @@ extern "C" int pjds_check_word(uint64_t *word, int32_t clear, void *stream) {
   for (int k = 0; k < 4 && !*word; ++k) *word = w[k];
   return PJDS_OK;
 }
+
+#ifdef PJDS_CHECKED
+int pjds::g_cooperative_limit = -1;
+extern "C" void pjds_checked_cooperative_limit(int32_t ctas) { pjds::g_cooperative_limit = ctas; }
+#endif
 
 extern "C" int pjds_wait_selftest(int32_t which, void *stream) {
   clear_error();

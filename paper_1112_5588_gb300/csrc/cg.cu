@@ -137,13 +137,14 @@ __global__ void __launch_bounds__(SOLVER_THREADS, 1) cg_kernel(const __grid_cons
 }
 
 template <typename TV, typename TL, int T>
-static int launch(const SolverShape &p, CgArgs<TL> &a, cudaStream_t s) {
-  return p.tile ? launch_solver(cg_kernel<TV, TL, T, true>, p, a, s)
-                : launch_solver(cg_kernel<TV, TL, T, false>, p, a, s);
+static int launch(const SolverShape &p, CgArgs<TL> &a, bool *fits, cudaStream_t s) {
+  return p.tile ? launch_solver(cg_kernel<TV, TL, T, true>, p, a, fits, s)
+                : launch_solver(cg_kernel<TV, TL, T, false>, p, a, fits, s);
 }
 
 template <typename TV, typename TL>
-static int run(const pjds_dev *Ah, const pjds_dev *Al, const CgSystem &c, const SolverShape &p, cudaStream_t s) {
+static int run(const pjds_dev *Ah, const pjds_dev *Al, const CgSystem &c, const SolverShape &p, bool *fits,
+               cudaStream_t s) {
   CgArgs<TL> a;
   a.hi = mat_of(Ah), a.lo = mat_of(Al);
   a.b = c.b, a.x = c.x, a.r64 = c.r64;
@@ -152,9 +153,9 @@ static int run(const pjds_dev *Ah, const pjds_dev *Al, const CgSystem &c, const 
   a.n = Ah->n_rows, a.max_outer = c.max_outer, a.inner = c.inner, a.tol = c.tol;
   a.n_max = Al->n_max;
   switch (p.T) {
-    case 4: return launch<TV, TL, 4>(p, a, s);
-    case 2: return launch<TV, TL, 2>(p, a, s);
-    default: return launch<TV, TL, 1>(p, a, s);
+    case 4: return launch<TV, TL, 4>(p, a, fits, s);
+    case 2: return launch<TV, TL, 2>(p, a, fits, s);
+    default: return launch<TV, TL, 1>(p, a, fits, s);
   }
 }
 
@@ -168,14 +169,13 @@ int cg_small(const pjds_dev *Ah, const pjds_dev *Al, const CgSystem &c, bool *ta
   if (e != cudaSuccess) return set_error(PJDS_ECUDA, "device query: %s", cudaGetErrorString(e));
   const SolverShape p = solver_shape(Al, 4, vector_bytes(Al->dtype), sms);
   if (!solver_takes(p, Ah->n_rows, sms)) return PJDS_OK;
-  *taken = true;
   e = cudaMemsetAsync(c.out, 0, sizeof(CgOut), s);
   if (e == cudaSuccess) e = cudaMemsetAsync(c.slots, 0, sizeof(GridSlots), s);
   if (e != cudaSuccess) return set_error(PJDS_ECUDA, "cg: %s", cudaGetErrorString(e));
-  int rc = Al->dtype == PJDS_F64   ? run<double, double>(Ah, Al, c, p, s)
-           : Al->dtype == PJDS_F32 ? run<float, float>(Ah, Al, c, p, s)
-                                   : run<dev::bf16_t, float>(Ah, Al, c, p, s);
-  if (rc) return rc;
+  int rc = Al->dtype == PJDS_F64   ? run<double, double>(Ah, Al, c, p, taken, s)
+           : Al->dtype == PJDS_F32 ? run<float, float>(Ah, Al, c, p, taken, s)
+                                   : run<dev::bf16_t, float>(Ah, Al, c, p, taken, s);
+  if (rc || !*taken) return rc;
   CgOut h;
   unsigned long long error = 0;
   e = cudaMemcpyAsync(&h, c.out, sizeof(h), cudaMemcpyDeviceToHost, s);

@@ -31,8 +31,8 @@ struct CgSystem {
 
 size_t cg_slots_bytes();
 
-// The whole solve in one cooperative launch, if the system is small enough for
-// it (*taken); waits for the stream.
+// The whole solve in one cooperative launch, if the system is small enough for it
+// and the context holds all its CTAs at once (*taken); waits for the stream then.
 int cg_small(const pjds_dev *Ah, const pjds_dev *Al, const CgSystem &c, bool *taken, cudaStream_t s);
 
 }  // namespace kry

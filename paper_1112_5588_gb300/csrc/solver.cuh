@@ -13,6 +13,7 @@
 #include <algorithm>
 
 #include "common.h"
+#include "cooperative.h"
 #include "gridsum.cuh"
 #include "spmv_kernels.cuh"
 
@@ -220,16 +221,18 @@ inline SolverShape solver_shape(const pjds_dev *A, int vectors, int vec_bytes, i
 inline bool solver_takes(const SolverShape &p, int32_t n, int sms) { return p.tile || n <= sms * SOLVER_THREADS; }
 
 // Launch a solver kernel; all its CTAs are resident, as they wait for one another.
+// *fits: false where the context does not hold so many (it may be limited to some
+// of the SMs); nothing ran then.
 template <typename Args>
-int launch_solver(void (*kernel)(const Args), const SolverShape &p, Args &a, cudaStream_t s) {
+int launch_solver(void (*kernel)(const Args), const SolverShape &p, Args &a, bool *fits, cudaStream_t s) {
   void *args[] = {&a};
   cudaError_t e = cudaSuccess;
   if (p.smem > 40 * 1024)
     e = cudaFuncSetAttribute((const void *)kernel, cudaFuncAttributeMaxDynamicSharedMemorySize, SOLVER_SMEM);
   if (e == cudaSuccess)
-    e = cudaLaunchCooperativeKernel((const void *)kernel, dim3((unsigned)p.grid), dim3((unsigned)p.threads), args,
-                                    p.smem, s);
-  return e == cudaSuccess ? PJDS_OK : set_error(PJDS_ECUDA, "solver launch: %s", cudaGetErrorString(e));
+    e = launch_cooperative((const void *)kernel, (unsigned)p.grid, (unsigned)p.threads, args, p.smem, s);
+  *fits = e != cudaErrorCooperativeLaunchTooLarge;
+  return e == cudaSuccess || !*fits ? PJDS_OK : set_error(PJDS_ECUDA, "solver launch: %s", cudaGetErrorString(e));
 }
 
 }  // namespace kry

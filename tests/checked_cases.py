@@ -14,6 +14,9 @@ the stored entries, a block longer than the longest row; also in the block
 product's launch for long rows) must be recorded with its code and skipped:
 the kernels check each index before the access.
 
+Refused: cooperative launches of more CTAs than a limit are refused, as in a
+context of fewer SMs: their callers' other way must give the same results.
+
 Prints one JSON line.
 """
 import json
@@ -225,6 +228,27 @@ def main():
         batch.spmm(D, torch.rand(Z.n_cols, 4, dtype=torch.float64, device="cuda"), Y)
         torch.cuda.synchronize()
         res["planted"][name] = [[{}, *split(pjds.pjds_check_word(clear=True))]]
+    # cooperative launches of more CTAs than a limit refused (0: all, -1: none): small CG systems
+    from paper_1112_5588_gb300 import krylov
+    from tests.test_gpu_krylov import _spd
+    S = _spd("tri", 4097)
+    rhs = synth.vector(S.n_rows, seed=3)
+    low = {dt: pjds.pjds_create(S.n_rows, S.n_cols, S.row_ptr, S.col, S.val, b=32, dtype=dt, permute_cols=True)
+           for dt in ("f64", "f32", "bf16")}
+    perm = low["f64"].perm.copy()
+    low = {dt: H.to_device("cuda") for dt, H in low.items()}
+    bp = torch.from_numpy(rhs[perm]).cuda()
+    res["refused_cg"] = []
+    for limit in (0, 8, -1):
+        pjds._lib.pjds_checked_cooperative_limit(limit)
+        for dt in low:
+            xp = torch.zeros_like(bp)
+            out = krylov.cg_solve(low["f64"], None if dt == "f64" else low[dt], bp, xp, max_outer=12, inner_iters=20,
+                                  tol=1e-13)
+            xs = np.empty(S.n_rows)
+            xs[perm] = xp.cpu().numpy()
+            rel = float(np.linalg.norm(rhs - oracle.crs_spmv(S, xs)) / np.linalg.norm(rhs))
+            res["refused_cg"].append([dt, limit, max(rel, out["rel_residual"]), out["outer"]])
     print(json.dumps(res))
 
 

@@ -75,3 +75,11 @@ def test_long_rows_of_a_block_product_are_checked(res):
         assert (code, idx) == (COLUMN, n["n_cols"] + 13), (code, idx)
     for cfg, code, idx in res["planted"]["long_block"]:
         assert (code == DIAG and idx >= n["n_max"] + 1) or (code == OFFSET and idx >= n["n_stored"]), (code, idx)
+
+
+def test_solves_where_cooperative_launches_are_refused(res):
+    # a context that does not hold a launch's CTAs at once (here: a limit of the checked build): the solve in
+    # launches of its own, to the same residual (kappa below 5, as in test_gpu_krylov.py)
+    assert {tuple(c[:2]) for c in res["refused_cg"]} == {(lo, lim) for lo in ("f64", "f32", "bf16") for lim in (0, 8, -1)}
+    for lo, limit, rel, outer in res["refused_cg"]:
+        assert rel <= 1e-12 and outer >= 1, (lo, limit, rel)
