@@ -18,6 +18,7 @@
 #include <vector>
 
 #include "common.h"
+#include "cooperative.h"
 #include "gridsum.cuh"
 #include "pjds_mlp.h"
 #include "pjds_tune.h"
@@ -523,7 +524,7 @@ extern "C" int pjds_mlp_train(pjds_mlp *m, const float *X, const float *y, int32
   const int32_t steps = (int32_t)(((int64_t)n + bsz - 1) / bsz);
   // CTAs: one on each SM as far as there are tiles (of all samples: the losses
   // need them too; a step's tiles may be fewer)
-  const int32_t grid = (int32_t)std::min<int64_t>(((int64_t)n + TS - 1) / TS, std::min(sms, MAX_CTAS));
+  int32_t grid = (int32_t)std::min<int64_t>(((int64_t)n + TS - 1) / TS, std::min(sms, MAX_CTAS));
   // the next epoch's order is drawn while an epoch runs, into the other buffer
   std::vector<int32_t> order[2];
   std::vector<float2> c[2];
@@ -559,7 +560,11 @@ extern "C" int pjds_mlp_train(pjds_mlp *m, const float *X, const float *y, int32
     if (e != cudaSuccess) return set_error(PJDS_ECUDA, "mlp epoch upload: %s", cudaGetErrorString(e));
     a.loss = loss_hist ? w.out + kept : nullptr;
     void *args[] = {&a};
-    e = cudaLaunchCooperativeKernel((const void *)train_kernel, dim3((unsigned)grid), dim3(NT), args, sizeof(Sm), s);
+    e = launch_cooperative((const void *)train_kernel, (unsigned)grid, NT, args, sizeof(Sm), s);
+    while (e == cudaErrorCooperativeLaunchTooLarge && grid > 1) {  // (a context limited to some of the SMs)
+      grid /= 2;
+      e = launch_cooperative((const void *)train_kernel, (unsigned)grid, NT, args, sizeof(Sm), s);
+    }
     if (e != cudaSuccess) return set_error(PJDS_ECUDA, "mlp training launch: %s", cudaGetErrorString(e));
     a.arrived += 2u * (uint32_t)steps * (uint32_t)grid;
     a.sums += loss_hist ? 1u : 0u;

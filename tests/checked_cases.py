@@ -249,6 +249,23 @@ def main():
             xs[perm] = xp.cpu().numpy()
             rel = float(np.linalg.norm(rhs - oracle.crs_spmv(S, xs)) / np.linalg.norm(rhs))
             res["refused_cg"].append([dt, limit, max(rel, out["rel_residual"]), out["outer"]])
+    # and an epoch of the tuner's training, on fewer CTAs then
+    from paper_1112_5588_gb300 import learned
+    rng = np.random.default_rng(9)
+    X = rng.standard_normal((2500, 15)).astype(np.float32)
+    t = (np.sin(X[:, 0]) + 0.5 * X[:, 1] * X[:, 2] - X[:, 3]).astype(np.float32)
+    res["refused_train"] = []
+    for limit in (-1, 1, 40):
+        pjds._lib.pjds_checked_cooperative_limit(limit)
+        m = learned.init(4)
+        hist = learned.train(m, X, t, epochs=3, batch=700, lr=1e-3, seed=2)
+        res["refused_train"].append([limit, [float(v) for v in hist], [float(v) for v in m.w2]])
+    pjds._lib.pjds_checked_cooperative_limit(0)
+    try:
+        learned.train(learned.init(4), X, t, epochs=1, batch=700, lr=1e-3)
+        res["refused_train_error"] = 0
+    except pjds.PjdsError as err:
+        res["refused_train_error"] = err.code
     print(json.dumps(res))
 
 

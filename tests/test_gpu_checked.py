@@ -83,3 +83,14 @@ def test_solves_where_cooperative_launches_are_refused(res):
     assert {tuple(c[:2]) for c in res["refused_cg"]} == {(lo, lim) for lo in ("f64", "f32", "bf16") for lim in (0, 8, -1)}
     for lo, limit, rel, outer in res["refused_cg"]:
         assert rel <= 1e-12 and outer >= 1, (lo, limit, rel)
+
+
+def test_training_where_cooperative_launches_are_refused(res):
+    # the same epochs on fewer CTAs: a gradient is the same terms added in another order (1e-6 of it), which Adam
+    # turns into at most lr = 1e-3 a step where a gradient is at its rounding, on the mean far less (12 steps)
+    (_, want, w), *others = res["refused_train"]
+    assert [c[0] for c in others] == [1, 40]
+    for limit, hist, v in others:
+        assert hist == pytest.approx(want, rel=2e-3), limit
+        assert sum(abs(a - b) for a, b in zip(v, w)) / len(w) <= 2e-5, limit
+    assert res["refused_train_error"] == -3  # no launch at all: PJDS_ECUDA
