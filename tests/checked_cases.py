@@ -135,17 +135,40 @@ def main():
         res["clean"].append(["batch", "f64", 32, kw.get("lanes") and "lanes" or kw.get("rule") and "rule" or "default",
                              w, ok])
 
-    # paired rows (block-structured, 2^18 rows of 64: pair_share 1000): the
-    # single product (two rows per thread), the paired block product and its
-    # pattern product
-    Pm = synth.block_dense(70_000, 4, 16, 0.05, seed=67)
-    lens = np.diff(Pm.row_ptr)
-    for dt, k in (("f32", 8), ("bf16", 16)):
+    # a batch of more tiles than CTAs (the work counter; the one above has a CTA for every tile)
+    many = [tiny.from_lengths(np.full(130_001, 17), 5_000, seed=1), mats["ragged"], mats["hmep"]]
+    for dt in ("f64", "f32", "bf16"):
+        devs = [pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dt).to_device("cuda")
+                for A in many]
+        xs = [torch.from_numpy(synth.vector(A.n_cols, seed=65)).to("cuda", D.vec_dtype) for A, D in zip(many, devs)]
+        ys = [torch.full((A.n_rows,), float("nan"), dtype=D.vec_dtype, device="cuda") for A, D in zip(many, devs)]
+        B = batch.Batch(devs, xs, ys)
+        assert B.info()["n_tiles"] > B.info()["n_ctas"]
+        B.run(use_graph=False)
+        torch.cuda.synchronize()
+        w = pjds.pjds_check_word(clear=True)
+        ok = all(bool(torch.isfinite(y).all()) for y in ys)
+        if dt == "f64":
+            ok = ok and all(parity.check_fp64(y.cpu().numpy(), oracle.crs_spmv(A, xv.cpu().numpy()),
+                                              oracle.crs_absmv(A, xv.cpu().numpy()), np.diff(A.row_ptr))["ok"]
+                            for A, xv, y in zip(many, xs, ys))
+        B.destroy()
+        res["clean"].append(["batch", dt, 32, "counter", w, ok])
+
+    # rows sharing their columns (2^18 rows of 64 or more: pair_share 1000), in 4x4 blocks and in blocks of 2: the
+    # single product (two rows per thread), the block product with four rows per thread ("quad") and, where the
+    # rows share in twos only, with two ("paired"), and their pattern products
+    from tests.test_gpu_batch import _block_rows
+    shared = {"quad": synth.block_dense(70_000, 4, 16, 0.05, seed=67),
+              "paired": _block_rows(262_147, 60_000, 2, 34, 0.01, seed=5)}
+    for name, dt, k in (("quad", "f32", 8), ("quad", "bf16", 16), ("paired", "f32", 8), ("paired", "bf16", 16)):
+        Pm = shared[name]
+        lens = np.diff(Pm.row_ptr)
         D = pjds.pjds_create(Pm.n_rows, Pm.n_cols, Pm.row_ptr, Pm.col, Pm.val, b=32, dtype=dt).to_device("cuda")
         assert D.pair_share >= 500 and pjds.pjds_spmv_resolve(D)["rows_per_thread"] == 2
         xt = torch.from_numpy(synth.vector(Pm.n_cols, seed=68)).to("cuda", D.vec_dtype)
         y = run(D, xt, {})
-        res["clean"].append(["paired", dt, 32, "spmv", pjds.pjds_check_word(clear=True), bool(torch.isfinite(y).all())])
+        res["clean"].append([name, dt, 32, "spmv", pjds.pjds_check_word(clear=True), bool(torch.isfinite(y).all())])
         X = np.stack([synth.vector(Pm.n_cols, seed=80 + c) for c in range(k)], axis=1).astype(np.float32)
         Xt = torch.from_numpy(np.ascontiguousarray(X)).cuda()
         for fn, tag in ((batch.spmm, "spmm"), (batch.spmm_pattern, "spmm_pattern")):
@@ -160,15 +183,16 @@ def main():
                 Yr, S = oracle.crs_spmm(Ar, Xd), oracle.crs_spmm(Ar._replace(val=np.abs(Ar.val)), np.abs(Xd))
                 Yg = Y.double().cpu().numpy()
                 ok = ok and all(parity.check_fp32(Yg[:, c], Yr[:, c], S[:, c], lens)["ok"] for c in (0, k - 1))
-            res["clean"].append(["paired", dt, 32, f"{tag} k={k}", w, ok])
-    # a column beyond n_cols in the paired block product: recorded and skipped
-    D = pjds.pjds_create(Pm.n_rows, Pm.n_cols, Pm.row_ptr, Pm.col, Pm.val, b=32, dtype="f32").to_device("cuda")
-    D.col[1] = Pm.n_cols + 11
-    Y = torch.empty(Pm.n_rows, 8, device="cuda")
-    batch.spmm(D, torch.rand(Pm.n_cols, 8, device="cuda"), Y)
-    torch.cuda.synchronize()
-    res["planted"]["paired_column"] = [[{}, *split(pjds.pjds_check_word(clear=True))]]
-    res["paired_n_cols"] = Pm.n_cols
+            res["clean"].append([name, dt, 32, f"{tag} k={k}", w, ok])
+    # a column beyond n_cols in them: recorded and skipped
+    for name, Pm in shared.items():
+        D = pjds.pjds_create(Pm.n_rows, Pm.n_cols, Pm.row_ptr, Pm.col, Pm.val, b=32, dtype="f32").to_device("cuda")
+        D.col[1] = Pm.n_cols + 11
+        Y = torch.empty(Pm.n_rows, 8, device="cuda")
+        batch.spmm(D, torch.rand(Pm.n_cols, 8, device="cuda"), Y)
+        torch.cuda.synchronize()
+        res["planted"][name + "_column"] = [[{}, *split(pjds.pjds_check_word(clear=True))]]
+        res[name + "_n_cols"] = Pm.n_cols
 
     # planted indices (fp64, original basis)
     A = mats["ragged"]

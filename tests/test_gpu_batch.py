@@ -358,8 +358,8 @@ def test_spmm_in_fours_in_a_captured_graph(mods):
 
 
 # block products launched while the one before runs, each on what that one has
-# written (one row, pairs, fours and the fall back from fours), in a row on a
-# stream and in a graph: bit for bit the products one by one
+# written (one row, fours and the fall back from fours; pairs: test_spmm_pairs), in
+# a row on a stream and in a graph: bit for bit the products one by one
 @pytest.mark.parametrize("dtype,k,bs,nb", [("f64", 2, 4, 5), ("f32", 4, 2, 8), ("bf16", 8, 2, 8), ("f32", 32, 4, 5),
                                            ("f32", 32, 2, 10), ("bf16", 32, 6, 4)])
 def test_spmm_one_after_another(mods, dtype, k, bs, nb):
@@ -515,3 +515,89 @@ def test_block_products_back_and_forth(mods, name, dtype, k):
     with torch.cuda.graph(graph):
         run()
     check(graph.replay)
+
+
+# two rows per thread (from 2^18 rows of 64 entries on): block rows of 2 and 6, which share no fours, so that
+# spmm_quad_kernel leaves the work to spmm_pair_kernel, an odd number of rows and rows with a column of their own,
+# every depth and width of a round, columns bit for bit the single products; products on one another's results, in
+# a row on a stream and in a graph
+@pytest.mark.parametrize("dtype,k,bs,nb", [("f32", 8, 2, 34), ("f32", 64, 6, 12), ("bf16", 8, 6, 12), ("bf16", 32, 2, 34)])
+def test_spmm_pairs(mods, dtype, k, bs, nb):
+    torch, pjds, batch = mods
+    A = _block_rows(262_147, 262_147 // bs // 2, bs, nb, 0.01, seed=k + bs)
+    assert A.nnz >= 64 * A.n_rows
+    A = A._replace(val=A.val / (bs * nb))
+    D = pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
+    assert D.pair_share >= 900
+    g = torch.Generator("cuda").manual_seed(k)
+    X = torch.rand(A.n_rows, k, device="cuda", generator=g) * 2 - 1
+    Y, P, Z = (torch.full((A.n_rows, k), float("nan"), device="cuda") for _ in range(3))
+    batch.spmm(D, X[:A.n_cols], Y)
+    batch.spmm_pattern(D, X[:A.n_cols], P)
+    y1, p1 = (torch.empty(A.n_rows, device="cuda") for _ in range(2))
+    for c in (0, 3, k - 1):
+        x = X[:A.n_cols, c].contiguous()
+        pjds.pjds_spmv_cfg(D, x, y1, threads_per_row=1, rows_per_thread=1)
+        pjds.pjds_spmv_pattern(D, x, p1, threads_per_row=1, rows_per_thread=1)
+        assert torch.equal(y1, Y[:, c].contiguous()) and torch.equal(p1, P[:, c].contiguous()), c
+    batch.spmm(D, Y[:A.n_cols], Z)
+    torch.cuda.synchronize()
+    a, b = X.clone(), torch.empty_like(X)
+    graph = torch.cuda.CUDAGraph()
+    with torch.cuda.graph(graph):
+        batch.spmm(D, a[:A.n_cols], b)
+        batch.spmm(D, b[:A.n_cols], a)
+    for go in (lambda: (batch.spmm(D, a[:A.n_cols], b), batch.spmm(D, b[:A.n_cols], a)), graph.replay):
+        a.copy_(X), b.fill_(float("nan"))
+        go()
+        torch.cuda.synchronize()
+        assert torch.equal(b, Y) and torch.equal(a, Z)
+
+
+# lanes of two chunks of one row on a matrix whose rows share nothing (spmm_kernel; on block matrices the fp32 and
+# bf16 products of test_spmm_two_chunk_lanes take four rows per thread)
+@pytest.mark.parametrize("dtype,k", [("f32", 64), ("bf16", 64), ("f64", 32)])
+def test_spmm_two_chunk_lanes_of_single_rows(mods, dtype, k):
+    torch, pjds, batch = mods
+    A = tiny.from_lengths(np.tile([20, 19, 21, 3], 18_000)[:70_001], 30_000, seed=3)
+    D = pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
+    assert D.pair_share < 500
+    X = torch.rand(A.n_cols, k, device="cuda", dtype=D.vec_dtype) * 2 - 1
+    Y, P = (torch.full((A.n_rows, k), float("nan"), dtype=D.vec_dtype, device="cuda") for _ in range(2))
+    batch.spmm(D, X, Y)
+    batch.spmm_pattern(D, X, P)
+    y1, p1 = (torch.empty(A.n_rows, dtype=D.vec_dtype, device="cuda") for _ in range(2))
+    for c in range(k):
+        x = X[:, c].contiguous()
+        pjds.pjds_spmv_cfg(D, x, y1, threads_per_row=1, rows_per_thread=1)
+        pjds.pjds_spmv_pattern(D, x, p1, threads_per_row=1, rows_per_thread=1)
+        assert torch.equal(y1, Y[:, c].contiguous()) and torch.equal(p1, P[:, c].contiguous()), c
+
+
+# batches of more tiles than CTAs, whose CTAs take tiles from the counter (all other batches of these tests are
+# small): direct, by graph and as pattern, twice each, in the three value types, bit for bit the single products of
+# the same plan
+@pytest.mark.parametrize("dtype", ["f64", "f32", "bf16"])
+def test_batches_of_more_tiles_than_ctas(mods, dtype):
+    torch, pjds, batch = mods
+    mats = [tiny.from_lengths(np.full(130_001, 17), 5_000, seed=1), synth.zipf_rows(200_003, s=1.8, len_max=400, seed=2),
+            tiny.random_lengths(1037, 1037, max_len=90, seed=3, p_empty=0.2)]
+    devs = [pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
+            for A in mats]
+    xs = [torch.from_numpy(synth.vector(A.n_cols, seed=4)).to("cuda", D.vec_dtype) for A, D in zip(mats, devs)]
+    ys = [torch.empty(A.n_rows, dtype=D.vec_dtype, device="cuda") for A, D in zip(mats, devs)]
+    want, ones = [torch.empty_like(y) for y in ys], [torch.empty_like(y) for y in ys]
+    for D, x, y, p in zip(devs, xs, want, ones):
+        pjds.pjds_spmv_cfg(D, x, y, plan=1)
+        pjds.pjds_spmv_pattern(D, x, p, plan=1)
+    B = batch.Batch(devs, xs, ys)
+    assert B.info()["n_tiles"] > B.info()["n_ctas"]
+    for go, expect in ((lambda: B.run(use_graph=False), want), (lambda: B.run(use_graph=True), want),
+                       (B.run_pattern, ones)):
+        for _ in range(2):
+            for y in ys:
+                y.fill_(float("nan"))
+            go()
+            torch.cuda.synchronize()
+            assert all(torch.equal(y, w) for y, w in zip(ys, expect))
+    B.destroy()

@@ -121,6 +121,42 @@ def test_permute_spmm_batch_write_only_their_outputs(mods):
         B.destroy()
 
 
+def test_block_products_of_several_kernels_write_only_y(mods):
+    # long rows in one launch and before the others, four rows per thread, the fall back from it and pairs
+    from tests.test_gpu_batch import _block_rows
+    torch, pjds, batch, krylov = mods
+    spread = lambda n: tiny.from_lengths(np.minimum(np.random.default_rng(2).zipf(1.9, size=n), 300), 9001, seed=6)
+    for A, dtype, k in ((spread(5_003), "f64", 2), (spread(66_001), "f32", 128), (spread(66_001), "f64", 64),
+                        (_block_rows(32_771, 9_000, 4, 5, 0.02, 1), "f32", 32),
+                        (_block_rows(32_771, 9_000, 2, 10, 0.02, 2), "bf16", 32),
+                        (_block_rows(262_147, 60_000, 2, 34, 0.02, 3), "f32", 8)):
+        D = pjds.pjds_create(A.n_rows, A.n_cols, A.row_ptr, A.col, A.val, b=32, dtype=dtype).to_device("cuda")
+        X = torch.rand(A.n_cols, k, device="cuda", dtype=D.vec_dtype)
+        for fn in (batch.spmm, batch.spmm_pattern):
+            raw, flat = guarded(torch, A.n_rows * k, D.vec_dtype)
+            fn(D, X, flat.view(A.n_rows, k))
+            torch.cuda.synchronize()
+            assert intact(torch, raw, A.n_rows * k, D.vec_dtype), (A.n_rows, dtype, k)
+            assert torch.isfinite(flat.float()).all()
+
+
+def test_batches_of_more_tiles_than_ctas_write_only_y(mods):
+    torch, pjds, batch, krylov = mods
+    mats = [tiny.from_lengths(np.full(130_001, 17), 5_000, seed=1), MATS[0](), MATS[1]()]
+    for dtype in ("f64", "f32", "bf16"):
+        devs = [pjds.pjds_create(M.n_rows, M.n_cols, M.row_ptr, M.col, M.val, b=32, dtype=dtype).to_device("cuda")
+                for M in mats]
+        xs = [torch.rand(M.n_cols, device="cuda", dtype=D.vec_dtype) for M, D in zip(mats, devs)]
+        guards = [guarded(torch, M.n_rows, D.vec_dtype) for M, D in zip(mats, devs)]
+        B = batch.Batch(devs, xs, [g[1] for g in guards])
+        assert B.info()["n_tiles"] > B.info()["n_ctas"]
+        for go in (lambda: B.run(use_graph=False), lambda: B.run(use_graph=True), B.run_pattern):
+            go()
+            torch.cuda.synchronize()
+            assert all(intact(torch, raw, M.n_rows, D.vec_dtype) for (raw, _), M, D in zip(guards, mats, devs))
+        B.destroy()
+
+
 def test_krylov_workspaces_and_outputs_stay_in_bounds(mods):
     torch, pjds, batch, krylov = mods
     S = synth.stencil27(g=13, seed=84)  # 2197 rows (odd)
@@ -137,6 +173,21 @@ def test_krylov_workspaces_and_outputs_stay_in_bounds(mods):
         krylov.cg_solve(D64, lo, b, x, max_outer=2, inner_iters=10, work=work)
         torch.cuda.synchronize()
         assert intact(torch, wraw, need, torch.uint8) and intact(torch, xraw, S.n_rows, torch.float64)
+    # a system too large for the one launch (more than 512 rows per SM, and a row too long for shared memory), odd
+    from tests.test_gpu_krylov import _spd
+    n = 512 * torch.cuda.get_device_properties(0).multi_processor_count + 177
+    A = _spd("arrow", n)
+    hi, lo32 = (pjds.pjds_create(n, n, A.row_ptr, A.col, A.val, dtype=dt, permute_cols=True).to_device("cuda")
+                for dt in ("f64", "f32"))
+    rhs = torch.rand(n, device="cuda", dtype=torch.float64)
+    for lo, vec in ((None, 0), (lo32, 1)):
+        need = krylov.cg_workspace_bytes(n, hi.n_pad, vec)
+        wraw, work = guarded(torch, need, torch.uint8)
+        xraw, x = guarded(torch, n, torch.float64)
+        x.zero_()
+        krylov.cg_solve(hi, lo, rhs, x, max_outer=2, inner_iters=10, work=work)
+        torch.cuda.synchronize()
+        assert intact(torch, wraw, need, torch.uint8) and intact(torch, xraw, n, torch.float64)
     steps = 12
     for D in (D64, D32):
         need = ctypes.c_size_t()

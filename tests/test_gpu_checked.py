@@ -62,11 +62,12 @@ def test_planted_block_length_is_recorded(res):
         assert (code == DIAG and idx >= n["n_max"] + 1) or (code == OFFSET and idx >= n["n_stored"]), (cfg, code, idx)
 
 
-def test_paired_block_product_column_is_recorded(res):
-    # the block product with one thread per pair of rows checks both rows' columns
-    for cfg, code, idx in res["planted"]["paired_column"]:
-        assert (code, idx) == (COLUMN, res["paired_n_cols"] + 11), (cfg, code, idx)
-    assert any(c[0] == "paired" for c in res["clean"])
+@pytest.mark.parametrize("name", ["quad", "paired"])
+def test_column_is_recorded_where_rows_share_theirs(res, name):
+    # the block product with four and with two rows per thread checks every row's columns
+    for cfg, code, idx in res["planted"][name + "_column"]:
+        assert (code, idx) == (COLUMN, res[name + "_n_cols"] + 11), (cfg, code, idx)
+    assert any(c[0] == name for c in res["clean"])
 
 
 def test_long_rows_of_a_block_product_are_checked(res):

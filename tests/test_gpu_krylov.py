@@ -74,7 +74,8 @@ def test_cg_matches_fp64_oracle(mods, oracle_lib, stencil, lo, max_outer, inner,
     assert h[0] == pytest.approx(1.0) and h[-1] < 1e-12
 
 
-def test_cg_is_deterministic_and_graph_equals_direct(mods, stencil):
+def test_cg_is_deterministic(mods, stencil):
+    # also with use_graph, which is accepted and changes nothing
     torch, pjds, krylov = mods
     A = stencil
     b = synth.vector(A.n_rows, seed=5)
@@ -121,7 +122,8 @@ def test_lanczos_fp64_matches_oracle(mods, oracle_lib):
     assert np.allclose(Vh @ Vh.T, np.eye(10), atol=1e-10)
 
 
-def test_lanczos_graph_equals_direct(mods):
+def test_lanczos_is_deterministic(mods):
+    # also with use_graph, which is accepted and changes nothing
     torch, pjds, krylov = mods
     A = synth.stencil27(g=12, seed=4)
     D, perm = _dev(pjds, A, "f32")
@@ -235,6 +237,28 @@ def test_cg_small_and_large_systems(mods, oracle_lib, name, n, lo, max_outer):
     assert rel <= 1e-12, (rel, res)
     assert res["rel_residual"] <= 1e-12 and res["inner_total"] == 20 * res["outer"]
     assert len(res["history"]) == res["outer"] + 1 and res["history"][-1] == res["rel_residual"]
+
+
+# more rows than the one launch takes (512 per SM; the arrow's long row keeps the matrix out of shared memory) with
+# every remainder of the vector kernels' 16-byte groups: a launch for every step, to the fp64 residual, twice the
+# same bits
+@pytest.mark.parametrize("lo,max_outer", [(None, 3), ("f32", 6), ("bf16", 12)])
+@pytest.mark.parametrize("more", [1, 178, 1027])
+def test_cg_larger_than_one_launch(mods, oracle_lib, more, lo, max_outer):
+    torch, pjds, krylov = mods
+    n = 512 * torch.cuda.get_device_properties(0).multi_processor_count + more
+    A = _spd("arrow", n)
+    b = synth.vector(n, seed=more)
+    D64, perm = _dev(pjds, A, "f64")
+    Dlo = _dev(pjds, A, lo)[0] if lo else None
+    bp = torch.from_numpy(b[perm]).cuda()
+    xs = [torch.zeros_like(bp) for _ in range(2)]
+    for xp in xs:
+        res = krylov.cg_solve(D64, Dlo, bp, xp, max_outer=max_outer, inner_iters=20, tol=1e-13)
+    assert torch.equal(*xs)
+    x = np.empty(n)
+    x[perm] = xs[0].cpu().numpy()
+    assert max(_true_rel_residual(oracle_lib, A, x, b), res["rel_residual"]) <= 1e-12  # (as above)
 
 
 # vectors far outside the range in which fp32 holds a product and its rounding
