@@ -54,7 +54,7 @@ int pjds_mlp_init(pjds_mlp *m, uint64_t seed);
  * matrices, feat[n][8] (host): per feature the smallest and largest value. */
 int pjds_mlp_fit_range(pjds_mlp *m, const float *feat, int32_t n);
 
-/* Set the model's standardisation from n samples X[n][13], y[n] (host):
+/* Set the model's standardisation from n samples X[n][15], y[n] (host):
  * population mean and standard deviation per column (1 where it is 0). */
 int pjds_mlp_fit_scaling(pjds_mlp *m, const float *X, const float *y, int32_t n);
 
@@ -63,7 +63,7 @@ int pjds_mlp_fit_scaling(pjds_mlp *m, const float *X, const float *y, int32_t n)
 int pjds_mlp_workspace_bytes(int32_t n, int32_t batch, size_t *bytes);
 
 /*
- * Train in place: X[n][13], y[n] on the host (raw, standardised on upload
+ * Train in place: X[n][15], y[n] on the host (raw, standardised on upload
  * with m's statistics), `epochs` passes of mini-batches of `batch` samples
  * (batch >= n: full batch, no shuffling; otherwise each epoch uses a
  * permutation drawn from a counter-based generator seeded with `seed`),
@@ -74,7 +74,7 @@ int pjds_mlp_workspace_bytes(int32_t n, int32_t batch, size_t *bytes);
 int pjds_mlp_train(pjds_mlp *m, const float *X, const float *y, int32_t n, int32_t epochs, int32_t batch, float lr,
                    uint64_t seed, float *loss_hist, void *work, size_t work_bytes, void *stream);
 
-/* Predictions (unstandardised) for n host inputs X[n][13] into out[n] (host). */
+/* Predictions (unstandardised) for n host inputs X[n][15] into out[n] (host). */
 int pjds_mlp_predict(const pjds_mlp *m, const float *X, int32_t n, float *out, void *work, size_t work_bytes,
                      void *stream);
 

@@ -8,10 +8,10 @@
 // so a run of inner iterations has no host round trip. Its launches follow one
 // another by programmatic dependent launch; no graph is recorded (a step takes
 // longer than its five launches, and a graph of 24 Lanczos steps took 0.3 ms to
-// record). Inner products accumulate in fp64 or, for vectors of floats, in twice
-// their precision: per-CTA partial sums into the workspace, which a launch of one
-// CTA adds in fixed point before it applies the scalar update. The sums depend on
-// the number of CTAs alone, so results are bitwise reproducible.
+// record). Inner products accumulate in fp64 or, for vectors of floats, in three
+// floats that are as good: per-CTA partial sums into the workspace, which a launch of
+// one CTA adds before it applies the scalar update. The sums depend on the number of
+// CTAs alone, so results are bitwise reproducible.
 #include <float.h>
 #include <math.h>
 #include <string.h>
@@ -124,9 +124,8 @@ struct Fin {
 // read-only path may be moved ahead of that wait, so no pointer in those kernels
 // is __restrict__. The products, which gather through it, are launched after the
 // kernel before them has ended.
-__device__ __forceinline__ void let_next_start() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 __device__ __forceinline__ void begin() {
-  let_next_start();
+  dev::let_next_start();
   asm volatile("griddepcontrol.wait;" ::: "memory");
 }
 
@@ -300,7 +299,7 @@ __global__ void __launch_bounds__(KT)
                     const int64_t *__restrict__ col_start, const int32_t *__restrict__ block_len,
                     const TX *__restrict__ x, TX *__restrict__ y, const TX *__restrict__ bv,
                     double *__restrict__ partial, int32_t n_rows, int32_t b) {
-  let_next_start();
+  dev::let_next_start();
   const TV *__restrict__ val = static_cast<const TV *>(val_);
   Dot<TX> dot;
   // rows in sorted order: the tile traversal table measured 1.7% slower here
@@ -333,7 +332,7 @@ __global__ void __launch_bounds__(KT, 6)
                      const int64_t *__restrict__ col_start, const int32_t *__restrict__ block_len,
                      const TX *__restrict__ x, TX *__restrict__ y, const TX *__restrict__ bv,
                      double *__restrict__ partial, int32_t n_rows, int32_t b) {
-  let_next_start();
+  dev::let_next_start();
   const TV *__restrict__ val = static_cast<const TV *>(val_);
   Dot<TX> dot;
   for (int64_t i = 2 * ((int64_t)blockIdx.x * KT + threadIdx.x); i < n_rows; i += 2 * (int64_t)gridDim.x * KT) {
@@ -764,22 +763,6 @@ struct Same {
   using type = T;
 };
 
-// Launch with programmatic dependence on the kernel before (see begin()), or
-// after its end.
-template <bool EARLY = true, typename... P, typename... A>
-static void launch(void (*kernel)(P...), int64_t grid, int threads, cudaStream_t s, A... args) {
-  cudaLaunchAttribute at{};
-  at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-  at.val.programmaticStreamSerializationAllowed = 1;
-  cudaLaunchConfig_t c{};
-  c.gridDim = dim3((unsigned)grid);
-  c.blockDim = dim3((unsigned)threads);
-  c.stream = s;
-  c.attrs = &at;
-  c.numAttrs = EARLY ? 1 : 0;
-  cudaLaunchKernelEx(&c, kernel, static_cast<P>(args)...);
-}
-
 // What the reductions need in a workspace, before its vectors: partial sums and
 // the scalar block.
 struct Reduce {
@@ -797,7 +780,7 @@ struct Reduce {
   }
   // add the n partial sums of the kernel before
   void sum(int64_t n, cudaStream_t s, int32_t op, int32_t j = 0, double *out = nullptr) const {
-    launch(reduce_kernel, 1, RT, s, partial, (int32_t)n, Fin{scal, out, op, j});
+    dev::launch_early(reduce_kernel, 1, RT, s, partial, (int32_t)n, Fin{scal, out, op, j});
   }
 };
 
@@ -810,7 +793,7 @@ static void launch_dot(const DotKernel<TX, MODE> &d, const pjds_dev *A, const ty
   // no more CTAs than fit at once, but no more rows of a thread than KEEP (from 7.5M rows on in fp32)
   const int64_t all = ((int64_t)A->n_rows + d.rows - 1) / d.rows;
   const int64_t grid = std::min<int64_t>(all, std::max<int64_t>(d.resident, (all * (d.rows / KT) + KEEP - 1) / KEEP));
-  launch<false>(d.fn, grid, KT, s, A->val, A->col, A->col_start, A->block_len, x, y, bv, red.partial, A->n_rows, A->b);
+  d.fn<<<(unsigned)grid, KT, 0, s>>>(A->val, A->col, A->col_start, A->block_len, x, y, bv, red.partial, A->n_rows, A->b);
   red.sum(grid, s, op, j, out);
 }
 
@@ -848,7 +831,7 @@ static int cg_run(const pjds_dev *Ah, const pjds_dev *Al, const double *b, doubl
   int rc;
   if ((rc = make_dot(Al, &dot_lo)) || (rc = make_dot(Ah, &dot_res)) || (rc = red.clear(s))) return rc;
   // ||b||
-  launch(sumsq_kernel<double>, nb, KT, s, b, red.partial, n);
+  dev::launch_early(sumsq_kernel<double>, nb, KT, s, b, red.partial, n);
   red.sum(nb, s, F_STORE, S_AUX2);
   double bn2 = 0.0;
   if ((rc = launch_check("cg ||b||"))) return rc;
@@ -874,15 +857,15 @@ static int cg_run(const pjds_dev *Ah, const pjds_dev *Al, const double *b, doubl
     rel = bnorm > 0.0 ? rn / bnorm : rn;
     if (out.n_history < PJDS_CG_HISTORY) out.history[out.n_history++] = rel;
     if (outer >= o.max_outer || rel <= o.tol || rn == 0.0) break;
-    launch(ir_start_kernel<TL>, nb, KT, s, r64, r, p, d, scal, red.partial, n);
+    dev::launch_early(ir_start_kernel<TL>, nb, KT, s, r64, r, p, d, scal, red.partial, n);
     red.sum(nb, s, F_RR);
     for (int it = 0; it < o.inner_iters; ++it) {
       launch_dot(dot_lo, Al, p, q, nullptr, red, s, F_ALPHA);                   // q = A p, (p, q), alpha
-      launch(cg_update_kernel<TL>, g_vec, KT, s, r, q, scal, red.partial, n);  // r, (r, r), beta
+      dev::launch_early(cg_update_kernel<TL>, g_vec, KT, s, r, q, scal, red.partial, n);  // r, (r, r), beta
       red.sum(g_vec, s, F_BETA);
-      launch(cg_dir_kernel<TL>, g_vec, KT, s, d, p, r, scal, n);  // d, p
+      dev::launch_early(cg_dir_kernel<TL>, g_vec, KT, s, d, p, r, scal, n);  // d, p
     }
-    launch(ir_correct_kernel<TL>, nb, KT, s, x, d, scal, n);
+    dev::launch_early(ir_correct_kernel<TL>, nb, KT, s, x, d, scal, n);
     if ((rc = launch_check("cg inner"))) break;
     out.outer = outer + 1;
     out.inner_total += o.inner_iters;
@@ -957,15 +940,15 @@ static int lanczos_run(const pjds_dev *A, const TX *v0, int32_t steps, double *a
   const int32_t g_vec = group_grid<TX>(n);
   // v_j: its row of the caller's basis, else the two buffers in turn
   auto vec = [&](int32_t j) { return basis ? basis + (int64_t)j * n : buf[j & 1]; };
-  launch(sumsq_kernel<TX>, nb, KT, s, v0, red.partial, n);
+  dev::launch_early(sumsq_kernel<TX>, nb, KT, s, v0, red.partial, n);
   red.sum(nb, s, F_NORM);
-  launch(lanczos_start_kernel<TX>, nb, KT, s, v0, vec(0), red.scal, n);
+  dev::launch_early(lanczos_start_kernel<TX>, nb, KT, s, v0, vec(0), red.scal, n);
   for (int32_t j = 0; j < steps; ++j) {
     TX *const v = vec(j);
     launch_dot(dot, A, v, w, nullptr, red, s, F_LALPHA, j, alpha);  // w = A v, alpha_j = (v, w)
-    launch(lanczos_orth_kernel<TX>, g_vec, KT, s, w, v, j > 0 ? vec(j - 1) : nullptr, red.scal, red.partial, j, n);
+    dev::launch_early(lanczos_orth_kernel<TX>, g_vec, KT, s, w, v, j > 0 ? vec(j - 1) : nullptr, red.scal, red.partial, j, n);
     red.sum(g_vec, s, F_LBETA, j + 1, beta);  // beta_j+1
-    if (j + 1 < steps) launch(lanczos_next_kernel<TX>, g_vec, KT, s, vec(j + 1), w, red.scal, n);
+    if (j + 1 < steps) dev::launch_early(lanczos_next_kernel<TX>, g_vec, KT, s, vec(j + 1), w, red.scal, n);
   }
   if ((rc = launch_check("lanczos steps"))) return rc;
   e = cudaMemcpyAsync(alpha_h, alpha, sizeof(double) * (size_t)steps, cudaMemcpyDeviceToHost, s);
@@ -1143,12 +1126,12 @@ extern "C" int pjds_ritz_refine(const pjds_dev *A_hi, const void *basis, int32_t
   cudaError_t e = cudaMemcpyAsync(sd, s_host, sizeof(double) * (size_t)k, cudaMemcpyHostToDevice, st);
   if (e != cudaSuccess) return set_error(PJDS_ECUDA, "ritz: %s", cudaGetErrorString(e));
   if (basis_dtype == PJDS_F64)
-    launch(ritz_combine_kernel<double>, nb, KT, st, static_cast<const double *>(basis), sd, k, n, y, red.partial);
+    dev::launch_early(ritz_combine_kernel<double>, nb, KT, st, static_cast<const double *>(basis), sd, k, n, y, red.partial);
   else
-    launch(ritz_combine_kernel<float>, nb, KT, st, static_cast<const float *>(basis), sd, k, n, y, red.partial);
+    dev::launch_early(ritz_combine_kernel<float>, nb, KT, st, static_cast<const float *>(basis), sd, k, n, y, red.partial);
   red.sum(nb, st, F_STORE, S_AUX0);
   launch_dot(dot, A_hi, y, w, nullptr, red, st, F_STORE, S_AUX1);  // w = A y, (y, w)
-  launch(ritz_residual_kernel, nb, KT, st, w, y, red.scal, red.partial, n);
+  dev::launch_early(ritz_residual_kernel, nb, KT, st, w, y, red.scal, red.partial, n);
   red.sum(nb, st, F_STORE, S_AUX2);
   if ((rc = launch_check("ritz refine"))) return rc;
   double h[3];

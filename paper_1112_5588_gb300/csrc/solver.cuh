@@ -1,6 +1,6 @@
-// Solver kernels that run a whole solve in one cooperative launch, for systems
-// small enough that a step's kernels are bound by latency: cg_kernel (cg.cu)
-// and lanczos_kernel (lanczos.cu). The CTAs keep their rows for the whole run:
+// Parts of a solver kernel that runs a whole solve in one cooperative launch, for
+// systems small enough that a step's kernels are bound by latency (cg_kernel,
+// cg.cu). The CTAs keep their rows for the whole run:
 // every vector but those that the next product gathers stays in shared memory,
 // and the step's scalars reach all CTAs through grid-wide sums (gridsum.cuh),
 // so nothing is launched, recorded or read back per step.
@@ -183,7 +183,6 @@ inline size_t tile_bytes(int64_t units, int64_t ur, int64_t n_max, int value_byt
 
 struct SolverShape {
   int32_t T, grid, threads;
-  int64_t units;  // of a CTA, at most
   size_t smem;    // of the vectors, and of the matrix if tile
   bool tile;      // the matrix is in shared memory
 };
@@ -197,13 +196,12 @@ struct SolverShape {
 inline SolverShape solver_shape(const pjds_dev *A, int vectors, int vec_bytes, int sms) {
   const int32_t n = A->n_rows;
   const double mean = (double)A->nnz / n;
-  SolverShape p{1, 1, 32, 0, 0, false};
+  SolverShape p{1, 1, 32, 0, false};
   while (p.T < 4 && (int64_t)n * p.T * 2 <= (int64_t)sms * SOLVER_THREADS && mean >= 2.0 * p.T) p.T *= 2;
   const int64_t ur = 32 / p.T, units = (n + ur - 1) / ur;
   p.grid = (int32_t)std::min<int64_t>(std::min(sms, GS_MAX_CTAS), std::max<int64_t>(1, (units + 3) / 4));
   const int64_t per = (units + p.grid - 1) / p.grid;
   p.threads = 32 * (int32_t)std::min<int64_t>(SOLVER_THREADS / 32, std::max<int64_t>(per, 4));
-  p.units = per;
   p.smem = (size_t)((per * ur * vectors * vec_bytes + 15) / 16 * 16);
   const size_t tile = tile_bytes(per, ur, A->n_max, value_bytes(A->dtype));
   if (p.smem + tile <= SOLVER_SMEM) {
@@ -217,7 +215,10 @@ inline SolverShape solver_shape(const pjds_dev *A, int vectors, int vec_bytes, i
 // memory, else up to one row per thread. Beyond, the launches of krylov.cu keep
 // more loads in flight (27-point stencil, fp32 CG of 300 steps from global
 // memory: 64,000 rows 5.7 against 7.5 ms, 125,000 rows 8.6 against 7.8, 216,000
-// rows 11.8 against 9.0).
+// rows 11.8 against 9.0). Short rows fit up to several times as many (CG of 200
+// steps, one launch / a launch for every step: rows of 3 entries fp32 100,000 rows
+// 2.0 / 3.4 ms, 300,000 2.5 / 3.8, 800,000 4.2 / 5.4, fp64 300,000 rows 4.0 / 4.3;
+// rows of 7 fp32 300,000 rows 2.7 / 3.9, fp64 200,000 rows 3.2 / 4.3).
 inline bool solver_takes(const SolverShape &p, int32_t n, int sms) { return p.tile || n <= sms * SOLVER_THREADS; }
 
 // Launch a solver kernel; all its CTAs are resident, as they wait for one another.

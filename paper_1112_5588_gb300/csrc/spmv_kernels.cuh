@@ -189,9 +189,9 @@ __device__ __forceinline__ TX gather(const TX *__restrict__ x, int32_t c) {
   return c >= 0 ? __ldg(x + c) : TX(0);
 }
 
-// Programmatic dependent launch: about 2 us a product less in a row of them, of any
-// length (27-point stencil 1M rows fp32 39.2 -> 37.1 us, HMEp-like 300k rows fp32
-// 18.5 -> 16.5, 6.2M rows fp64 279 -> 276.5, Zipf 1M rows fp64 33.3 -> 31.3). A kernel that
+// Programmatic dependent launch: about 2 us a product less in a row of them (27-point
+// stencil 1M rows fp32 39.2 -> 37.1 us, HMEp-like 300k rows fp32 18.5 -> 16.5; on
+// products of more than 200 us less than their spread). A kernel that
 // is launched with it may be placed on the SMs when every CTA of the kernel before
 // has called let_next_start() or ended, and waits in after_previous() until that
 // kernel is completed and visible; so its launch is over by then. The kernel

@@ -80,8 +80,8 @@ def cg_solve_static(A_hi, A_lo, b: torch.Tensor, x: torch.Tensor, max_outer: int
                     tol: float = 0.0, stream=None) -> dict:
     """pjds_cg_solve_static: the same solve as cg_solve, for callers that
     cannot allocate device memory; the library's static device workspace
-    (at most 131072 rows) is used instead of a caller workspace, and the
-    no stream or CUDA graph is created."""
+    (at most 131072 rows) is used instead of a caller workspace, and no
+    stream or CUDA graph is created."""
     for t, nm in ((b, "b"), (x, "x")):
         _p._check_vec(t, A_hi.n_rows, torch.float64, nm)
     o = _CgOpts(max_outer, inner_iters, tol, 0, 0)
