@@ -37,7 +37,8 @@ extern "C" {
  * (6 and 50: 300 inner steps). use_graph is accepted and changes nothing: a small
  * system (one whose inner matrix fits in the SMs' shared memory, about 125,000
  * rows of 24 fp32 entries, or one of at most 512 rows per SM) is solved by one
- * cooperative launch, a larger one by launches of its own for every step. */
+ * cooperative launch of a CTA per SM, a larger one, or any one in a context that
+ * does not hold that launch, by launches of its own for every step. */
 typedef struct pjds_cg_opts {
   int32_t max_outer;
   int32_t inner_iters;

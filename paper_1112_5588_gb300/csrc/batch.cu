@@ -397,7 +397,8 @@ __device__ __forceinline__ void shared_rows(const TV *__restrict__ val, const in
 // 5.2 GB gathered with one row per thread) and their latency. Times on that
 // matrix, before (one row or one pair per thread) and now: fp32 k = 8 / 16 / 32 /
 // 64 / 128 104 / 173 / 330 / 660 / 1260 us, now 95 / 115 / 200 / 326 / 617; bf16
-// values 101 / 150 / 240 / 480 / 912, now 93 / 111 / 195 / 328 / 662.
+// values 101 / 150 / 240 / 480 / 912, now 93 / 111 / 195 / 328 / 662 (and 1 to 5 us
+// for the launch that it would fall back to).
 // U jagged diagonals a round and MB CTAs per SM: 4 and 2 while the launch has
 // fewer than 2^18 threads (k = 16: 115 us against 146 with 2 and 3), else 2 and 3
 // (k = 64: 326 against 386).

@@ -6,7 +6,7 @@
 // recorded graph (a graph is recorded for every solve, a reducing launch ends
 // with 4.5 us of fp64 trees and a last CTA's pass over the partial sums): 300
 // steps on the 27-point stencil, 6 refinements, 1,000 rows fp64 5.6 -> 2.3 ms,
-// 4,096 rows fp32 5.2 -> 2.4, 19,683 rows fp32 6.2 -> 2.7 and fp64 5.6 -> 3.2,
+// 4,096 rows fp32 5.2 -> 2.5, 19,683 rows fp32 6.2 -> 2.8 and fp64 5.6 -> 3.2,
 // 125,000 rows fp32 7.8 -> 4.6 ms.
 #include <math.h>
 #include <string.h>

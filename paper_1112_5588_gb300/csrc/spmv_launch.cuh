@@ -202,7 +202,8 @@ int launch_pjds(const pjds_dev *A, const void *x, void *y, const LaunchCfg &c, c
 // stencil 405k rows fp64 28.9 / 33.0, 1M rows fp64 61.0 / 68.9, fp32 38.1 / 36.4,
 // bf16 37.1 / 43.1, 250k rows bf16 11.0 / 13.1; rows of 144 in dense blocks, 100k
 // fp32 36.0 / 24.6, bf16 41.4 / 33.4, 248k fp64 109 / 93, bf16 50 / 66, 600k fp64
-// 179 / 187. (256-thread CTAs with 8 were 11-24% slower in fp64 on millions of
+// 179 / 187. (Between the sizes of the lines the matrices differ: at 300k rows in
+// fp64 8 is still better on one, at 405k 4 on another. 256-thread CTAs with 8 were 11-24% slower in fp64 on millions of
 // rows.)
 template <typename TV, typename TX>
 int launch_ellr(const ellr_dev *A, const void *x, void *y, int nt, cudaStream_t s) {

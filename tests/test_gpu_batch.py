@@ -336,7 +336,7 @@ def test_spmm_rows_sharing_their_columns_in_fours(mods, dtype, n, k, bs, nb, mix
 
 
 def test_spmm_in_fours_in_a_captured_graph(mods):
-    # two overlapping launches and what follows them on the stream
+    # two launches and what follows them on the stream
     torch, pjds, batch = mods
     for bs, nb in ((4, 5), (2, 10)):
         A = _block_rows(33_000, 8_000, bs, nb, 0.0, seed=bs)
