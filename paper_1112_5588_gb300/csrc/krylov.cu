@@ -790,9 +790,10 @@ template <typename TX, int MODE>
 static void launch_dot(const DotKernel<TX, MODE> &d, const pjds_dev *A, const typename Same<TX>::type *x,
                        typename Same<TX>::type *y, const typename Same<TX>::type *bv, const Reduce &red, cudaStream_t s,
                        int32_t op, int32_t j = 0, double *out = nullptr) {
-  // no more CTAs than fit at once, but no more rows of a thread than KEEP (from 7.5M rows on in fp32)
+  // no more CTAs than fit at once, but with floats no more rows of a thread than KEEP (from 7.5M rows on)
   const int64_t all = ((int64_t)A->n_rows + d.rows - 1) / d.rows;
-  const int64_t grid = std::min<int64_t>(all, std::max<int64_t>(d.resident, (all * (d.rows / KT) + KEEP - 1) / KEEP));
+  const int64_t least = sizeof(TX) == 4 ? (all * (d.rows / KT) + KEEP - 1) / KEEP : 1;
+  const int64_t grid = std::min<int64_t>(all, std::max<int64_t>(d.resident, least));
   d.fn<<<(unsigned)grid, KT, 0, s>>>(A->val, A->col, A->col_start, A->block_len, x, y, bv, red.partial, A->n_rows, A->b);
   red.sum(grid, s, op, j, out);
 }
